@@ -923,7 +923,6 @@ VP_API int sim_create(const sim_system *systems, int32_t n_systems, const int32_
   r |= upload(h, &d.sys_nbg, sys_nbg);
   d.max_nbg = sys_nbg.empty() ? 0 : *std::max_element(sys_nbg.begin(), sys_nbg.end());
   r |= upload(h, &d.tiles, tiles);
-  r |= upload(h, &d.work, work);
   {
     // tiles close to the diagonal hold the pairs close in sequence, which are
     // mostly near pairs: they run first so that the long ones do not trail
@@ -933,7 +932,13 @@ VP_API int sim_create(const sim_system *systems, int32_t n_systems, const int32_
       const int2 ta = tiles[work[a].y], tb = tiles[work[b].y];
       return ta.y - ta.x < tb.y - tb.x;
     });
-    r |= upload(h, &d.work_order, order);
+    std::vector<CvItem> items(work.size());
+    for (size_t k = 0; k < work.size(); ++k) {
+      const int2 wk = work[order[k]], bij = tiles[wk.y];
+      const TrialInfo &T = h->tinfo[wk.x];
+      items[k] = CvItem{order[k], wk.y, T.atom0, T.cv0, T.n_cv, bij.x, bij.y, 0, T.box, T.inv_box};
+    }
+    r |= upload(h, &d.cv_item, items);
   }
   r |= dalloc(h, &d.cnat, tiles.size() * CV_T * CV_T);
   r |= dalloc(h, &d.cnat_ff, tiles.size() * CV_T * CV_T);

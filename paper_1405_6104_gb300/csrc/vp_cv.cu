@@ -10,10 +10,9 @@
 // the functional needs it to ~1e-6 relative.  Gradients are accumulated in
 // 64-bit fixed point, z partial sums in FP64.
 //
-// Work item = (trial, 32 x 32 tile of the pair triangle); one warp per item.
-// Lane l owns i = bi*32 + l; at step k it takes column (l + k) mod 32, and the
-// column accumulators travel one lane per step around the warp so that every
-// column sum is built in a fixed order without atomics inside the tile.
+// Work item = (trial, 32 x 32 tile of the pair triangle); one warp per item,
+// or one block per item when there are few.  Lane l owns i = bi*32 + l; at
+// step k it takes column (l + k) mod 32.
 #include "vp_cvpair.cuh"
 #include "vp_dev.cuh"
 #include "vp_cv_dev.cuh"
@@ -92,6 +91,14 @@ __global__ void __launch_bounds__(CV_WARPS * 32) k_cv(Dev d, SimConst c) {
   cv_tile(d, c, sh[wib], wq);
 }
 
+constexpr int CV_BLOCK_WARPS = 4;
+template <int NW>
+__global__ void __launch_bounds__(NW * 32) k_cv_block(Dev d, SimConst c) {
+  __shared__ CvBlockShared<NW> sh;
+  PDL_WAIT();
+  cv_tile_block<NW>(d, c, sh, blockIdx.x);
+}
+
 // per trial: z, the ratchet amplitude a, z_m and Phi (Eqs. VR, VMDcondition).
 // One block per trial; the reduction order (over CVFIN_THREADS virtual
 // threads) is fixed, so every trial's z does not depend on the batch or on
@@ -138,9 +145,23 @@ void launch_cnat(const Dev &d, const SimConst &c, const double *native, const in
 void launch_zconst(const Dev &d, const int32_t *sys_tile0, const int32_t *sys_ntiles, cudaStream_t s) {
   k_zconst<<<d.n_trials, 256, 0, s>>>(d, sys_tile0, sys_ntiles);
 }
-// variants: 0: 4 warps per block, 1: 2 warps, 2: 8 warps
+// variants (one warp per tile): 0: 4 warps per block, 1: 2 warps, 2: 8 warps
 void launch_cv(const Dev &d, const SimConst &c, cudaStream_t s, int variant, bool after_kernel) {
   if (d.total_work <= 0) return;
+  // Few tiles leave one or two warps per SM, each in a chain of some 1500
+  // cycles per 32 near pairs: then a block of four warps works on one tile.
+  // One trial of 540 / 1800 reaction-coordinate atoms (136 / 1653 tiles): k_cv
+  // 24.2 -> 6.4 / 31 -> 16 us, the MD step 54.6 -> 50.2 / 78 -> 68 us; 2176
+  // tiles: 28.8 -> 20.5 us, the step unchanged (the kernel hides behind the
+  // list and pair kernels).  From about 16 tiles per SM on the GPU is full and
+  // the block form's barriers and scan only cost issue slots (8704 tiles: the
+  // step 956 -> 964 us, 16 530: 451 -> 457).  Eight warps per tile: no faster.
+  if (d.total_work <= 16 * d.n_sm) {
+    const dim3 g((unsigned)d.total_work), b(32 * CV_BLOCK_WARPS);
+    if (after_kernel) launch_pdl(k_cv_block<CV_BLOCK_WARPS>, g, b, s, d, c);
+    else k_cv_block<CV_BLOCK_WARPS><<<g, b, 0, s>>>(d, c);
+    return;
+  }
   const int w = variant == 1 ? 2 : variant == 2 ? 8 : 4;
   const dim3 g((unsigned)((d.total_work + w - 1) / w)), b((unsigned)(32 * w));
   if (!after_kernel) {  // first on its stream: an ordinary launch

@@ -9,106 +9,186 @@ namespace vp {
 
 __device__ __forceinline__ long long gsum(int hi, unsigned lo) { return (long long)hi * 16777216ll + (long long)lo; }
 
+// The near pair (il, jc) of a tile: its z term, and its gradient contribution
+// into the tile's shared accumulators.  One definition for the warp and the
+// block form of a tile, so both give the same bits.
+template <class SH>
+__device__ __forceinline__ ff cv_near_pair(SH &sh, const CvConst &k, const float2 *cn, float L, float iL, unsigned e) {
+  const int il = e & 31, jc = e >> 5;
+  const float3 pi = make_float3(sh.s_x[il][0], sh.s_x[il][1], sh.s_x[il][2]);
+  ff dx, dy, dz;
+  cv_delta(pi, sh.s_x[CV_T + jc][0], sh.s_x[CV_T + jc][1], sh.s_x[CV_T + jc][2], L, iL, dx, dy, dz);
+  const float2 cv2 = cn[((jc - il) & (CV_T - 1)) * CV_T + il];
+  const ff cnat = {cv2.x, cv2.y};
+  const ff r2 = ff_add(ff_add(ff_sqr(dx), ff_sqr(dy)), ff_sqr(dz));
+  const CvPair cp = cv_contact<false>(r2, k);
+  const ff h = ff_add(cp.Ct, ff_neg(cnat));
+  // dz/dx_i = -w d, dz/dx_j = +w d with d = x_j - x_i, w = 2 h C~'(r)/r
+  const float wgt = 2.0f * h.hi * cp.dCt / cp.r;
+  if (wgt != 0.0f) {
+    const long long gx = fx_from(wgt * dx.hi), gy = fx_from(wgt * dy.hi), gz = fx_from(wgt * dz.hi);
+    const long long gv[3] = {gx, gy, gz};
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      atomicAdd(&sh.s_ghi[il][q], (int)((-gv[q]) >> 24));
+      atomicAdd(&sh.s_glo[il][q], (unsigned)((-gv[q]) & 0xffffff));
+      atomicAdd(&sh.s_ghi[CV_T + jc][q], (int)(gv[q] >> 24));
+      atomicAdd(&sh.s_glo[CV_T + jc][q], (unsigned)(gv[q] & 0xffffff));
+    }
+  }
+  // z term: C~ (C~ - 2 C~_nat) = (C~ - C~_nat)^2 - C~_nat^2
+  return ff_mul(cp.Ct, ff_add(cp.Ct, ff{-2.0f * cnat.hi, -2.0f * cnat.lo}));  // doubling is exact
+}
+
+// whether a pair at the (unimaged) FP32 difference (dx, dy, dz) is closer than the contact cut-off
+__device__ __forceinline__ bool cv_is_near(float dx, float dy, float dz, float L, float iL, float rc2_far) {
+  dx -= L * rintf(dx * iL);
+  dy -= L * rintf(dy * iL);
+  dz -= L * rintf(dz * iL);
+  return dx * dx + dy * dy + dz * dz < rc2_far;
+}
+
+// the accumulated gradient of atom a (0..63) of the tile, into the trial's sums
+template <class SH>
+__device__ __forceinline__ void cv_flush_atom(const Dev &d, SH &sh, int a, int g) {
+  const long long a0 = gsum(sh.s_ghi[a][0], sh.s_glo[a][0]), a1 = gsum(sh.s_ghi[a][1], sh.s_glo[a][1]),
+                  a2 = gsum(sh.s_ghi[a][2], sh.s_glo[a][2]);
+  if (a0 | a1 | a2) { red_add(d.gx + g, a0); red_add(d.gy + g, a1); red_add(d.gz + g, a2); }
+}
+
 // One warp's tile of the contact-pair triangle: the work item wq of the flat
-// (trial, tile) list, in the work order.
+// (trial, tile) list, in the work order (costliest tiles first; the partial
+// sums of z keep their slots).
 __device__ __forceinline__ void cv_tile(const Dev &d, const SimConst &c, CvWarpShared &sh, int wq) {
-  auto &s_near = sh.s_near;
   auto &s_x = sh.s_x;
-  auto &s_ghi = sh.s_ghi;
-  auto &s_glo = sh.s_glo;
   const int lane = threadIdx.x & 31;
-  const int w = d.work_order[wq];  // costliest tiles first (the partial sums keep their slots)
-  const int2 wk = d.work[w];
-  const TrialInfo T = d.tinfo[wk.x];
-  const int2 bij = d.tiles[wk.y];
-  const int ncv = T.n_cv, msep = c.cv_min_sep;
-  const float L = T.box, iL = T.inv_box;
-  const int i = bij.x * CV_T + lane;
-  const int jl = bij.y * CV_T + lane;
+  const CvItem W = d.cv_item[wq];
+  const int ncv = W.n_cv, msep = c.cv_min_sep;
+  const float L = W.box, iL = W.inv_box;
+  const int i = W.bi * CV_T + lane;
+  const int jl = W.bj * CV_T + lane;
   float3 xi = make_float3(0.f, 0.f, 0.f), xj = make_float3(0.f, 0.f, 0.f);
-  if (i < ncv) { float4 q = d.pos[d.slot_of[T.atom0 + i]]; xi = make_float3(q.x, q.y, q.z); }
-  if (jl < ncv) { float4 q = d.pos[d.slot_of[T.atom0 + jl]]; xj = make_float3(q.x, q.y, q.z); }
+  if (i < ncv) { float4 q = d.pos[d.slot_of[W.atom0 + i]]; xi = make_float3(q.x, q.y, q.z); }
+  if (jl < ncv) { float4 q = d.pos[d.slot_of[W.atom0 + jl]]; xj = make_float3(q.x, q.y, q.z); }
   s_x[lane][0] = xi.x; s_x[lane][1] = xi.y; s_x[lane][2] = xi.z;
   s_x[CV_T + lane][0] = xj.x; s_x[CV_T + lane][1] = xj.y; s_x[CV_T + lane][2] = xj.z;
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
-    s_ghi[lane][q] = 0; s_ghi[CV_T + lane][q] = 0;
-    s_glo[lane][q] = 0u; s_glo[CV_T + lane][q] = 0u;
+    sh.s_ghi[lane][q] = 0; sh.s_ghi[CV_T + lane][q] = 0;
+    sh.s_glo[lane][q] = 0u; sh.s_glo[CV_T + lane][q] = 0u;
   }
   // ---- phase 1: near pairs of the tile ----
   int n_near = 0;
   for (int k = 0; k < CV_T; ++k) {
     const int jc = (lane + k) & (CV_T - 1);
-    const int j = bij.y * CV_T + jc;
+    const int j = W.bj * CV_T + jc;
     const float xjx = __shfl_sync(0xffffffffu, xj.x, jc);
     const float xjy = __shfl_sync(0xffffffffu, xj.y, jc);
     const float xjz = __shfl_sync(0xffffffffu, xj.z, jc);
-    bool near = false;
-    if (i < ncv && j < ncv && j - i > msep) {
-      float dx = xjx - xi.x, dy = xjy - xi.y, dz = xjz - xi.z;
-      dx -= L * rintf(dx * iL);
-      dy -= L * rintf(dy * iL);
-      dz -= L * rintf(dz * iL);
-      near = dx * dx + dy * dy + dz * dz < c.cv_rc2_far;
-    }
+    const bool near = i < ncv && j < ncv && j - i > msep &&
+                      cv_is_near(xjx - xi.x, xjy - xi.y, xjz - xi.z, L, iL, c.cv_rc2_far);
     const unsigned bal = __ballot_sync(0xffffffffu, near);
-    if (near) s_near[n_near + __popc(bal & ((1u << lane) - 1u))] = (unsigned short)(lane | (jc << 5));
+    if (near) sh.s_near[n_near + __popc(bal & ((1u << lane) - 1u))] = (unsigned short)(lane | (jc << 5));
     n_near += __popc(bal);
   }
   __syncwarp();
   // ---- phase 2: the near pairs, densely ----
   const CvConst k = cv_const(c);
-  const float2 *cn = d.cnat_ff + (size_t)wk.y * CV_T * CV_T;
+  const float2 *cn = d.cnat_ff + (size_t)W.tile * CV_T * CV_T;
   ff zacc = {0.f, 0.f};
-  for (int base = 0; base < n_near; base += 32) {
-    const int idx = base + lane;
-    if (idx < n_near) {
-      const unsigned e = s_near[idx];
-      const int il = e & 31, jc = e >> 5;
-      const float3 pi = make_float3(s_x[il][0], s_x[il][1], s_x[il][2]);
-      ff dx, dy, dz;
-      cv_delta(pi, s_x[CV_T + jc][0], s_x[CV_T + jc][1], s_x[CV_T + jc][2], L, iL, dx, dy, dz);
-      const float2 cv2 = cn[((jc - il) & (CV_T - 1)) * CV_T + il];
-      const ff cnat = {cv2.x, cv2.y};
-      const ff r2 = ff_add(ff_add(ff_sqr(dx), ff_sqr(dy)), ff_sqr(dz));
-      const CvPair cp = cv_contact<false>(r2, k);
-      const ff h = ff_add(cp.Ct, ff_neg(cnat));
-      // z term: C~ (C~ - 2 C~_nat) = (C~ - C~_nat)^2 - C~_nat^2
-      zacc = ff_add(zacc, ff_mul(cp.Ct, ff_add(cp.Ct, ff{-2.0f * cnat.hi, -2.0f * cnat.lo})));  // doubling is exact
-      // dz/dx_i = -w d, dz/dx_j = +w d with d = x_j - x_i, w = 2 h C~'(r)/r
-      const float wgt = 2.0f * h.hi * cp.dCt / cp.r;
-      if (wgt != 0.0f) {
-        const long long gx = fx_from(wgt * dx.hi), gy = fx_from(wgt * dy.hi), gz = fx_from(wgt * dz.hi);
-        const long long gv[3] = {gx, gy, gz};
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-          atomicAdd(&s_ghi[il][q], (int)((-gv[q]) >> 24));
-          atomicAdd(&s_glo[il][q], (unsigned)((-gv[q]) & 0xffffff));
-          atomicAdd(&s_ghi[CV_T + jc][q], (int)(gv[q] >> 24));
-          atomicAdd(&s_glo[CV_T + jc][q], (unsigned)(gv[q] & 0xffffff));
-        }
-      }
-    }
-  }
+  for (int base = 0; base < n_near; base += 32)
+    if (base + lane < n_near) zacc = ff_add(zacc, cv_near_pair(sh, k, cn, L, iL, sh.s_near[base + lane]));
   __syncwarp();
   if (n_near > 0) {
-    if (i < ncv) {
-      const long long a0 = gsum(s_ghi[lane][0], s_glo[lane][0]),
-                      a1 = gsum(s_ghi[lane][1], s_glo[lane][1]),
-                      a2 = gsum(s_ghi[lane][2], s_glo[lane][2]);
-      if (a0 | a1 | a2) { red_add(d.gx + T.cv0 + i, a0); red_add(d.gy + T.cv0 + i, a1); red_add(d.gz + T.cv0 + i, a2); }
-    }
-    if (jl < ncv) {
-      const long long a0 = gsum(s_ghi[CV_T + lane][0], s_glo[CV_T + lane][0]),
-                      a1 = gsum(s_ghi[CV_T + lane][1], s_glo[CV_T + lane][1]),
-                      a2 = gsum(s_ghi[CV_T + lane][2], s_glo[CV_T + lane][2]);
-      if (a0 | a1 | a2) { red_add(d.gx + T.cv0 + jl, a0); red_add(d.gy + T.cv0 + jl, a1); red_add(d.gz + T.cv0 + jl, a2); }
-    }
+    if (i < ncv) cv_flush_atom(d, sh, lane, W.cv0 + i);
+    if (jl < ncv) cv_flush_atom(d, sh, CV_T + lane, W.cv0 + jl);
   }
   double zl = ff_to_d(zacc);
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) zl += __shfl_xor_sync(0xffffffffu, zl, off);
-  if (lane == 0) d.z_part[w] = zl;
+  if (lane == 0) d.z_part[W.w] = zl;
+}
+
+// The same tile by a block of NW warps: the 32 rotations of phase 1 and the
+// chunks of 32 near pairs of phase 2 are dealt out over the warps.  The near
+// pairs keep the order the one-warp form lists them in, and the z terms go
+// through shared memory so that each lane of the first warp adds them in that
+// order too: z and the gradient are the same bit for bit.
+template <int NW>
+struct CvBlockShared {
+  unsigned short s_near[CV_T * CV_T];
+  float s_x[2 * CV_T][3];
+  int s_ghi[2 * CV_T][3];
+  unsigned s_glo[2 * CV_T][3];
+  unsigned s_bal[CV_T];
+  float2 s_term[CV_T * CV_T];
+};
+
+template <int NW>
+__device__ __forceinline__ void cv_tile_block(const Dev &d, const SimConst &c, CvBlockShared<NW> &sh, int wq) {
+  constexpr int KW = CV_T / NW;  // rotations per warp
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const CvItem W = d.cv_item[wq];
+  const int ncv = W.n_cv, msep = c.cv_min_sep;
+  const float L = W.box, iL = W.inv_box;
+  if (threadIdx.x < 2 * CV_T) {
+    const int a = (warp == 0 ? W.bi : W.bj) * CV_T + lane;
+    float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (a < ncv) q = d.pos[d.slot_of[W.atom0 + a]];
+    sh.s_x[threadIdx.x][0] = q.x; sh.s_x[threadIdx.x][1] = q.y; sh.s_x[threadIdx.x][2] = q.z;
+  }
+  for (int q = threadIdx.x; q < 2 * CV_T * 3; q += NW * 32) {
+    (&sh.s_ghi[0][0])[q] = 0;
+    (&sh.s_glo[0][0])[q] = 0u;
+  }
+  __syncthreads();
+  const int i = W.bi * CV_T + lane;
+  const float3 xi = make_float3(sh.s_x[lane][0], sh.s_x[lane][1], sh.s_x[lane][2]);
+  unsigned bal[KW];
+#pragma unroll
+  for (int q = 0; q < KW; ++q) {
+    const int jc = (lane + warp * KW + q) & (CV_T - 1);
+    const int j = W.bj * CV_T + jc;
+    const float *x = sh.s_x[CV_T + jc];
+    const bool near = i < ncv && j < ncv && j - i > msep &&
+                      cv_is_near(x[0] - xi.x, x[1] - xi.y, x[2] - xi.z, L, iL, c.cv_rc2_far);
+    bal[q] = __ballot_sync(0xffffffffu, near);
+    if (lane == 0) sh.s_bal[warp * KW + q] = bal[q];
+  }
+  __syncthreads();
+  int incl = __popc(sh.s_bal[lane]);
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, incl, off);
+    if (lane >= off) incl += v;
+  }
+  const int n_near = __shfl_sync(0xffffffffu, incl, 31);
+#pragma unroll
+  for (int q = 0; q < KW; ++q) {
+    const int end = __shfl_sync(0xffffffffu, incl, warp * KW + q);
+    if ((bal[q] >> lane) & 1u)
+      sh.s_near[end - __popc(bal[q]) + __popc(bal[q] & ((1u << lane) - 1u))] =
+          (unsigned short)(lane | (((lane + warp * KW + q) & (CV_T - 1)) << 5));
+  }
+  __syncthreads();
+  const CvConst k = cv_const(c);
+  const float2 *cn = d.cnat_ff + (size_t)W.tile * CV_T * CV_T;
+  for (int p = threadIdx.x; p < n_near; p += NW * 32) {
+    const ff t = cv_near_pair(sh, k, cn, L, iL, sh.s_near[p]);
+    sh.s_term[p] = make_float2(t.hi, t.lo);
+  }
+  __syncthreads();
+  if (warp == 0) {
+    ff zacc = {0.f, 0.f};
+    for (int p = lane; p < n_near; p += 32) zacc = ff_add(zacc, ff{sh.s_term[p].x, sh.s_term[p].y});
+    double zl = ff_to_d(zacc);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) zl += __shfl_xor_sync(0xffffffffu, zl, off);
+    if (lane == 0) d.z_part[W.w] = zl;
+  } else if (warp <= 2 && n_near > 0) {
+    const int a = (warp == 1 ? W.bi : W.bj) * CV_T + lane;
+    if (a < ncv) cv_flush_atom(d, sh, (warp - 1) * CV_T + lane, W.cv0 + a);
+  }
 }
 
 

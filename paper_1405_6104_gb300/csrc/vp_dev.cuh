@@ -52,8 +52,8 @@ struct Dev {
   int32_t max_nbg;                     // largest group count of a system
   // reaction coordinate
   int2 *tiles;                         // per system tile (bi, bj), concatenated
-  int2 *work;                          // flat (trial, global tile) work items
-  int32_t *work_order;                 // the order warps take them: tiles near the diagonal (most near pairs) first
+  CvItem *cv_item;                     // the (trial, tile) work items in the order they are taken: tiles near
+                                       // the diagonal (most near pairs) first
   double *cnat;                        // [tiles * 1024] C~ of the native structure in tile-skew order
   float2 *cnat_ff;                     // the same as float-float (hi, lo), read by the per-step kernel
   int32_t *sys_ncv, *sys_minsep;

@@ -92,6 +92,15 @@ struct TrialState {
   double zconst;       // sum of C~_nat^2 over the trial's contact pairs
 };
 
+// one (trial, 32 x 32 tile) work item of the reaction coordinate with what the
+// kernel needs of its trial and tile: one load instead of a chain of three
+struct __align__(16) CvItem {
+  int32_t w, tile;     // slot of the partial sum of z; the tile among all systems' tiles
+  int32_t atom0, cv0;  // as in TrialInfo
+  int32_t n_cv, bi, bj, pad_;
+  float box, inv_box;
+};
+
 // per-system, caller-ordered atom data
 struct AtomSys {
   float invm, c1, c2sd, qs;   // 1/m, exp(-gamma dt), sqrt((1-c1^2) kT/m), q*sqrt(f)
