@@ -283,12 +283,14 @@ int sim_pairlist(sim_handle *h, int32_t trial, int32_t *pairs, int64_t cap, int6
 int sim_list_positions(sim_handle *h, int32_t trial, double *pos);
 int sim_diagnostics(sim_handle *h, int64_t *out);
 
-/* Autotuner: times the launch-shape variants of the pair kernel (0-2: the
- * i-atoms in registers with register caps of 4, 5 or 6 blocks per SM; 3-5:
- * the i-atoms in shared memory with caps of 6, 7 or 8 blocks per SM; 6-8:
- * packed FP32x2 arithmetic, i-atoms in shared memory, caps of 5, 6 or 7;
- * 3-8 need at most 16 LJ types, else run as variant 0; all give bit-identical
- * forces) and of the reaction-coordinate kernel
+/* Autotuner: times the launch-shape variants of the pair kernel (0-2: any
+ * number of LJ types, register caps of 4, 5 or 6 blocks per SM; 3-8: packed
+ * FP32x2 arithmetic, for at most 16 LJ types, else run as variant 0 -- 3, 4:
+ * one warp per block, two groups of list entries at a time, 20 or 16 warps
+ * per SM; 5, 6: persistent blocks, two groups at a time, 4 or 5 blocks per
+ * SM; 7, 8: one group at a time, 6 or 7 blocks; all give bit-identical
+ * forces; an untuned batch takes 0, 3 or 6 by its types and size) and of the
+ * reaction-coordinate kernel
  * (2, 4 or 8 warps per block) on this batch, reps launches each, into scratch
  * accumulators (the state is untouched), and uses the fastest from then on.
  * Size classes: the trials are grouped by round(log2 atoms) and density; when

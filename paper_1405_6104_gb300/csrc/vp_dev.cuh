@@ -171,6 +171,7 @@ void launch_list_positions(const Dev &d, int32_t trial, double *out, int32_t n, 
 // clist (optional): the i-clusters to work on (n_items of them), else all
 void launch_pair(const Dev &d, const SimConst &c, bool energy, int32_t only_trial, cudaStream_t s, int variant = 0,
                  const int *clist = nullptr, int n_items = 0);
+int default_pair_variant(const Dev &d, const SimConst &c);
 void launch_bonded(const Dev &d, cudaStream_t s);
 constexpr int PAIR_VARIANTS = 9;
 // reaction coordinate and functional (vp_cv.cu)

@@ -239,21 +239,19 @@ __global__ void __launch_bounds__(128, MINB) k_pair(Dev d, SimConst c, int only_
 }
 
 
-// Force-only kernel (the hot path).  Per warp, shared memory holds the LJ
+// Force-only kernel for any number of LJ types (up to MAX_TYPES; the packed
+// kernels' tables hold SMALL_TYPES).  Per warp, shared memory holds the LJ
 // coefficients of its 8 i-atoms against every type (row a at a fixed stride,
 // so the pair loop addresses them with immediate offsets) and the 27 image
-// shifts of its box; the list mask enters the squared distance as a penalty
-// (0 or 1e30), so a masked pair falls outside the cut-off without any
-// per-pair bit test.  Arithmetic per pair: 3 FADD, 6 FMUL, 12 FFMA, 1 RSQ,
-// 1 LDS, 1 FSETP + FSEL.
-// SHI: the i-atoms are read from shared memory (one broadcast LDS.128 per
-// pair) instead of being held in 32 registers, which lets more warps reside.
-// TS is the row stride of the per-warp LJ table (at least the number of types).
-template <int MINB, bool SHI, int TS>
+// shifts of its box, registers the i-atoms; the list mask enters the squared
+// distance as a penalty (0 or 1e30), so a masked pair falls outside the
+// cut-off without any per-pair bit test.  Arithmetic per pair: 3 FADD, 6 FMUL,
+// 12 FFMA, 1 RSQ, 1 LDS, 1 FSETP + FSEL.
+template <int MINB>
 __global__ void __launch_bounds__(PF_WARPS * 32, MINB) k_pair_f(Dev d, SimConst c, const int *clist, int n_items) {
+  constexpr int TS = MAX_TYPES;
   __shared__ float2 s_cij[PF_WARPS][CL][TS];
   __shared__ float4 s_sh[PF_WARPS][64];
-  __shared__ float4 s_i[PF_WARPS][CL];
   __shared__ float s_red[PF_WARPS][3 * CL * 33];
   const int wib = threadIdx.x >> 5;
   const int item = blockIdx.x * PF_WARPS + wib;
@@ -274,7 +272,6 @@ __global__ void __launch_bounds__(PF_WARPS * 32, MINB) k_pair_f(Dev d, SimConst 
     xi[a] = p.x; yi[a] = p.y; zi[a] = p.z; qi[a] = p.w;
     ti[a] = d.type[I * CL + a];
   }
-  if (SHI && lane < CL) s_i[wib][lane] = d.pos[I * CL + lane];
   // per-warp tables: LJ rows of the i-atoms, image shifts (code = (nx+1) | (ny+1)<<2 | (nz+1)<<4)
   for (int k = lane; k < CL * NT; k += 32) {
     const int a = k / NT, tj = k - a * NT;
@@ -322,7 +319,7 @@ __global__ void __launch_bounds__(PF_WARPS * 32, MINB) k_pair_f(Dev d, SimConst 
       constexpr bool MASKED = decltype(mtag)::value;
 #pragma unroll
       for (int a = 0; a < CL; ++a) {
-        const float4 ia = SHI ? s_i[wib][a] : make_float4(xi[a], yi[a], zi[a], qi[a]);
+        const float4 ia = make_float4(xi[a], yi[a], zi[a], qi[a]);
         const float pen = MASKED ? ((mb & (1u << a)) ? 0.0f : MASK_PEN) : 0.0f;
         const float dx = __fsub_rn(xj, ia.x), dy = __fsub_rn(yj, ia.y), dz = __fsub_rn(zj, ia.z);
         const float r2 = __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmaf_rn(dx, dx, pen)));
@@ -353,7 +350,7 @@ __global__ void __launch_bounds__(PF_WARPS * 32, MINB) k_pair_f(Dev d, SimConst 
       // some entry of this group needs pair-by-pair minimum images
 #pragma unroll
       for (int a = 0; a < CL; ++a) {
-        const float4 ia = SHI ? s_i[wib][a] : make_float4(xi[a], yi[a], zi[a], qi[a]);
+        const float4 ia = make_float4(xi[a], yi[a], zi[a], qi[a]);
         const float pen = (mb & (1u << a)) ? 0.0f : MASK_PEN;
         float dx = __fsub_rn(xj, ia.x), dy = __fsub_rn(yj, ia.y), dz = __fsub_rn(zj, ia.z);
         if (exact) {
@@ -421,10 +418,10 @@ __global__ void __launch_bounds__(PF_WARPS * 32, MINB) k_pair_f(Dev d, SimConst 
 // all variants give bit-identical forces.
 
 
-template <int MINB>
+template <int MINB, int U>
 __global__ void __launch_bounds__(PF_WARPS * 32, MINB) k_pair_f2(Dev d, SimConst c, unsigned *next, const int *clist,
                                                                    int n_items) {
-  __shared__ PairF2Shared sh;
+  __shared__ PairF2Shared<PF_WARPS> sh;
   const int lane = threadIdx.x & 31;
   // persistent warps: each takes the next i-cluster from a counter until none
   // is left, so that short and long lists even out across the SMs
@@ -434,8 +431,19 @@ __global__ void __launch_bounds__(PF_WARPS * 32, MINB) k_pair_f2(Dev d, SimConst
     if (lane == 0) got = atomicAdd(next, 1u);
     const int item = (int)__shfl_sync(0xffffffffu, got, 0);
     if (item >= n_items) return;
-    pair_cluster_f2(d, c, sh, clist ? clist[item] : item);
+    pair_cluster_f2<U>(d, c, sh, clist ? clist[item] : item);
   }
+}
+
+// The same with one warp per block and i-cluster, the blocks dealt out by the
+// hardware: without the counter's fetch before every cluster, and with lists
+// of every length on every SM (they get shorter along the clusters), a batch
+// whose clusters are few per SM is done sooner.
+template <int U, int MINB>
+__global__ void __launch_bounds__(32, MINB) k_pair_w(Dev d, SimConst c, const int *clist, int n_items) {
+  __shared__ PairF2Shared<1> sh;
+  const int item = blockIdx.x;
+  pair_cluster_f2<U>(d, c, sh, clist ? clist[item] : item);
 }
 
 __global__ void __launch_bounds__(256) k_bonded(Dev d) {
@@ -447,11 +455,22 @@ void launch_bonded(const Dev &d, cudaStream_t s) {
   k_bonded<<<dim3((unsigned)((d.max_nbg + 255) / 256), (unsigned)d.n_trials), 256, 0, s>>>(d);
 }
 
-// variants differ in the register cap (blocks per SM the compiler must fit)
-// and in where the i-atoms live: 0/1/2: registers, 4/5/6 blocks; 3/4/5:
-// shared memory and an LJ table for at most SMALL_TYPES types (less shared
-// memory per block), 6/7/8 blocks (larger type sets fall back to variant 0).
-// All variants do the same arithmetic in the same order (bit-identical forces).
+// Variants (all do the same arithmetic in the same order: bit-identical
+// forces).  0, 1, 2: any number of types, registers capped for 4, 5 or 6
+// blocks per SM.  The others need at most SMALL_TYPES types (else variant 0
+// runs): 3, 4: one warp per block, two groups of entries at a time, 20 or 16
+// warps per SM; 5, 6: persistent blocks, two groups at a time, 4 or 5 blocks;
+// 7, 8: persistent blocks, one group at a time, 6 or 7 blocks.
+// The variant of a batch that has not been tuned: the packed kernels whenever
+// the types fit.  Up to 300 clusters per SM one warp per block is the faster
+// form (the MD step of one 11 040-atom trial 43.1 us against 51.2, of 16
+// trials 213 against 219, of ten 30 000-atom trials 352.2 against 352.9), in
+// larger batches the persistent one (64 trials 695 against 706 us).
+int default_pair_variant(const Dev &d, const SimConst &c) {
+  if (c.n_types > SMALL_TYPES) return 0;
+  return d.total_clus <= 300 * d.n_sm ? 3 : 6;
+}
+
 void launch_pair(const Dev &d, const SimConst &c, bool energy, int32_t only_trial, cudaStream_t s, int variant,
                  const int *clist, int n_items) {
   long long threads = (long long)d.total_clus * 32;
@@ -466,23 +485,23 @@ void launch_pair(const Dev &d, const SimConst &c, bool energy, int32_t only_tria
   const unsigned fb = (unsigned)((n_items + PF_WARPS - 1) / PF_WARPS);
   if (variant >= 3 && c.n_types > SMALL_TYPES) variant = 0;
   switch (variant) {
-    case 1: k_pair_f<5, false, MAX_TYPES><<<fb, PF_WARPS * 32, 0, s>>>(d, c, clist, n_items); break;
-    case 2: k_pair_f<6, false, MAX_TYPES><<<fb, PF_WARPS * 32, 0, s>>>(d, c, clist, n_items); break;
-    case 3: k_pair_f<6, true, SMALL_TYPES><<<fb, PF_WARPS * 32, 0, s>>>(d, c, clist, n_items); break;
-    case 4: k_pair_f<7, true, SMALL_TYPES><<<fb, PF_WARPS * 32, 0, s>>>(d, c, clist, n_items); break;
-    case 5: k_pair_f<8, true, SMALL_TYPES><<<fb, PF_WARPS * 32, 0, s>>>(d, c, clist, n_items); break;
-    case 6: case 7: case 8: {
+    case 1: k_pair_f<5><<<fb, PF_WARPS * 32, 0, s>>>(d, c, clist, n_items); break;
+    case 2: k_pair_f<6><<<fb, PF_WARPS * 32, 0, s>>>(d, c, clist, n_items); break;
+    case 3: k_pair_w<2, 20><<<n_items, 32, 0, s>>>(d, c, clist, n_items); break;
+    case 4: k_pair_w<2, 16><<<n_items, 32, 0, s>>>(d, c, clist, n_items); break;
+    case 5: case 6: case 7: case 8: {
       // persistent grid: as many blocks as can be resident, sized from the SM
       // count; the counter hands out the i-clusters
       const int minb = variant - 1;
       const unsigned pb = std::min(fb, (unsigned)(d.n_sm * minb));
       cudaMemsetAsync(d.pair_next, 0, sizeof(unsigned), s);
-      if (variant == 6) k_pair_f2<5><<<pb, PF_WARPS * 32, 0, s>>>(d, c, d.pair_next, clist, n_items);
-      else if (variant == 7) k_pair_f2<6><<<pb, PF_WARPS * 32, 0, s>>>(d, c, d.pair_next, clist, n_items);
-      else k_pair_f2<7><<<pb, PF_WARPS * 32, 0, s>>>(d, c, d.pair_next, clist, n_items);
+      if (variant == 5) k_pair_f2<4, 2><<<pb, PF_WARPS * 32, 0, s>>>(d, c, d.pair_next, clist, n_items);
+      else if (variant == 6) k_pair_f2<5, 2><<<pb, PF_WARPS * 32, 0, s>>>(d, c, d.pair_next, clist, n_items);
+      else if (variant == 7) k_pair_f2<6, 1><<<pb, PF_WARPS * 32, 0, s>>>(d, c, d.pair_next, clist, n_items);
+      else k_pair_f2<7, 1><<<pb, PF_WARPS * 32, 0, s>>>(d, c, d.pair_next, clist, n_items);
       break;
     }
-    default: k_pair_f<4, false, MAX_TYPES><<<fb, PF_WARPS * 32, 0, s>>>(d, c, clist, n_items); break;
+    default: k_pair_f<4><<<fb, PF_WARPS * 32, 0, s>>>(d, c, clist, n_items); break;
   }
 }
 

@@ -27,7 +27,7 @@ union StepShared {
   // the forces phase: a warp works on reaction-coordinate tiles and on pair
   // clusters in any order, so both have their own tables
   struct {
-    PairF2Shared pair;
+    PairF2Shared<PF_WARPS> pair;
     CvWarpShared cv[PF_WARPS];
   } force;
   ListShared list;
@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(STEP_THREADS, MINB)
       if (item < n_cv) {
         cv_tile(d, c, sh.force.cv[wib], item);
       } else if (item < n_cv + n_pair) {
-        pair_cluster_f2(d, c, sh.force.pair, item - n_cv);
+        pair_cluster_f2<1>(d, c, sh.force.pair, item - n_cv);
       } else if (item < n_cv + n_pair + n_bond) {
         const int k = (item - n_cv - n_pair) * 32 + lane;
         if (k < d.n_trials * d.max_nbg) bonded_group(d, k / d.max_nbg, k % d.max_nbg);
