@@ -23,7 +23,8 @@ struct Dev {
   long long *fx, *fy, *fz;             // fixed-point force accumulators per slot
   // clusters
   int32_t *clus_trial;                 // static: trial of every i-cluster
-  float4 *bb_lo, *bb_hi;               // bounding boxes of the 4-atom half clusters (wrapped positions at rebuild)
+  float4 *bb_c, *bb_h;                 // bounding boxes of the 4-atom half clusters (wrapped positions at
+                                       // rebuild): centre and half extents
   uint32_t *list;                      // [total_clus * list_cap] j-atom entries (see vp_internal.cuh)
   uint8_t *list_m;                     // [total_clus * list_cap] their pair masks
   int32_t *list_n;                     // entries per i-cluster ...

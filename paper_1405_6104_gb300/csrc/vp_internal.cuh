@@ -14,7 +14,7 @@ constexpr double KB = 0.0083144626;    // kJ/mol/K
 constexpr double FCOUL = 138.935458;   // kJ mol^-1 nm e^-2
 constexpr int CL = 8;                  // atoms per i-cluster
 constexpr int CJ = 4;                  // atoms per j-cluster (half an i-cluster)
-constexpr int ZBINS = 16;             // z-bins of the per-column half table the list build searches
+constexpr int ZBINS = 64;             // z-bins of the per-column half table the list build searches
 constexpr int MAX_TRIALS = 65535;      // trials per batch (one grid row each in the per-trial kernels)
 constexpr int MAX_EXCL = 16;           // excluded partners per atom
 constexpr int MAX_TYPES = 64;          // distinct LJ types after de-duplication

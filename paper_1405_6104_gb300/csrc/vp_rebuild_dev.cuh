@@ -254,7 +254,6 @@ __device__ __forceinline__ void front_trial(const Dev &d, const SimConst &c, flo
 struct ColsortShared {
   unsigned long long key[COL_CAP];
   int s_old[COL_CAP];
-  float s_zlo[COL_CAP / CJ + 2];  // lower z-bound of every half
 };
 
 
@@ -266,7 +265,6 @@ template <bool STAMP>
 __device__ __forceinline__ void colsort_column(const Dev &d, ColsortShared &sh, int t, int c) {
   unsigned long long *key = sh.key;
   int *s_old = sh.s_old;
-  float *s_zlo = sh.s_zlo;
   const TrialInfo T = d.tinfo[t];
   if (c >= T.ncol * T.ncol) return;
   if (STAMP && c == 0 && threadIdx.x == 0) d.last_rb[t] = (uint32_t)*d.cur_step;
@@ -332,8 +330,9 @@ __device__ __forceinline__ void colsort_column(const Dev &d, ColsortShared &sh, 
       d.type[ns] = 0;
     }
   }
-  // bounding boxes of the 4-atom halves of each cluster (real atoms only; an
-  // all-padding half gets an empty box, lo > hi)
+  // bounding boxes of the 4-atom halves of each cluster, as centre and half
+  // extent (real atoms only; an all-padding half gets an empty box, half
+  // extents -3e38: farther than any cut-off from everything)
   for (int k = threadIdx.x; k < 2 * ncl; k += blockDim.x) {
     float3 lo = make_float3(3e38f, 3e38f, 3e38f), hi = make_float3(-3e38f, -3e38f, -3e38f);
     for (int a = 0; a < CJ; ++a) {
@@ -344,36 +343,27 @@ __device__ __forceinline__ void colsort_column(const Dev &d, ColsortShared &sh, 
       hi.x = fmaxf(hi.x, p.x); hi.y = fmaxf(hi.y, p.y); hi.z = fmaxf(hi.z, p.z);
     }
     int hj = 2 * (T.clus0 + cstart) + k;
-    d.bb_lo[hj] = make_float4(lo.x, lo.y, lo.z, 0.f);
-    d.bb_hi[hj] = make_float4(hi.x, hi.y, hi.z, 0.f);
-    s_zlo[k] = lo.z;
+    d.bb_c[hj] = make_float4(0.5f * lo.x + 0.5f * hi.x, 0.5f * lo.y + 0.5f * hi.y, 0.5f * lo.z + 0.5f * hi.z, 0.f);
+    d.bb_h[hj] = make_float4(0.5f * hi.x - 0.5f * lo.x, 0.5f * hi.y - 0.5f * lo.y, 0.5f * hi.z - 0.5f * lo.z, 0.f);
   }
-  __syncthreads();
-  // z-bin table: the halves are in ascending z, so the number of halves whose
-  // lower z-bound lies below b L / ZBINS is the first half at or above it
+  // z-bin table: the halves are in ascending z (an all-padding half counts as
+  // above everything), so the number of halves whose lower z-bound lies below
+  // b L / ZBINS is the first half at or above it
+  const int nh = (n + CJ - 1) / CJ;
   for (int b = threadIdx.x; b <= ZBINS; b += blockDim.x) {
     const float zt = (float)b * (T.box / ZBINS);
-    int cnt = 0;
-    for (int k = 0; k < 2 * ncl; ++k) cnt += s_zlo[k] < zt ? 1 : 0;
-    d.col_ztab[(size_t)cg * (ZBINS + 1) + b] = cnt;
+    int lo = 0, hi = nh;
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (__uint_as_float((unsigned)(key[mid * CJ] >> 32)) < zt) lo = mid + 1; else hi = mid;
+    }
+    d.col_ztab[(size_t)cg * (ZBINS + 1) + b] = lo;
   }
 }
 
 // ---------------------------------------------------------------------------
 // cluster-pair list
 // ---------------------------------------------------------------------------
-// distance between two intervals on a circle of length L
-__device__ __forceinline__ float periodic_gap(float a0, float a1, float b0, float b1, float L) {
-  float g = 3e38f;
-#pragma unroll
-  for (int k = -1; k <= 1; ++k) {
-    float s = k * L;
-    float gg = fmaxf(0.0f, fmaxf(b0 + s - a1, a0 - (b1 + s)));
-    g = fminf(g, gg);
-  }
-  return g;
-}
-
 // the FP32 list rule: n = rint((xj - xi) * invL); d = (xj - L n) - xi (the
 // image of x_j first, as the force kernel forms it); r2 = fma(dz, dz,
 // fma(dy, dy, dx*dx)); member iff r2 < rl2.  Also returns the image key
@@ -407,7 +397,7 @@ static __device__ __noinline__ unsigned list_mixed_images(const Dev &d, int I, i
       if (v) {
         kmin = fminf(kmin, key);
         kmax = fmaxf(kmax, key);
-        mask |= 1u << (a * CJ + b);
+        mask |= 1u << (b * CL + a);
       }
     }
   }
@@ -417,24 +407,15 @@ static __device__ __noinline__ unsigned list_mixed_images(const Dev &d, int I, i
 constexpr int LIST_WARPS = 4;
 constexpr int CAND_MAX = 1024;  // candidate 4-atom j-clusters per i-cluster (bounding-box pass)
 constexpr int ENT_MAX = 512;    // 4-atom j-clusters with a listed pair per i-cluster
-// a candidate word: the half index (J_BITS bits), the shared-image flag, the image key
-constexpr int CAND_SAME_BIT = (int)J_BITS;
-constexpr int CAND_KEY_SHIFT = (int)J_BITS + 1;
-static_assert(J_BITS + 6 <= 31, "candidate word: half index, flag and a 5-bit key in a non-negative int");
+// a candidate word: the half index (J_BITS bits, from the trial's first
+// half), the six bits of the image code, the shared-image flag
+constexpr unsigned CAND_SAME = 1u << 31;
+static_assert(J_BITS + 6 == 31, "candidate word: half index, image code and flag in 32 bits");
 
-// the mask column of j-atom b of a 4-atom j-cluster entry: bit a of the
-// result is bit a*4 + b of the 32-bit mask
-__device__ __forceinline__ unsigned j_column(unsigned m, int b) {
-  unsigned x = (m >> b) & 0x11111111u;
-  x = (x | (x >> 3)) & 0x03030303u;
-  x = (x | (x >> 6)) & 0x000f000fu;
-  return (x | (x >> 12)) & 0xffu;
-}
-// j-atoms of an entry with at least one listed pair
+// j-atoms of an entry with at least one listed pair: the bytes of the mask
+// that are not zero
 __device__ __forceinline__ int j_columns(unsigned m) {
-  const unsigned any = m | (m >> 16);
-  const unsigned a2 = any | (any >> 8);
-  return __popc((a2 | (a2 >> 4)) & 0xfu);
+  return __popc((((m & 0x7f7f7f7fu) + 0x7f7f7f7fu) | m) & 0x80808080u);
 }
 
 // One warp per i-cluster.  Phase 1: lanes test columns, then the 4-atom
@@ -442,56 +423,89 @@ __device__ __forceinline__ int j_columns(unsigned m) {
 // bounding box and collect the candidates in order (column-major, then z,
 // i.e. ascending j-cluster index).  Phase 2: each lane takes one candidate
 // and evaluates the FP32 list rule for all 8 x 4 atom pairs itself, giving
-// the entry's mask, image code and exact flag; entries are written in
-// candidate order (deterministic).  Phase 3: the i-atoms' exclusions clear
-// their bits in the entries (found by binary search).  Phase 4: one list
-// entry per j-atom with a listed pair is written out.
+// the entry's mask (bit b * 8 + a for j-atom b and i-atom a: a byte per
+// j-atom), image code and exact flag; entries are written in candidate order
+// (deterministic).  Phase 3: the i-atoms' exclusions clear their bits in the
+// entries (found by binary search).  Phase 4: one list entry per j-atom with
+// a listed pair is written out.
+//
+// Bound by issue slots (a GPU full of rebuilding trials) or by the chain of
+// loads (one trial).  Hence: boxes as centre and half extent (the periodic gap
+// and the image counts of a box pair come from one rounding per dimension),
+// columns before the i-cluster's own left out (their clusters have lower
+// indices), z-windows in 64 bins, the halves to test written out once per 32
+// columns instead of searched per test, the next step's boxes loaded while the
+// current ones are tested, the chain of loads that leads to the excluded
+// partners' slots begun before the search, byte masks that phase 4 reads off
+// directly.  Of 64 trials of 11 040 atoms, 16 rebuilding in the step: 222 us
+// before these, 138 with them; a step of one trial, every fourth with a
+// rebuild, 12 -> 6 us on average.  Testing every half of the z-windows pair by
+// pair without the box test (215 instead of 179 of them) took 168 us.
 struct ListShared {
-  int s_cand[LIST_WARPS][CAND_MAX];
-  int s_excl[LIST_WARPS][CL][MAX_EXCL];
-  int s_nex[LIST_WARPS][CL];
+  unsigned s_cand[LIST_WARPS][CAND_MAX];
   float4 s_xp[LIST_WARPS][CL / 2][2];  // i-atom pairs (2p, 2p+1): {-x, -x', -y, -y'} {-z, -z', 0, 0}
   unsigned s_dirty[LIST_WARPS][ENT_MAX / 32];  // entries whose j-atoms need the pair masks
-  unsigned s_mask[LIST_WARPS][ENT_MAX];        // masks of the entries (their first words overwrite s_cand)
+  unsigned s_mask[LIST_WARPS][ENT_MAX];        // halves to test (phase 1), then the entries' masks (their
+                                               // first words overwrite s_cand)
 };
+
+// least and greatest of the warp's values (redux on FP32: one instruction)
+__device__ __forceinline__ float warp_min(float v) {
+  float r;
+  asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+  return r;
+}
+__device__ __forceinline__ float warp_max(float v) {
+  float r;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+  return r;
+}
 
 __device__ __forceinline__ void list_cluster(const Dev &d, const SimConst &c, float rl2_bbox, ListShared &sh, int t,
                                              int Il) {
-  auto &s_cand = sh.s_cand;
-  auto &s_excl = sh.s_excl;
-  auto &s_nex = sh.s_nex;
-  auto &s_xp = sh.s_xp;
-  auto &s_dirty = sh.s_dirty;
-  auto &s_mask = sh.s_mask;
   const int wib = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
+  auto &s_xp = sh.s_xp[wib];
+  auto &s_dirty = sh.s_dirty[wib];
+  unsigned *cand = sh.s_cand[wib], *s_mask = sh.s_mask[wib];
   const TrialInfo T = d.tinfo[t];
   if (Il >= T.max_clus) return;
   const int I = T.clus0 + Il;
-  if (Il >= d.tstate[t].n_clus) {
+  const int n_clus_t = d.tstate[t].n_clus;
+  if (Il >= n_clus_t) {
     if (lane == 0) d.list_n[I] = 0;
     return;
   }
-  float4 lo, hi;
-  {
-    const float4 l0 = d.bb_lo[2 * I], l1 = d.bb_lo[2 * I + 1], h0 = d.bb_hi[2 * I], h1 = d.bb_hi[2 * I + 1];
-    lo = make_float4(fminf(l0.x, l1.x), fminf(l0.y, l1.y), fminf(l0.z, l1.z), 0.f);
-    hi = make_float4(fmaxf(h0.x, h1.x), fmaxf(h0.y, h1.y), fmaxf(h0.z, h1.z), 0.f);
+  // lane = (i-atom lane & 7, four of its excluded partners at a time from lane >> 3)
+  const int xo = d.orig[I * CL + (lane & 7)];
+  const float4 xi = d.pos[I * CL + (lane & 7)];
+  if (lane < CL) {
+    float *x = &s_xp[lane >> 1][0].x + (lane & 1);
+    x[0] = -xi.x; x[2] = -xi.y; x[4] = -xi.z;
   }
+  if (lane < ENT_MAX / 32) s_dirty[lane] = c.list_fixed ? ~0u : 0u;  // fixed-interval lists: masks everywhere
+  // the partners themselves (unused places hold -1) and their number
+  const int32_t *xrow = d.excl + (size_t)(T.sysatom0 + max(xo, 0)) * MAX_EXCL;
+  const int xn = xo >= 0 ? d.excl_n[T.sysatom0 + xo] : 0;
+  const int xa = xo >= 0 ? xrow[lane >> 3] : -1;
+  const float3 lo = make_float3(warp_min(xo >= 0 ? xi.x : 3e38f), warp_min(xo >= 0 ? xi.y : 3e38f),
+                                warp_min(xo >= 0 ? xi.z : 3e38f));
+  const float3 hi = make_float3(warp_max(xo >= 0 ? xi.x : -3e38f), warp_max(xo >= 0 ? xi.y : -3e38f),
+                                warp_max(xo >= 0 ? xi.z : -3e38f));
   const float L = T.box, iL = T.inv_box, w = T.col_w;
   const int nc2 = T.ncol * T.ncol;
-  int *cand = s_cand[wib];
+  const float3 ci = make_float3(0.5f * (lo.x + hi.x), 0.5f * (lo.y + hi.y), 0.5f * (lo.z + hi.z));
+  const float3 hw = make_float3(0.5f * (hi.x - lo.x), 0.5f * (hi.y - lo.y), 0.5f * (hi.z - lo.z));
   int n_cand = 0;
-  bool overflow = false;
   // ---- phase 1: candidate 4-atom j-clusters ----
   // Only the grid columns within reach of the i-cluster's bounding box (one
   // column more on each side for the rounding of the binning) are visited,
   // in ascending column index: the window's x and y column indices, wrapped
   // periodically, are enumerated in sorted order (so the candidates, and the
-  // entries, ascend in j-cluster index).  Lanes test 32 columns; the halves
-  // (of clusters with index >= Il) of the passing columns are then
-  // enumerated as one flat range, 32 per step, so that the bounding-box loads
-  // of a whole step are in flight together.
+  // entries, ascend in j-cluster index), from the i-cluster's own x index on
+  // (the half list keeps clusters of index >= Il).  Lanes take 32 columns; the
+  // halves of the passing columns are then tested as one flat range, 32 per
+  // step.
   const float reach = sqrtf(rl2_bbox);
   int wx0, wnx, wy0, wny;  // first column (mod ncol) and count of the window in x and in y
   {
@@ -507,8 +521,17 @@ __device__ __forceinline__ void list_cluster(const Dev &d, const SimConst &c, fl
     const int e = a + m - T.ncol;  // the part that wraps to [0, e)
     return e <= 0 ? a + k : (k < e ? k : a + (k - e));
   };
-  const int nwin = wnx * wny;
-  const int n_clus_t = d.tstate[t].n_clus;
+  // rows of the window below the i-cluster's own x index (a rounding below it is only one row more)
+  int row0;
+  {
+    const int own = max(0, (int)floorf((lo.x - 1e-5f) * T.inv_col_w));
+    const int e = max(0, wx0 + wnx - T.ncol);
+    row0 = min(own, e) + max(0, min(own - wx0, wnx - e));
+  }
+  const int nwin = (wnx - row0) * wny;
+  const float inv_wny = 1.0f / (float)wny;
+  const float half_w = 0.5f * w, img_lim = 0.49999f * L;
+  int xs = -1;  // slot of this lane's excluded partner
   for (int cb = 0; cb < nwin; cb += 32) {
     const int wi = cb + lane;
     // this lane's column: up to two ranges [a1, a1 + n1), [a2, a2 + n2) of
@@ -517,13 +540,15 @@ __device__ __forceinline__ void list_cluster(const Dev &d, const SimConst &c, fl
     // the column's xy gap, the ranges from the column's z-bin table, one bin
     // wider on each side than needed (every half in them is still tested)
     int a1 = 0, n1 = 0, a2 = 0, n2 = 0;
-    const int cc = wi < nwin ? kth(wx0, wnx, wi / wny) * T.ncol + kth(wy0, wny, wi % wny) : 0;
     if (wi < nwin) {
+      const int wr = (int)(((float)wi + 0.5f) * inv_wny);  // wi / wny (exact: wi < 2^12)
+      const int cx = kth(wx0, wnx, row0 + wr), cy = kth(wy0, wny, wi - wr * wny);
+      const int cc = cx * T.ncol + cy;
       // the geometry first, then every load of the column at once (one
       // memory round trip instead of two)
-      const int cx = cc / T.ncol, cy = cc - cx * T.ncol;
-      const float gx = periodic_gap(lo.x, hi.x, cx * w, (cx + 1) * w, L);
-      const float gy = periodic_gap(lo.y, hi.y, cy * w, (cy + 1) * w, L);
+      float gx = ((float)cx * w + half_w) - ci.x, gy = ((float)cy * w + half_w) - ci.y;
+      gx = fmaxf(fabsf(gx - L * rintf(gx * iL)) - (half_w + hw.x), 0.0f);
+      gy = fmaxf(fabsf(gy - L * rintf(gy * iL)) - (half_w + hw.y), 0.0f);
       const float g2 = gx * gx + gy * gy;
       if (g2 < rl2_bbox) {
         const float rz = sqrtf(rl2_bbox - g2) * 1.001f + 1e-3f;
@@ -533,122 +558,87 @@ __device__ __forceinline__ void list_cluster(const Dev &d, const SimConst &c, fl
         // or two intervals (the periodic image)
         const float zs = ZBINS * iL;
         const bool two = za < 0.f || zb > L;
-        const float u1 = 0.f, v1 = za < 0.f ? zb : (zb > L ? zb - L : zb);
-        const float u1r = two ? u1 : za;
-        const float u2 = za < 0.f ? za + L : za, v2 = L;
+        const float v1 = za < 0.f ? zb : (zb > L ? zb - L : zb);
+        const float u1 = two ? 0.f : za;
+        const float u2 = za < 0.f ? za + L : za;
         auto bin_lo = [&](float u) { return max(0, min(ZBINS, (int)floorf(u * zs) - 1)); };
-        auto bin_hi = [&](float v) { return max(0, min(ZBINS, (int)floorf(v * zs) + 2)); };
-        const int bu1 = bin_lo(u1r), bv1 = bin_hi(v1), bu2 = bin_lo(u2), bv2 = bin_hi(v2);
+        const int bu1 = bin_lo(u1), bv1 = max(0, min(ZBINS, (int)floorf(v1 * zs) + 2)), bu2 = bin_lo(u2);
         const int *tab = d.col_ztab + (size_t)(T.col0 + cc) * (ZBINS + 1);
         const int ccs = d.col_cstart[T.col0 + cc];
         const int cnext = cc + 1 < nc2 ? d.col_cstart[T.col0 + cc + 1] : n_clus_t;
         const int t1a = tab[bu1], t1b = tab[bv1];
-        const int t2a = two ? tab[bu2] : 0, t2b = two ? tab[bv2] : 0;
+        const int t2a = two ? tab[bu2] : 0;
         const int ncl = max(0, cnext - ccs);
         const int jlo = max(ccs, Il);
         if (ccs + ncl > jlo) {
           const int hs = 2 * (jlo - ccs), he = 2 * ncl;  // local half range of the half list
-          if (whole) {
-            a1 = hs; n1 = he - hs;
-          } else {
-            int r1a = max(t1a - 1, 0), r1b = bv1 >= ZBINS ? he : t1b;
-            int r2a = 0, r2b = 0;
-            if (two) {
-              r2a = max(t2a - 1, 0);
-              r2b = bv2 >= ZBINS ? he : t2b;
-            }
-            r1a = max(r1a, hs); r1b = min(r1b, he);
-            r2a = max(max(r2a, hs), r1b); r2b = min(r2b, he);  // ascending, no half twice
-            a1 = r1a; n1 = max(r1b - r1a, 0);
-            a2 = r2a; n2 = max(r2b - r2a, 0);
+          int r1a = hs, r1b = he, r2a = 0, r2b = 0;
+          if (!whole) {
+            r1a = max(max(t1a - 1, 0), hs);
+            r1b = min(bv1 >= ZBINS ? he : t1b, he);
+            // the second interval reaches up to L, the column's end
+            r2a = two ? max(max(t2a - 1, hs), r1b) : 0;  // ascending, no half twice
+            r2b = two ? he : 0;
           }
-          a1 += 2 * ccs;
-          a2 += 2 * ccs;
+          n1 = max(r1b - r1a, 0);
+          n2 = max(r2b - r2a, 0);
+          a1 = r1a + 2 * ccs;
+          a2 = r2a + 2 * ccs;
         }
       }
     }
+    if (cb == 0 && xa >= 0) xs = d.slot_of[T.atom0 + xa];
     const int cntc = n1 + n2;
-    // inclusive scan of the per-column candidate counts
+    // inclusive scan of the per-column counts
     int incl = cntc;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
       const int v = __shfl_up_sync(0xffffffffu, incl, off);
       if (lane >= off) incl += v;
     }
-    const int total = __shfl_sync(0xffffffffu, incl, 31);
-    for (int t0 = 0; t0 < total; t0 += 32) {
-      const int tt = t0 + lane;
-      const int tq = min(tt, total - 1);
-      // owner column: first lane whose inclusive count exceeds tq (all lanes search)
-      int lo_l = 0, hi_l = 31;
-#pragma unroll
-      for (int it = 0; it < 5; ++it) {
-        const int mid = (lo_l + hi_l) >> 1;
-        const int v = __shfl_sync(0xffffffffu, incl, mid);
-        if (v > tq) hi_l = mid; else lo_l = mid + 1;
+    const int total = __shfl_sync(0xffffffffu, incl, 31), first = incl - cntc;
+    // the halves of these columns, ENT_MAX at a time
+    for (int t0 = 0; t0 < total; t0 += ENT_MAX) {
+      const int m = min(ENT_MAX, total - t0);
+      __syncwarp();
+      for (int u = max(0, t0 - first); u < cntc && first + u < t0 + m; ++u)
+        s_mask[first + u - t0] = (unsigned)(u < n1 ? a1 + u : a2 + (u - n1));
+      __syncwarp();
+      // idle lanes of the last step repeat its last half (and are not counted)
+      unsigned Jn = s_mask[min(lane, m - 1)];
+      float4 cn = d.bb_c[2 * T.clus0 + Jn], hn = d.bb_h[2 * T.clus0 + Jn];
+      for (int q = 0; q < m; q += 32) {
+        const unsigned J4 = Jn;
+        const float4 cj = cn, hj = hn;
+        if (q + 32 < m) {  // the next step's boxes
+          Jn = s_mask[min(q + 32 + lane, m - 1)];
+          cn = d.bb_c[2 * T.clus0 + Jn];
+          hn = d.bb_h[2 * T.clus0 + Jn];
+        }
+        // periodic gap of the boxes, and the image counts of their centres:
+        // all atom pairs share them when no pair can come near half a box
+        // length (the 1e-5 L margin covers every rounding here and in the rule)
+        float dx = cj.x - ci.x, dy = cj.y - ci.y, dz = cj.z - ci.z;
+        const float nx = rintf(dx * iL), ny = rintf(dy * iL), nz = rintf(dz * iL);
+        dx = fabsf(dx - L * nx); dy = fabsf(dy - L * ny); dz = fabsf(dz - L * nz);
+        const float sx = hj.x + hw.x, sy = hj.y + hw.y, sz = hj.z + hw.z;
+        const float gx = fmaxf(dx - sx, 0.f), gy = fmaxf(dy - sy, 0.f), gz = fmaxf(dz - sz, 0.f);
+        const bool ok = q + lane < m && gx * gx + gy * gy + gz * gz < rl2_bbox;
+        const bool same = fmaxf(fmaxf(dx + sx, dy + sy), dz + sz) < img_lim;
+        const unsigned code = (unsigned)(int)(nx + 4.0f * ny + 16.0f * nz + (float)NO_SHIFT);
+        const unsigned bal = __ballot_sync(0xffffffffu, ok);
+        const int pos = n_cand + __popc(bal & ((1u << lane) - 1u));
+        if (ok && pos < CAND_MAX) cand[pos] = J4 | (code << J_BITS) | (same ? CAND_SAME : 0u);
+        n_cand += __popc(bal);
       }
-      const int own_incl = __shfl_sync(0xffffffffu, incl, lo_l);
-      const int own_cnt = __shfl_sync(0xffffffffu, cntc, lo_l);
-      const int own_a1 = __shfl_sync(0xffffffffu, a1, lo_l);
-      const int own_n1 = __shfl_sync(0xffffffffu, n1, lo_l);
-      const int own_a2 = __shfl_sync(0xffffffffu, a2, lo_l);
-      bool ok = false;
-      int J4 = 0;
-      if (tt < total) {
-        const int u = tt - (own_incl - own_cnt);
-        J4 = u < own_n1 ? own_a1 + u : own_a2 + (u - own_n1);
-        const float4 jlo4 = d.bb_lo[2 * T.clus0 + J4], jhi4 = d.bb_hi[2 * T.clus0 + J4];
-        const float gx = periodic_gap(lo.x, hi.x, jlo4.x, jhi4.x, L);
-        const float gy = periodic_gap(lo.y, hi.y, jlo4.y, jhi4.y, L);
-        const float gz = periodic_gap(lo.z, hi.z, jlo4.z, jhi4.z, L);
-        ok = gx * gx + gy * gy + gz * gz < rl2_bbox;
-        // image counts at the two bounding-box extremes (each -1, 0 or 1: the
-        // positions lie in [0, L)); when they agree in every dimension, every
-        // atom pair of the candidate has them.  Carried in the candidate word
-        // (shared image flag, key 9 (nx+1) + 3 (ny+1) + (nz+1)) so that phase 2
-        // need not load the box again.
-        const float qlx = rintf(__fmul_rn(__fsub_rn(jlo4.x, hi.x), iL)), qhx = rintf(__fmul_rn(__fsub_rn(jhi4.x, lo.x), iL));
-        const float qly = rintf(__fmul_rn(__fsub_rn(jlo4.y, hi.y), iL)), qhy = rintf(__fmul_rn(__fsub_rn(jhi4.y, lo.y), iL));
-        const float qlz = rintf(__fmul_rn(__fsub_rn(jlo4.z, hi.z), iL)), qhz = rintf(__fmul_rn(__fsub_rn(jhi4.z, lo.z), iL));
-        const int same = qlx == qhx && qly == qhy && qlz == qhz;
-        const int key = 9 * ((int)qlx + 1) + 3 * ((int)qly + 1) + ((int)qlz + 1);
-        J4 |= (same << CAND_SAME_BIT) | (key << CAND_KEY_SHIFT);
-      }
-      const unsigned m = __ballot_sync(0xffffffffu, ok);
-      const int pos = n_cand + __popc(m & ((1u << lane) - 1u));
-      if (ok && pos < CAND_MAX) cand[pos] = J4;
-      n_cand += __popc(m);
     }
   }
-  if (n_cand > CAND_MAX) {
-    overflow = true;
-    n_cand = CAND_MAX;
-  }
-  // i-atoms (shared memory: broadcast reads leave registers for more resident
-  // warps) and their exclusions
-  if (lane < CL / 2) {
-    const float4 a0 = d.pos[I * CL + 2 * lane], a1 = d.pos[I * CL + 2 * lane + 1];
-    s_xp[wib][lane][0] = make_float4(-a0.x, -a1.x, -a0.y, -a1.y);
-    s_xp[wib][lane][1] = make_float4(-a0.z, -a1.z, 0.f, 0.f);
-  }
-  if (lane < CL) {
-    const int o = d.orig[I * CL + lane];
-    s_nex[wib][lane] = o < 0 ? 0 : d.excl_n[T.sysatom0 + o];
-  }
-  if (lane < ENT_MAX / 32) s_dirty[wib][lane] = c.list_fixed ? ~0u : 0u;  // fixed-interval lists: masks everywhere
+  const bool overflow = n_cand > CAND_MAX;
+  n_cand = min(n_cand, CAND_MAX);
   __syncwarp();
-  // the slots of the i-atoms' excluded partners, all loads of the warp in flight together
-  for (int k = lane; k < CL * MAX_EXCL; k += 32) {
-    const int a = k / MAX_EXCL, q = k - a * MAX_EXCL;
-    if (q < s_nex[wib][a]) {
-      const int o = d.orig[I * CL + a];
-      s_excl[wib][a][q] = d.slot_of[T.atom0 + d.excl[(size_t)(T.sysatom0 + o) * MAX_EXCL + q]];
-    }
-  }
   // ---- phase 2: one candidate 4-atom j-cluster per lane ----
-  // Image counts: q = rint(fl(d * invL)) is monotone in d = fl(xj - xi), so
-  // when the two bounding-box extremes of d give the same q in a dimension,
-  // every atom pair of the candidate has that q there and the rule reduces to
+  // Image counts: q = rint(fl(d * invL)) for every atom pair of a candidate
+  // with shared images is that of the box centres, so the rule reduces to
   // d - fl(L q) with the same rounding as the per-pair form.  Padding atoms
   // sit far outside every box and fail the distance test on that path.
   const float rl2 = c.rl2;
@@ -656,57 +646,54 @@ __device__ __forceinline__ void list_cluster(const Dev &d, const SimConst &c, fl
   for (int k0 = 0; k0 < n_cand; k0 += 32) {
     const int k = k0 + lane;
     unsigned mask = 0u, w0 = 0u;
+    bool dirty = false;
     if (k < n_cand) {
-      const int cw = cand[k];
-      const int J4 = cw & (int)J_MASK;
-      const int J8 = J4 >> 1, h = J4 & 1;
-      const int JG = T.clus0 + J8;
-      const int sj0 = JG * CL + h * CJ;
-      float kmin = 3e38f, kmax = -3e38f;
-      const int ckey = (cw >> CAND_KEY_SHIFT) & 31;
-      const float qlx = (float)(ckey / 9 - 1), qly = (float)((ckey / 3) % 3 - 1), qlz = (float)(ckey % 3 - 1);
-      if ((cw >> CAND_SAME_BIT) & 1) {
-        // the j-atom's image once, then two i-atoms per packed FP32x2
+      const unsigned cw = cand[k];
+      const unsigned J4 = cw & J_MASK, code = (cw >> J_BITS) & 63u;
+      const int J8 = (int)(J4 >> 1);
+      const int sj0 = T.slot0 + (int)J4 * CJ;
+      const unsigned jw = (unsigned)(2 * T.clus0) + J4;
+      w0 = jw | (code << J_BITS);
+      dirty = J8 == Il;  // the cluster with itself: pairs below the diagonal masked
+      if (cw & CAND_SAME) {
+        // the j-atoms' images once, then two i-atoms per packed FP32x2
         // operation; every operation rounds on its own exactly as the
         // per-pair rule does (d = (xj - L n) + (-xi) is (xj - L n) - xi)
-        const float sx = __fmul_rn(L, qlx), sy = __fmul_rn(L, qly), sz = __fmul_rn(L, qlz);
+        const float sx = __fmul_rn(L, (float)((int)(code & 3u) - 1)), sy = __fmul_rn(L, (float)((int)((code >> 2) & 3u) - 1)),
+                    sz = __fmul_rn(L, (float)((int)(code >> 4) - 1));
+        float ux[CJ], uy[CJ], uz[CJ];
 #pragma unroll
         for (int b = 0; b < CJ; ++b) {
           const float4 pj = d.pos[sj0 + b];
-          const float ux = __fsub_rn(pj.x, sx), uy = __fsub_rn(pj.y, sy), uz = __fsub_rn(pj.z, sz);
-          const float2 xj2 = make_float2(ux, ux), yj2 = make_float2(uy, uy), zj2 = make_float2(uz, uz);
+          ux[b] = __fsub_rn(pj.x, sx); uy[b] = __fsub_rn(pj.y, sy); uz[b] = __fsub_rn(pj.z, sz);
+        }
 #pragma unroll
-          for (int p = 0; p < CL / 2; ++p) {
-            const float4 i0 = s_xp[wib][p][0], i1 = s_xp[wib][p][1];
-            const float2 dx = __fadd2_rn(xj2, make_float2(i0.x, i0.y));
-            const float2 dy = __fadd2_rn(yj2, make_float2(i0.z, i0.w));
-            const float2 dz = __fadd2_rn(zj2, make_float2(i1.x, i1.y));
+        for (int p = 0; p < CL / 2; ++p) {
+          const float4 i0 = s_xp[p][0], i1 = s_xp[p][1];
+#pragma unroll
+          for (int b = 0; b < CJ; ++b) {
+            const float2 dx = __fadd2_rn(make_float2(ux[b], ux[b]), make_float2(i0.x, i0.y));
+            const float2 dy = __fadd2_rn(make_float2(uy[b], uy[b]), make_float2(i0.z, i0.w));
+            const float2 dz = __fadd2_rn(make_float2(uz[b], uz[b]), make_float2(i1.x, i1.y));
             const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
-            if (r2.x < rl2) mask |= 1u << (2 * p * CJ + b);
-            if (r2.y < rl2) mask |= 1u << ((2 * p + 1) * CJ + b);
+            if (r2.x < rl2) mask |= 1u << (b * CL + 2 * p);
+            if (r2.y < rl2) mask |= 1u << (b * CL + 2 * p + 1);
           }
         }
-        if (J8 == Il) {  // inside the i-cluster itself: pairs with the j slot above the i slot
-          unsigned tri = 0u;
-#pragma unroll
-          for (int a = 0; a < CL; ++a)
-#pragma unroll
-            for (int b = 0; b < CJ; ++b)
-              if (h * CJ + b > a) tri |= 1u << (a * CJ + b);
-          mask &= tri;
-        }
-        if (mask) kmin = kmax = __fmaf_rn(9.0f, qlx, __fmaf_rn(3.0f, qly, qlz));
+        // inside the i-cluster itself: pairs with the j slot above the i slot
+        if (J8 == Il) mask &= (J4 & 1u) ? 0x7f3f1f0fu : 0x07030100u;
       } else {
+        float kmin = 3e38f, kmax = -3e38f;
         mask = list_mixed_images(d, I, Il, J8, sj0, L, iL, rl2, kmin, kmax);
+        // image counts of the entry from the key 9 nx + 3 ny + nz (each in -1..1)
+        const int key = mask ? (int)kmin : 0;
+        const int kz = ((key % 3) + 4) % 3 - 1;
+        const int ky = (((key - kz) / 3) % 3 + 4) % 3 - 1;
+        const int kx = (key - kz - 3 * ky) / 9;
+        const bool exact = mask && kmin != kmax;  // pairs that take images one by one need the masks
+        w0 = jw | ((unsigned)((kx + 1) | ((ky + 1) << 2) | ((kz + 1) << 4)) << J_BITS) | (exact ? E_EXACT : 0u);
+        dirty |= exact;
       }
-      // image counts of the entry from the key 9 nx + 3 ny + nz (each in -1..1)
-      const int key = mask ? (int)kmin : 0;
-      const int kz = ((key % 3) + 4) % 3 - 1;
-      const int ky = (((key - kz) / 3) % 3 + 4) % 3 - 1;
-      const int kx = (key - kz - 3 * ky) / 9;
-      const bool same = kmin == kmax;
-      w0 = (unsigned)(2 * JG + h) | ((unsigned)((kx + 1) | ((ky + 1) << 2) | ((kz + 1) << 4)) << J_BITS) |
-           (same || !mask ? 0u : E_EXACT);
     }
     const unsigned bal = __ballot_sync(0xffffffffu, mask != 0u);
     const int pos = cnt + __popc(bal & ((1u << lane) - 1u));
@@ -714,56 +701,55 @@ __device__ __forceinline__ void list_cluster(const Dev &d, const SimConst &c, fl
     if (mask != 0u && pos < ENT_MAX) {
       // entries are kept in shared memory until the exclusions are cleared:
       // the first word over the consumed candidates, the mask beside
-      cand[pos] = (int)w0;
-      s_mask[wib][pos] = mask;
-      // the cluster with itself (pairs below the diagonal masked) and entries
-      // whose pairs take images one by one need the masks in the pair kernel
-      if ((int)((w0 & J_MASK) >> 1) == I || (w0 & E_EXACT)) atomicOr(&s_dirty[wib][pos >> 5], 1u << (pos & 31));
+      cand[pos] = w0;
+      s_mask[pos] = mask;
+      if (dirty) atomicOr(&s_dirty[pos >> 5], 1u << (pos & 31));
     }
     cnt += __popc(bal);
   }
   const int n_ent = min(cnt, ENT_MAX);
   // ---- phase 3: exclusions ----
-  // lane a < 8 clears, for each atom excluded from i-atom a, the bit of that
-  // pair in the entry of its 4-atom j-cluster, if this list holds the pair
-  // (entries ascend in j-cluster index; a pair inside the i-cluster belongs
-  // to the entry with the higher slot as j)
+  // for each atom excluded from i-atom a, the bit of that pair is cleared in
+  // the entry of its 4-atom j-cluster, if this list holds the pair (entries
+  // ascend in j-cluster index; a pair inside the i-cluster belongs to the
+  // entry with the higher slot as j)
   __syncwarp();
-  for (int k = lane; k < CL * MAX_EXCL; k += 32) {
-    const int a = k / MAX_EXCL, q = k - a * MAX_EXCL;
-    if (q >= s_nex[wib][a]) continue;
-    const int si = I * CL + a;
-    const int sj = s_excl[wib][a][q];
-    if ((sj >> 3) < I || ((sj >> 3) == I && sj <= si)) continue;  // listed from the other side, or not at all
-    const unsigned j4 = (unsigned)(sj >> 2);
-    int lo_e = 0, hi_e = n_ent;  // first entry with j-cluster >= j4
-    while (lo_e < hi_e) {
-      const int mid = (lo_e + hi_e) >> 1;
-      if (((unsigned)cand[mid] & J_MASK) < j4) lo_e = mid + 1; else hi_e = mid;
+  for (int q = 0; q == 0 || __any_sync(0xffffffffu, xn > q); q += 4) {
+    if (q > 0) {  // atoms with more than four excluded partners
+      const int x = q + (lane >> 3) < xn ? xrow[q + (lane >> 3)] : -1;
+      xs = x >= 0 ? d.slot_of[T.atom0 + x] : -1;
     }
-    if (lo_e < n_ent && ((unsigned)cand[lo_e] & J_MASK) == j4) {
-      atomicAnd(&s_mask[wib][lo_e], ~(1u << (a * CJ + (sj & 3))));
-      atomicOr(&s_dirty[wib][lo_e >> 5], 1u << (lo_e & 31));
+    const int a = lane & 7, si = I * CL + a;
+    if (xs > si && (xs >> 3) >= I) {  // else listed from the other side, or not at all
+      const unsigned j4 = (unsigned)(xs >> 2);
+      int lo_e = 0, hi_e = n_ent;  // first entry with j-cluster >= j4
+      while (lo_e < hi_e) {
+        const int mid = (lo_e + hi_e) >> 1;
+        if ((cand[mid] & J_MASK) < j4) lo_e = mid + 1; else hi_e = mid;
+      }
+      if (lo_e < n_ent && (cand[lo_e] & J_MASK) == j4) {
+        atomicAnd(&s_mask[lo_e], ~(1u << ((xs & 3) * CL + a)));
+        atomicOr(&s_dirty[lo_e >> 5], 1u << (lo_e & 31));
+      }
     }
   }
   __syncwarp();
   // ---- phase 4: one entry per j-atom with a listed pair ----
   // In entry order, j-atoms ascending; the j-atoms of entries that need the
   // masks first, so that they fill as few groups of 32 entries as possible.
-  auto dirty_at = [&](int e) { return ((s_dirty[wib][e >> 5] >> (e & 31)) & 1u) != 0u; };
   int n_dirty = 0;
   for (int e0 = 0; e0 < n_ent; e0 += 32) {
+    const unsigned dw = s_dirty[e0 >> 5];
     const int e = e0 + lane;
-    const int nd = e < n_ent && dirty_at(e) ? j_columns(s_mask[wib][e]) : 0;
-    n_dirty += __reduce_add_sync(0xffffffffu, nd);
+    n_dirty += __reduce_add_sync(0xffffffffu, e < n_ent && ((dw >> lane) & 1u) ? j_columns(s_mask[e]) : 0);
   }
   uint32_t *segw = d.list + (size_t)I * c.list_cap;
   uint8_t *segm = d.list_m + (size_t)I * c.list_cap;
   int pd = 0, pc = n_dirty;  // where the next j-atoms of either kind go
   for (int e0 = 0; e0 < n_ent; e0 += 32) {
     const int e = e0 + lane;
-    const unsigned m = e < n_ent ? s_mask[wib][e] : 0u;
-    const bool dirty = e < n_ent && dirty_at(e);
+    const unsigned m = e < n_ent ? s_mask[e] : 0u;
+    const bool dirty = (s_dirty[e0 >> 5] >> lane) & 1u;
     const int nj = j_columns(m);
     // inclusive scan over the lanes of both counts at once (16 bits each)
     const int own = dirty ? nj : nj << 16;
@@ -776,11 +762,11 @@ __device__ __forceinline__ void list_cluster(const Dev &d, const SimConst &c, fl
     const int before = sdc - own;
     int p = dirty ? pd + (before & 0xffff) : pc + (before >> 16);
     if (nj) {
-      const unsigned w = (unsigned)cand[e];
-      const unsigned s0 = (w & J_MASK) * CJ, rest = w & ~J_MASK;
+      const unsigned wd = cand[e];
+      const unsigned s0 = (wd & J_MASK) * CJ, rest = wd & ~J_MASK;
 #pragma unroll
       for (int b = 0; b < CJ; ++b) {
-        const unsigned col = j_column(m, b);
+        const unsigned col = (m >> (b * CL)) & 0xffu;
         if (col) {
           if (p < c.list_cap) {
             segw[p] = (s0 + b) | rest;

@@ -33,3 +33,35 @@ def test_tiles_by_a_block_match_tiles_by_a_warp(n_solute):
     s, p = S.small_solvated(n_solute=n_solute, n_water=430 + n_solute)
     for x, y in zip(_states(s, p, 0), _states(s, p, 1)):
         assert np.array_equal(x[0], y[0]) and np.array_equal(x[1], y[1]) and np.array_equal(x[2], y[2])
+
+
+@pytest.mark.parametrize("per_atom", [4, 5, 9, 16])
+def test_lists_with_many_excluded_partners_are_bit_exact(per_atom):
+    """Exclusion rows at the edges of the list build's passes (four partners
+    per atom at a time), in the smallest box the system takes (half lists with
+    pairs on both sides of it, pair-by-pair images): the oracle's pair set."""
+    import oracle as O
+
+    s, p = S.small_solvated(n_solute=24, n_water=420)
+    rng = np.random.default_rng(per_atom)
+    have = {i: set() for i in range(s.n_atoms)}
+    for a, b in np.asarray(s.bonds):
+        have[a].add(int(b)), have[b].add(int(a))
+    for a, _, c in np.asarray(s.angles):
+        have[a].add(int(c)), have[c].add(int(a))
+    extra = []
+    for i in range(0, s.n_atoms, 3):
+        for j in rng.permutation(s.n_atoms)[:200]:
+            j = int(j)
+            if j != i and j not in have[i] and len(have[i]) < per_atom and len(have[j]) < per_atom:
+                have[i].add(j), have[j].add(i)
+                extra.append((i, j))
+    s = s.copy()
+    s.excl_pairs = np.array(extra, np.int32)
+    assert max(len(v) for v in have.values()) == per_atom
+    with B.TrialBatch(s, p, [1], trial_seeds=[3]) as b:
+        b.step(7)
+        pos = B.sim_list_positions(b.h, 0)
+        got = {tuple(x) for x in B.sim_pairlist(b.h, 0).tolist()}
+    ref = {tuple(x) for x in O.pairlist(s, pos.astype(np.float32), p.r_cut + p.skin).tolist()}
+    assert got == ref and len(ref) > 10 * s.n_atoms
