@@ -15,193 +15,274 @@
 // fixed-point accumulation), and a per-atom combination.
 #include <cstring>
 #include <string>
-#include <vector>
 
 #include "vp_adjoint.cuh"
-#include "vp_cvpair.cuh"
+#include "vp_cv_dev.cuh"
 
 namespace vp {
 
 struct AdjDev {
-  const float *frames;  // [nf][3 n_cv]
+  float *frames;        // [nf][3 n_cv]
   int nf, n_cv, min_sep, n_tiles;
   const int2 *tiles;    // the system's tiles
-  const double *cnat;   // the system's C~_nat in tile-skew order
-  const double *gm;     // gamma_i m_i of the system's atoms
+  const float2 *cnat;   // the system's C~_nat in tile-skew order (float-float)
+  const double *inv_gm; // 1 / (gamma_i m_i) of the system's atoms
   float L, iL;
   double zconst;
   long long *gx, *gy, *gz;  // [nf][n_cv]
-  long long *hx, *hy, *hz;  // [nf][n_cv]
+  long long *hx, *hy, *hz;  // [nf][n_cv], after g
   float *w;                 // [nf][3 n_cv]
   double *zpart;            // [nf][n_tiles]
   double *z, *Q;            // [nf]
   double *coef;             // [2 nf]: A_n, B_n
+  double *phi;              // [1]
 };
 
-__global__ void __launch_bounds__(128) k_adj_cv(AdjDev a, CvConst k) {
-  const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (w >= a.nf * a.n_tiles) return;
-  const int f = w / a.n_tiles, t = w - f * a.n_tiles;
+struct AdjFramePos {
+  const float *X;
+  __device__ __forceinline__ float3 operator()(int a) const { return make_float3(X[3 * a], X[3 * a + 1], X[3 * a + 2]); }
+};
+
+__device__ __forceinline__ CvTile adj_tile(const AdjDev &a, const CvConst &k, int f, int t) {
   const int2 bij = a.tiles[t];
-  const float *X = a.frames + (size_t)f * 3 * a.n_cv;
-  const int i = bij.x * CV_T + lane, jl = bij.y * CV_T + lane;
-  float3 xi = make_float3(0.f, 0.f, 0.f), xj = make_float3(0.f, 0.f, 0.f);
-  if (i < a.n_cv) xi = make_float3(X[3 * i], X[3 * i + 1], X[3 * i + 2]);
-  if (jl < a.n_cv) xj = make_float3(X[3 * jl], X[3 * jl + 1], X[3 * jl + 2]);
-  const double *cn = a.cnat + (size_t)t * CV_T * CV_T;
-  long long gix = 0, giy = 0, giz = 0, gjx = 0, gjy = 0, gjz = 0;
-  ff zacc = {0.f, 0.f};
-  for (int s = 0; s < CV_T; ++s) {
-    const int jc = (lane + s) & (CV_T - 1);
-    const int j = bij.y * CV_T + jc;
-    const float xjx = __shfl_sync(0xffffffffu, xj.x, jc);
-    const float xjy = __shfl_sync(0xffffffffu, xj.y, jc);
-    const float xjz = __shfl_sync(0xffffffffu, xj.z, jc);
-    if (i < a.n_cv && j < a.n_cv && j - i > a.min_sep) {
-      ff dx, dy, dz;
-      cv_delta(xi, xjx, xjy, xjz, a.L, a.iL, dx, dy, dz);
-      const float r2f = dx.hi * dx.hi + dy.hi * dy.hi + dz.hi * dz.hi;
-      if (r2f < k.rc2_far) {
-        const ff cnat = ff_from_d(cn[s * CV_T + lane]);
-        const ff r2 = ff_add(ff_add(ff_sqr(dx), ff_sqr(dy)), ff_sqr(dz));
-        const CvPair cp = cv_contact<false>(r2, k);
-        const ff h = ff_add(cp.Ct, ff_neg(cnat));
-        zacc = ff_add(zacc, ff_mul(cp.Ct, ff_add(cp.Ct, ff_neg(ff_mul_f(cnat, 2.0f)))));
-        const float wgt = 2.0f * h.hi * cp.dCt / cp.r;
-        const long long gx = fx_from(wgt * dx.hi), gy = fx_from(wgt * dy.hi), gz = fx_from(wgt * dz.hi);
-        gix -= gx; giy -= gy; giz -= gz;
-        gjx += gx; gjy += gy; gjz += gz;
-      }
-    }
-    const int src = (lane + 1) & 31;
-    gjx = __shfl_sync(0xffffffffu, gjx, src);
-    gjy = __shfl_sync(0xffffffffu, gjy, src);
-    gjz = __shfl_sync(0xffffffffu, gjz, src);
-  }
   const size_t base = (size_t)f * a.n_cv;
-  if (i < a.n_cv && (gix | giy | giz)) { red_add(a.gx + base + i, gix); red_add(a.gy + base + i, giy); red_add(a.gz + base + i, giz); }
-  if (jl < a.n_cv && (gjx | gjy | gjz)) { red_add(a.gx + base + jl, gjx); red_add(a.gy + base + jl, gjy); red_add(a.gz + base + jl, gjz); }
-  double zl = ff_to_d(zacc);
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) zl += __shfl_xor_sync(0xffffffffu, zl, off);
-  if (lane == 0) a.zpart[(size_t)f * a.n_tiles + t] = zl;
+  return CvTile{a.n_cv, bij.x, bij.y, a.min_sep, a.L, a.iL, k.rc2_far, a.cnat + (size_t)t * CV_T * CV_T,
+                a.gx + base, a.gy + base, a.gz + base, a.zpart + (size_t)f * a.n_tiles + t};
 }
 
-// per frame: z, Q and w = g/(gamma m)
-__global__ void __launch_bounds__(256) k_adj_fin(AdjDev a) {
-  __shared__ double rz[256], rq[256];
+// z partial sums and gradients, a warp (NW = 1) or a block of NW warps per
+// (frame, tile): the tile routines of the batched kernel, which evaluate the
+// near pairs densely and leave a tile of far blocks at once.  One lane per i
+// and a loop over j, near or far, took 625 us for 51 frames of 1800 atoms.
+template <int NW>
+__global__ void __launch_bounds__(128) k_adj_cv(AdjDev a, CvConst k) {
+  if constexpr (NW == 1) {
+    __shared__ CvWarpShared sh[4];
+    const int w = blockIdx.x * 4 + (threadIdx.x >> 5);
+    if (w >= a.nf * a.n_tiles) return;
+    const int f = w / a.n_tiles, t = w - f * a.n_tiles;
+    cv_tile(adj_tile(a, k, f, t), k, sh[threadIdx.x >> 5], AdjFramePos{a.frames + (size_t)f * 3 * a.n_cv});
+  } else {
+    __shared__ CvBlockShared sh;
+    const int f = blockIdx.x / a.n_tiles, t = blockIdx.x - f * a.n_tiles;
+    cv_tile_block<NW>(adj_tile(a, k, f, t), k, sh, AdjFramePos{a.frames + (size_t)f * 3 * a.n_cv});
+  }
+}
+
+// per frame: z, Q and w = g/(gamma m) (a stored 1/(gamma m): FP64 division is
+// slow on this part)
+constexpr int FIN_THREADS = 512;
+__global__ void __launch_bounds__(FIN_THREADS) k_adj_fin(AdjDev a) {
+  __shared__ double rz[FIN_THREADS / 32], rq[FIN_THREADS / 32];
   const int f = blockIdx.x;
   double zs = 0.0, q = 0.0;
-  for (int t = threadIdx.x; t < a.n_tiles; t += blockDim.x) zs += a.zpart[(size_t)f * a.n_tiles + t];
+  for (int t = threadIdx.x; t < a.n_tiles; t += FIN_THREADS) zs += a.zpart[(size_t)f * a.n_tiles + t];
   const double sc = 2.3283064365386963e-10;
-  for (int i = threadIdx.x; i < a.n_cv; i += blockDim.x) {
+  for (int i = threadIdx.x; i < a.n_cv; i += FIN_THREADS) {
     const size_t k = (size_t)f * a.n_cv + i;
     const double gx = (double)a.gx[k] * sc, gy = (double)a.gy[k] * sc, gz = (double)a.gz[k] * sc;
-    const double gm = a.gm[i];
-    q += (gx * gx + gy * gy + gz * gz) / gm;
-    a.w[3 * k] = (float)(gx / gm);
-    a.w[3 * k + 1] = (float)(gy / gm);
-    a.w[3 * k + 2] = (float)(gz / gm);
+    const double ig = a.inv_gm[i];
+    q += (gx * gx + gy * gy + gz * gz) * ig;
+    a.w[3 * k] = (float)(gx * ig);
+    a.w[3 * k + 1] = (float)(gy * ig);
+    a.w[3 * k + 2] = (float)(gz * ig);
   }
-  rz[threadIdx.x] = zs;
-  rq[threadIdx.x] = q;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    zs += __shfl_xor_sync(0xffffffffu, zs, off);
+    q += __shfl_xor_sync(0xffffffffu, q, off);
+  }
+  if ((threadIdx.x & 31) == 0) { rz[threadIdx.x >> 5] = zs; rq[threadIdx.x >> 5] = q; }
   __syncthreads();
-  for (int off = blockDim.x / 2; off > 0; off >>= 1) {
-    if (threadIdx.x < off) { rz[threadIdx.x] += rz[threadIdx.x + off]; rq[threadIdx.x] += rq[threadIdx.x + off]; }
-    __syncthreads();
-  }
   if (threadIdx.x == 0) {
-    a.z[f] = a.zconst + rz[0];
-    a.Q[f] = rq[0];
+    for (int k = 1; k < FIN_THREADS / 32; ++k) { zs += rz[k]; q += rq[k]; }
+    a.z[f] = a.zconst + zs;
+    a.Q[f] = q;
   }
 }
 
-// coefficients A_n, B_n and Phi from z and Q along the path (z_m starts at z_0)
-__global__ void k_adj_scan(const double *z, const double *Q, int nf, double c, double *coef, double *route,
-                           double *phi_out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  for (int f = 0; f < nf; ++f) route[f] = 0.0;
-  double m = z[0], Phi = 0.0;
-  int arg = 0;
-  for (int f = 1; f < nf; ++f) {
-    const double a = z[f] > m ? z[f] - m : 0.0;
-    Phi += c * a * a * Q[f];
-    if (a > 0.0) route[arg] += 2.0 * a * Q[f];
-    coef[2 * f + 1] = 2.0 * c * a * a;
-    coef[2 * f] = 2.0 * c * a * Q[f];
-    if (z[f] < m) { m = z[f]; arg = f; }
+// Coefficients A_n, B_n and Phi from z and Q along the path (z_m starts at
+// z_0), one block.  Per SCAN frames: one warp forms the running minimum before
+// each frame (a scan of 32 at a time) and a = (z - z_m)_+; all threads write
+// the coefficients; then one thread sums Phi and another what the frames pass
+// on to the frame their running minimum sits at (those frames are
+// consecutive, so one running sum, put down when the minimum moves), both in
+// frame order.  The two sums are chains of one dependent operation per frame
+// on shared memory; one thread doing everything from global memory took 294
+// us for 501 frames.
+constexpr int SCAN = 1024;
+__global__ void __launch_bounds__(256) k_adj_scan(const double *z, const double *Q, int nf, double c, double *coef,
+                                                  double *phi_out) {
+  __shared__ double s_z[SCAN], s_q[SCAN], s_a[SCAN];
+  __shared__ bool s_new[SCAN];
+  __shared__ double s_m;
+  const double z0 = z[0];
+  // a path that starts at NaN never compares below or above its minimum
+  const bool dead = isnan(z0);
+  double Phi = 0.0, R = 0.0;  // thread 32, thread 64
+  int arg = 0;                // thread 64
+  if (threadIdx.x == 0) {
+    s_m = z0;
+    coef[0] = 0.0;
+    coef[1] = 0.0;
   }
-  coef[0] = 0.0;
-  coef[1] = 0.0;
-  for (int f = 0; f < nf; ++f) coef[2 * f] -= c * route[f];
-  if (phi_out) *phi_out = Phi;
-}
-
-// H_z w per frame: a pair adds K (w_j - w_i) to atom j and subtracts it from
-// atom i, K v = f'' u (u.v) + (f'/r)(v - u (u.v)), f = (C~ - C~_nat)^2
-__global__ void __launch_bounds__(128) k_adj_hw(AdjDev a, CvConst k) {
-  const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (w >= a.nf * a.n_tiles) return;
-  const int f = w / a.n_tiles, t = w - f * a.n_tiles;
-  if (a.coef[2 * f + 1] == 0.0) return;  // no bias at this frame: no Hessian term
-  const int2 bij = a.tiles[t];
-  const float *X = a.frames + (size_t)f * 3 * a.n_cv;
-  const float *W = a.w + (size_t)f * 3 * a.n_cv;
-  const int i = bij.x * CV_T + lane, jl = bij.y * CV_T + lane;
-  float3 xi = make_float3(0.f, 0.f, 0.f), xj = make_float3(0.f, 0.f, 0.f);
-  float3 wi = make_float3(0.f, 0.f, 0.f), wj = make_float3(0.f, 0.f, 0.f);
-  if (i < a.n_cv) {
-    xi = make_float3(X[3 * i], X[3 * i + 1], X[3 * i + 2]);
-    wi = make_float3(W[3 * i], W[3 * i + 1], W[3 * i + 2]);
-  }
-  if (jl < a.n_cv) {
-    xj = make_float3(X[3 * jl], X[3 * jl + 1], X[3 * jl + 2]);
-    wj = make_float3(W[3 * jl], W[3 * jl + 1], W[3 * jl + 2]);
-  }
-  const double *cn = a.cnat + (size_t)t * CV_T * CV_T;
-  long long hix = 0, hiy = 0, hiz = 0, hjx = 0, hjy = 0, hjz = 0;
-  for (int s = 0; s < CV_T; ++s) {
-    const int jc = (lane + s) & (CV_T - 1);
-    const int j = bij.y * CV_T + jc;
-    const float xjx = __shfl_sync(0xffffffffu, xj.x, jc);
-    const float xjy = __shfl_sync(0xffffffffu, xj.y, jc);
-    const float xjz = __shfl_sync(0xffffffffu, xj.z, jc);
-    const float wjx = __shfl_sync(0xffffffffu, wj.x, jc);
-    const float wjy = __shfl_sync(0xffffffffu, wj.y, jc);
-    const float wjz = __shfl_sync(0xffffffffu, wj.z, jc);
-    if (i < a.n_cv && j < a.n_cv && j - i > a.min_sep) {
-      ff dx, dy, dz;
-      cv_delta(xi, xjx, xjy, xjz, a.L, a.iL, dx, dy, dz);
-      const float r2f = dx.hi * dx.hi + dy.hi * dy.hi + dz.hi * dz.hi;
-      if (r2f < k.rc2_far) {
-        const ff r2 = ff_add(ff_add(ff_sqr(dx), ff_sqr(dy)), ff_sqr(dz));
-        const CvPair cp = cv_contact<true>(r2, k);
-        const float h = ff_add(cp.Ct, ff_neg(ff_from_d(cn[s * CV_T + lane]))).hi;
-        const float f1 = 2.0f * h * cp.dCt;
-        const float f2 = 2.0f * (cp.dCt * cp.dCt + h * cp.d2Ct);
-        const float ir = 1.0f / cp.r;
-        const float ux = dx.hi * ir, uy = dy.hi * ir, uz = dz.hi * ir;
-        const float vx = wjx - wi.x, vy = wjy - wi.y, vz = wjz - wi.z;
-        const float uv = ux * vx + uy * vy + uz * vz;
-        const float q = f1 * ir;
-        const float kx = f2 * ux * uv + q * (vx - ux * uv);
-        const float ky = f2 * uy * uv + q * (vy - uy * uv);
-        const float kz = f2 * uz * uv + q * (vz - uz * uv);
-        const long long ex = fx_from(kx), ey = fx_from(ky), ez = fx_from(kz);
-        hix -= ex; hiy -= ey; hiz -= ez;
-        hjx += ex; hjy += ey; hjz += ez;
+  __syncthreads();
+  for (int f0 = 1; f0 < nf; f0 += SCAN) {
+    const int n = min(SCAN, nf - f0);
+    for (int k = threadIdx.x; k < n; k += blockDim.x) {
+      s_z[k] = z[f0 + k];
+      s_q[k] = Q[f0 + k];
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      double m = s_m;
+      for (int b = 0; b < n; b += 32) {
+        const int k = b + (int)threadIdx.x;
+        const double v = k < n && !isnan(s_z[k]) ? s_z[k] : INFINITY;
+        double incl = v;  // least of this and the earlier lanes' values
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+          const double o = __shfl_up_sync(0xffffffffu, incl, off);
+          if ((int)threadIdx.x >= off && o < incl) incl = o;
+        }
+        double before = __shfl_up_sync(0xffffffffu, incl, 1);
+        before = threadIdx.x == 0 || m < before ? m : before;  // z_m before frame k
+        if (k < n) {
+          s_a[k] = !dead && s_z[k] > before ? s_z[k] - before : 0.0;
+          s_new[k] = !dead && s_z[k] < before;
+        }
+        const double last = __shfl_sync(0xffffffffu, incl, 31);
+        if (last < m) m = last;
+      }
+      if (threadIdx.x == 0) s_m = m;
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < n; k += blockDim.x) {
+      const double a = s_a[k];
+      coef[2 * (f0 + k) + 1] = 2.0 * c * a * a;
+      coef[2 * (f0 + k)] = 2.0 * c * a * s_q[k];
+    }
+    __syncthreads();
+    if (threadIdx.x == 32) {
+      for (int k = 0; k < n; ++k) Phi = fma(c * s_a[k] * s_a[k], s_q[k], Phi);
+    } else if (threadIdx.x == 64) {
+      for (int k = 0; k < n; ++k) {
+        if (s_a[k] > 0.0) R = fma(2.0 * s_a[k], s_q[k], R);
+        if (s_new[k]) {
+          coef[2 * arg] = fma(-c, R, coef[2 * arg]);
+          arg = f0 + k;
+          R = 0.0;
+        }
       }
     }
-    const int src = (lane + 1) & 31;
-    hjx = __shfl_sync(0xffffffffu, hjx, src);
-    hjy = __shfl_sync(0xffffffffu, hjy, src);
-    hjz = __shfl_sync(0xffffffffu, hjz, src);
+    __syncthreads();  // the shared arrays are taken anew
   }
+  if (threadIdx.x == 64) coef[2 * arg] = fma(-c, R, coef[2 * arg]);
+  if (threadIdx.x == 32 && phi_out) *phi_out = Phi;
+}
+
+// shared memory of a tile of H_z w
+struct AdjHwShared {
+  unsigned short s_near[CV_T * CV_T];
+  float s_x[2 * CV_T][3], s_w[2 * CV_T][3];
+  int s_ghi[2 * CV_T][3];
+  unsigned s_glo[2 * CV_T][3];
+};
+
+// One near pair of H_z w: it adds K (w_j - w_i) to atom j and subtracts it
+// from atom i, K v = f'' u (u.v) + (f'/r)(v - u (u.v)), f = (C~ - C~_nat)^2.
+// The sums are 64-bit fixed point, kept per tile as two 32-bit parts (see
+// CvWarpShared); a contribution too large for those goes straight to memory
+// (the sum is the same).
+__device__ __forceinline__ void adj_hw_pair(AdjHwShared &sh, const CvTile &t, const CvConst &k, unsigned e) {
+  const int il = e & 31, jc = e >> 5;
+  const float3 xi = make_float3(sh.s_x[il][0], sh.s_x[il][1], sh.s_x[il][2]);
+  ff dx, dy, dz;
+  cv_delta(xi, sh.s_x[CV_T + jc][0], sh.s_x[CV_T + jc][1], sh.s_x[CV_T + jc][2], t.L, t.iL, dx, dy, dz);
+  const float2 cv2 = t.cn[((jc - il) & (CV_T - 1)) * CV_T + il];
+  const ff r2 = ff_add(ff_add(ff_sqr(dx), ff_sqr(dy)), ff_sqr(dz));
+  const CvPair cp = cv_contact<true>(r2, k);
+  const float h = ff_add(cp.Ct, ff{-cv2.x, -cv2.y}).hi;
+  const float f1 = 2.0f * h * cp.dCt;
+  const float f2 = 2.0f * (cp.dCt * cp.dCt + h * cp.d2Ct);
+  const float ir = 1.0f / cp.r;
+  const float ux = dx.hi * ir, uy = dy.hi * ir, uz = dz.hi * ir;
+  const float vx = sh.s_w[CV_T + jc][0] - sh.s_w[il][0], vy = sh.s_w[CV_T + jc][1] - sh.s_w[il][1],
+              vz = sh.s_w[CV_T + jc][2] - sh.s_w[il][2];
+  const float uv = ux * vx + uy * vy + uz * vz;
+  const float q = f1 * ir;
+  const float kx = f2 * ux * uv + q * (vx - ux * uv);
+  const float ky = f2 * uy * uv + q * (vy - uy * uv);
+  const float kz = f2 * uz * uv + q * (vz - uz * uv);
+  const long long ev[3] = {fx_from(kx), fx_from(ky), fx_from(kz)};
+  long long *const gp[3] = {t.gx, t.gy, t.gz};
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const long long v = ev[c];
+    if (v == 0) continue;
+    if (v < (1ll << 49) && v > -(1ll << 49)) {
+      atomicAdd(&sh.s_ghi[il][c], (int)((-v) >> 24));
+      atomicAdd(&sh.s_glo[il][c], (unsigned)((-v) & 0xffffff));
+      atomicAdd(&sh.s_ghi[CV_T + jc][c], (int)(v >> 24));
+      atomicAdd(&sh.s_glo[CV_T + jc][c], (unsigned)(v & 0xffffff));
+    } else {
+      red_add(gp[c] + t.bi * CV_T + il, (long long)(0ull - (unsigned long long)v));
+      red_add(gp[c] + t.bj * CV_T + jc, v);
+    }
+  }
+}
+
+// H_z w per frame with a bias, a warp (NW = 1) or a block of NW warps per (frame, tile)
+template <int NW>
+__global__ void __launch_bounds__(128) k_adj_hw(AdjDev a, CvConst k) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __shared__ AdjHwShared s_sh[NW == 1 ? 4 : 1];
+  __shared__ unsigned s_bal[CV_T];
+  const int w = NW == 1 ? blockIdx.x * 4 + warp : blockIdx.x;
+  if (w >= a.nf * a.n_tiles) return;
+  const int f = w / a.n_tiles;
+  if (a.coef[2 * f + 1] == 0.0) return;  // no bias at this frame: no Hessian term
+  CvTile t = adj_tile(a, k, f, w - f * a.n_tiles);
   const size_t base = (size_t)f * a.n_cv;
-  if (i < a.n_cv && (hix | hiy | hiz)) { red_add(a.hx + base + i, hix); red_add(a.hy + base + i, hiy); red_add(a.hz + base + i, hiz); }
-  if (jl < a.n_cv && (hjx | hjy | hjz)) { red_add(a.hx + base + jl, hjx); red_add(a.hy + base + jl, hjy); red_add(a.hz + base + jl, hjz); }
+  t.gx = a.hx + base; t.gy = a.hy + base; t.gz = a.hz + base;
+  const AdjFramePos pos{a.frames + 3 * base}, wof{a.w + 3 * base};
+  AdjHwShared &sh = s_sh[NW == 1 ? warp : 0];
+  int n_near;
+  if constexpr (NW == 1) {
+    const int i = t.bi * CV_T + lane, j = t.bj * CV_T + lane;
+    const bool iv = i < t.n_cv, jv = j < t.n_cv;
+    float3 xi = make_float3(0.f, 0.f, 0.f), xj = xi, wi = xi, wj = xi;
+    if (iv) { xi = pos(i); wi = wof(i); }
+    if (jv) { xj = pos(j); wj = wof(j); }
+    if (cv_tile_far(t, iv, jv, xi, xj)) return;
+    n_near = cv_near_list(t, sh.s_near, xi, xj);
+    if (n_near == 0) return;
+    const float x6[6] = {xi.x, xi.y, xi.z, xj.x, xj.y, xj.z}, w6[6] = {wi.x, wi.y, wi.z, wj.x, wj.y, wj.z};
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+      const int row = lane + (q >= 3 ? CV_T : 0), c = q % 3;
+      sh.s_x[row][c] = x6[q];
+      sh.s_w[row][c] = w6[q];
+      sh.s_ghi[row][c] = 0;
+      sh.s_glo[row][c] = 0u;
+    }
+    __syncwarp();
+  } else {
+    const bool far = cv_block_begin<NW>(t, sh, pos);
+    if (far) return;
+    if (threadIdx.x < 2 * CV_T) {
+      const int q = (warp == 0 ? t.bi : t.bj) * CV_T + lane;
+      const float3 v = q < t.n_cv ? wof(q) : make_float3(0.f, 0.f, 0.f);
+      sh.s_w[threadIdx.x][0] = v.x; sh.s_w[threadIdx.x][1] = v.y; sh.s_w[threadIdx.x][2] = v.z;
+    }
+    n_near = cv_near_list_block<NW>(t, sh.s_near, s_bal, sh.s_x);
+  }
+  for (int p = NW == 1 ? lane : (int)threadIdx.x; p < n_near; p += NW * 32) adj_hw_pair(sh, t, k, sh.s_near[p]);
+  if constexpr (NW == 1) __syncwarp(); else __syncthreads();
+  for (int q = NW == 1 ? lane : (int)threadIdx.x; q < 2 * CV_T; q += NW * 32) {
+    const int atom = (q < CV_T ? t.bi : t.bj) * CV_T + (q & (CV_T - 1));
+    if (atom < t.n_cv) cv_flush_atom(sh, q, t.gx + atom, t.gy + atom, t.gz + atom);
+  }
 }
 
 __global__ void k_adj_out(AdjDev a, double *grad) {
@@ -214,80 +295,24 @@ __global__ void k_adj_out(AdjDev a, double *grad) {
   grad[3 * k + 2] = A * (double)a.gz[k] * sc + B * (double)a.hz[k] * sc;
 }
 
-// ---------------------------------------------------------------------------
-
-int adjoint_frames(const AdjInput &in, cudaStream_t st, std::string &err) {
-  const int nf = in.n_frames, ncv = in.n_cv, nt = in.n_tiles;
-  const size_t na = (size_t)nf * ncv;
-  AdjDev a{};
-  a.nf = nf; a.n_cv = ncv; a.min_sep = in.min_sep; a.n_tiles = nt;
-  a.tiles = in.tiles; a.cnat = in.cnat; a.gm = in.gm; a.L = in.L; a.iL = in.iL; a.zconst = in.zconst;
-  std::vector<void *> bufs;
-  auto alloc = [&](size_t bytes) -> void * {
-    void *p = nullptr;
-    if (cudaMalloc(&p, bytes ? bytes : 8) != cudaSuccess) return nullptr;
-    bufs.push_back(p);
-    return p;
-  };
-  auto freeall = [&]() { for (void *p : bufs) cudaFree(p); };
-  float *dframes = (float *)alloc(sizeof(float) * 3 * na);
-  a.gx = (long long *)alloc(sizeof(long long) * 3 * na);
-  a.hx = (long long *)alloc(sizeof(long long) * 3 * na);
-  a.w = (float *)alloc(sizeof(float) * 3 * na);
-  a.zpart = (double *)alloc(sizeof(double) * (size_t)nf * (nt > 0 ? nt : 1));
-  a.z = (double *)alloc(sizeof(double) * nf);
-  a.Q = (double *)alloc(sizeof(double) * nf);
-  a.coef = (double *)alloc(sizeof(double) * 2 * nf);
-  double *route = (double *)alloc(sizeof(double) * nf);
-  double *dphi = (double *)alloc(sizeof(double));
-  double *dgrad = (double *)alloc(sizeof(double) * 3 * na);
-  for (void *p : bufs)
-    if (!p) { freeall(); err = "cudaMalloc failed"; return SIM_ECUDA; }
-  a.frames = dframes;
-  a.gy = a.gx + na; a.gz = a.gy + na;
-  a.hy = a.hx + na; a.hz = a.hy + na;
-  std::vector<float> hf(3 * na);
-  for (size_t k = 0; k < 3 * na; ++k) hf[k] = (float)in.frames[k];
-  cudaMemcpyAsync(dframes, hf.data(), sizeof(float) * 3 * na, cudaMemcpyHostToDevice, st);
-  cudaMemsetAsync(a.gx, 0, sizeof(long long) * 3 * na, st);
-  cudaMemsetAsync(a.hx, 0, sizeof(long long) * 3 * na, st);
-  const long long warps = (long long)nf * nt;
-  if (warps > 0) k_adj_cv<<<(unsigned)((warps * 32 + 127) / 128), 128, 0, st>>>(a, in.k);
-  k_adj_fin<<<nf, 256, 0, st>>>(a);
-  if (in.coef) {
-    cudaMemcpyAsync(a.coef, in.coef, sizeof(double) * 2 * nf, cudaMemcpyHostToDevice, st);
-  } else {
-    k_adj_scan<<<1, 32, 0, st>>>(a.z, a.Q, nf, in.c, a.coef, route, dphi);
-  }
-  if (warps > 0) k_adj_hw<<<(unsigned)((warps * 32 + 127) / 128), 128, 0, st>>>(a, in.k);
-  if (na > 0) k_adj_out<<<(unsigned)((na + 255) / 256), 256, 0, st>>>(a, dgrad);
-  cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess && in.grad) e = cudaMemcpyAsync(in.grad, dgrad, sizeof(double) * 3 * na, cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess && in.z_out) e = cudaMemcpyAsync(in.z_out, a.z, sizeof(double) * nf, cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess && in.Q_out) e = cudaMemcpyAsync(in.Q_out, a.Q, sizeof(double) * nf, cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess && in.phi && !in.coef) e = cudaMemcpyAsync(in.phi, dphi, sizeof(double), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  freeall();
-  if (e != cudaSuccess) { err = cudaGetErrorString(e); return SIM_ECUDA; }
-  return SIM_OK;
-}
-
-// ---------------------------------------------------------------------------
-// refinement of a path by descent on the functional (frames as variables)
-// ---------------------------------------------------------------------------
-__global__ void k_to_f32(const double *x, float *y, size_t n) {
+// frames in FP32, the precision the functional is evaluated at; the gradient sums cleared
+__global__ void k_adj_begin(AdjDev a, const double *x, size_t n) {
   const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < n) y[k] = (float)x[k];
+  if (k >= n) return;
+  a.frames[k] = (float)x[k];
+  a.gx[k] = 0;  // gx, gy, gz lie one after another: n = 3 nf n_cv entries
 }
 
-// y = x - eta g on frames 1 .. nf-2, rounded to FP32 (the precision the
-// functional is evaluated at, so that the returned path is exactly the one
-// scored); y = x on the end frames, which stay put
-__global__ void k_descend(const double *x, const double *g, double eta, double *y, size_t per_frame, int nf) {
+// y = x - eta g on frames 1 .. nf-2, rounded to FP32 (so that the returned
+// path is exactly the one scored); y = x on the end frames, which stay put
+__global__ void k_descend(AdjDev a, const double *x, const double *g, double eta, double *y, size_t per_frame, int nf) {
   const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= per_frame * (size_t)nf) return;
   const int f = (int)(k / per_frame);
-  y[k] = (f == 0 || f == nf - 1) ? x[k] : (double)(float)(x[k] - eta * g[k]);
+  const double v = (f == 0 || f == nf - 1) ? x[k] : (double)(float)(x[k] - eta * g[k]);
+  y[k] = v;
+  a.frames[k] = (float)v;
+  a.gx[k] = 0;
 }
 
 // |g|^2 over frames 1 .. nf-2: fixed-order block sums, then one block
@@ -306,72 +331,160 @@ __global__ void k_sq_interior(const double *g, size_t per_frame, int nf, double 
   if (threadIdx.x == 0) part[blockIdx.x] = red[0];
 }
 
-int refine_frames(const AdjInput &in, double *frames, int n_iter, double step, double *phi_hist, int *n_accepted,
-                  cudaStream_t st, std::string &err) {
-  const int nf = in.n_frames, ncv = in.n_cv, nt = in.n_tiles;
-  const size_t na = (size_t)nf * ncv, nx = 3 * na;
-  AdjDev a{};
-  a.nf = nf; a.n_cv = ncv; a.min_sep = in.min_sep; a.n_tiles = nt;
-  a.tiles = in.tiles; a.cnat = in.cnat; a.gm = in.gm; a.L = in.L; a.iL = in.iL; a.zconst = in.zconst;
-  std::vector<void *> bufs;
-  auto alloc = [&](size_t bytes) -> void * {
-    void *p = nullptr;
-    if (cudaMalloc(&p, bytes ? bytes : 8) != cudaSuccess) return nullptr;
-    bufs.push_back(p);
-    return p;
-  };
-  auto freeall = [&]() { for (void *p : bufs) cudaFree(p); };
-  constexpr int SQ_BLOCKS = 64;
-  float *f32 = (float *)alloc(sizeof(float) * nx);
-  double *X = (double *)alloc(sizeof(double) * nx), *Y = (double *)alloc(sizeof(double) * nx);
-  double *G = (double *)alloc(sizeof(double) * nx);
-  a.gx = (long long *)alloc(sizeof(long long) * 3 * na);
-  a.hx = (long long *)alloc(sizeof(long long) * 3 * na);
-  a.w = (float *)alloc(sizeof(float) * nx);
-  a.zpart = (double *)alloc(sizeof(double) * (size_t)nf * (nt > 0 ? nt : 1));
-  a.z = (double *)alloc(sizeof(double) * nf);
-  a.Q = (double *)alloc(sizeof(double) * nf);
-  a.coef = (double *)alloc(sizeof(double) * 2 * nf);
-  double *route = (double *)alloc(sizeof(double) * nf);
-  double *dphi = (double *)alloc(sizeof(double));
-  double *part = (double *)alloc(sizeof(double) * SQ_BLOCKS);
-  for (void *p : bufs)
-    if (!p) { freeall(); err = "cudaMalloc failed"; return SIM_ECUDA; }
-  a.frames = f32;
-  a.gy = a.gx + na; a.gz = a.gy + na;
-  a.hy = a.hx + na; a.hz = a.hy + na;
-  const long long warps = (long long)nf * nt;
-  const unsigned gx_blocks = (unsigned)((nx + 255) / 256);
-  // Phi (and, when want_grad, dPhi/dX into G) at the frames in src
-  auto eval = [&](const double *src, bool want_grad, double &phi) -> cudaError_t {
-    k_to_f32<<<gx_blocks, 256, 0, st>>>(src, f32, nx);
-    cudaMemsetAsync(a.gx, 0, sizeof(long long) * 3 * na, st);
-    cudaMemsetAsync(a.hx, 0, sizeof(long long) * 3 * na, st);
-    if (warps > 0) k_adj_cv<<<(unsigned)((warps * 32 + 127) / 128), 128, 0, st>>>(a, in.k);
-    k_adj_fin<<<nf, 256, 0, st>>>(a);
-    k_adj_scan<<<1, 32, 0, st>>>(a.z, a.Q, nf, in.c, a.coef, route, dphi);
-    if (want_grad) {
-      if (warps > 0) k_adj_hw<<<(unsigned)((warps * 32 + 127) / 128), 128, 0, st>>>(a, in.k);
-      if (na > 0) k_adj_out<<<(unsigned)((na + 255) / 256), 256, 0, st>>>(a, G);
+// ---------------------------------------------------------------------------
+
+void AdjWorkspace::release() {
+  if (p) cudaFree(p);
+  p = nullptr;
+  n = 0;
+}
+
+void *AdjWorkspace::reserve(size_t bytes) {
+  if (bytes > n) {
+    release();
+    if (cudaMalloc(&p, bytes) != cudaSuccess) {
+      p = nullptr;
+      return nullptr;
     }
+    n = bytes;
+  }
+  return p;
+}
+
+namespace {
+
+// carves the arrays of one call out of the workspace, 256 bytes apart
+struct Carve {
+  char *base;
+  size_t off = 0;
+  template <class T>
+  T *take(size_t n) {
+    T *r = reinterpret_cast<T *>(base + off);
+    off += ((n ? n : 1) * sizeof(T) + 255) & ~(size_t)255;
+    return r;
+  }
+};
+
+// the arrays every evaluation needs (with base = nullptr only their size counts)
+AdjDev adj_arrays(const AdjInput &in, Carve &c) {
+  const size_t na = (size_t)in.n_frames * in.n_cv;
+  AdjDev a{};
+  a.nf = in.n_frames; a.n_cv = in.n_cv; a.min_sep = in.min_sep; a.n_tiles = in.n_tiles;
+  a.tiles = in.tiles; a.cnat = in.cnat; a.inv_gm = in.inv_gm; a.L = in.L; a.iL = in.iL; a.zconst = in.zconst;
+  a.frames = c.take<float>(3 * na);
+  a.gx = c.take<long long>(3 * na);
+  a.gy = a.gx + na; a.gz = a.gy + na;
+  a.hx = c.take<long long>(3 * na);
+  a.hy = a.hx + na; a.hz = a.hy + na;
+  a.w = c.take<float>(3 * na);
+  a.zpart = c.take<double>((size_t)in.n_frames * in.n_tiles);
+  a.z = c.take<double>(in.n_frames);
+  a.Q = c.take<double>(in.n_frames);
+  a.coef = c.take<double>(2 * (size_t)in.n_frames);
+  a.phi = c.take<double>(1);
+  return a;
+}
+
+// few tiles: a block each (see launch_cv)
+bool block_form(const AdjInput &in) { return (long long)in.n_frames * in.n_tiles <= 16ll * in.n_sm; }
+
+void launch_adj_cv(const AdjInput &in, const AdjDev &a, cudaStream_t st) {
+  const long long tiles = (long long)a.nf * a.n_tiles;
+  if (tiles > 0) {
+    if (block_form(in)) k_adj_cv<CV_BLOCK_WARPS><<<(unsigned)tiles, 32 * CV_BLOCK_WARPS, 0, st>>>(a, in.k);
+    else k_adj_cv<1><<<(unsigned)((tiles + 3) / 4), 128, 0, st>>>(a, in.k);
+  }
+  k_adj_fin<<<a.nf, FIN_THREADS, 0, st>>>(a);
+}
+
+void launch_adj_grad(const AdjInput &in, const AdjDev &a, double *grad, cudaStream_t st) {
+  const long long tiles = (long long)a.nf * a.n_tiles;
+  const size_t na = (size_t)a.nf * a.n_cv;
+  if (na == 0) return;
+  cudaMemsetAsync(a.hx, 0, sizeof(long long) * 3 * na, st);
+  if (tiles > 0) {
+    if (block_form(in)) k_adj_hw<CV_BLOCK_WARPS><<<(unsigned)tiles, 32 * CV_BLOCK_WARPS, 0, st>>>(a, in.k);
+    else k_adj_hw<1><<<(unsigned)((tiles + 3) / 4), 128, 0, st>>>(a, in.k);
+  }
+  k_adj_out<<<(unsigned)((na + 255) / 256), 256, 0, st>>>(a, grad);
+}
+
+}  // namespace
+
+int adjoint_frames(const AdjInput &in, AdjWorkspace &ws, cudaStream_t st, std::string &err) {
+  const int nf = in.n_frames;
+  const size_t nx = 3 * (size_t)nf * in.n_cv;
+  Carve size{nullptr};
+  adj_arrays(in, size);
+  size.take<double>(nx);
+  size.take<double>(nx);
+  Carve c{(char *)ws.reserve(size.off)};
+  if (!c.base) { err = "cudaMalloc failed"; return SIM_ECUDA; }
+  const AdjDev a = adj_arrays(in, c);
+  double *dx = c.take<double>(nx), *dgrad = c.take<double>(nx);
+  cudaError_t e = cudaMemcpyAsync(dx, in.frames, sizeof(double) * nx, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess && in.coef)
+    e = cudaMemcpyAsync(a.coef, in.coef, sizeof(double) * 2 * nf, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) {
+    if (nx > 0) k_adj_begin<<<(unsigned)((nx + 255) / 256), 256, 0, st>>>(a, dx, nx);
+    launch_adj_cv(in, a, st);
+    if (!in.coef) k_adj_scan<<<1, 256, 0, st>>>(a.z, a.Q, nf, in.c, a.coef, a.phi);
+    launch_adj_grad(in, a, dgrad, st);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess && in.grad) e = cudaMemcpyAsync(in.grad, dgrad, sizeof(double) * nx, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess && in.z_out) e = cudaMemcpyAsync(in.z_out, a.z, sizeof(double) * nf, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess && in.Q_out) e = cudaMemcpyAsync(in.Q_out, a.Q, sizeof(double) * nf, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess && in.phi && !in.coef) e = cudaMemcpyAsync(in.phi, a.phi, sizeof(double), cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  ws.trim();
+  if (e != cudaSuccess) { err = cudaGetErrorString(e); return SIM_ECUDA; }
+  return SIM_OK;
+}
+
+// ---------------------------------------------------------------------------
+// refinement of a path by descent on the functional (frames as variables)
+// ---------------------------------------------------------------------------
+int refine_frames(const AdjInput &in, double *frames, int n_iter, double step, double *phi_hist, int *n_accepted,
+                  AdjWorkspace &ws, cudaStream_t st, std::string &err) {
+  const int nf = in.n_frames, ncv = in.n_cv;
+  const size_t nx = 3 * (size_t)nf * ncv;
+  constexpr int SQ_BLOCKS = 64;
+  Carve size{nullptr};
+  adj_arrays(in, size);
+  for (int k = 0; k < 3; ++k) size.take<double>(nx);
+  size.take<double>(SQ_BLOCKS);
+  Carve c{(char *)ws.reserve(size.off)};
+  if (!c.base) { err = "cudaMalloc failed"; return SIM_ECUDA; }
+  const AdjDev a = adj_arrays(in, c);
+  double *X = c.take<double>(nx), *Y = c.take<double>(nx), *G = c.take<double>(nx), *part = c.take<double>(SQ_BLOCKS);
+  const unsigned gx_blocks = (unsigned)((nx + 255) / 256);
+  // Phi at the frames now in a.frames (their z and grad z stay for grad())
+  auto eval = [&](double &phi) -> cudaError_t {
+    launch_adj_cv(in, a, st);
+    k_adj_scan<<<1, 256, 0, st>>>(a.z, a.Q, nf, in.c, a.coef, a.phi);
     cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&phi, dphi, sizeof(double), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&phi, a.phi, sizeof(double), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     return e;
   };
-  auto sq = [&](double &v) -> cudaError_t {
+  // dPhi/dX into G and its square over the free frames, at the frames just evaluated
+  auto grad = [&](double &v) -> cudaError_t {
+    launch_adj_grad(in, a, G, st);
     k_sq_interior<<<SQ_BLOCKS, 256, 0, st>>>(G, 3 * (size_t)ncv, nf, part);
     double h[SQ_BLOCKS];
-    cudaError_t e = cudaMemcpyAsync(h, part, sizeof(h), cudaMemcpyDeviceToHost, st);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h, part, sizeof(h), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     v = 0.0;
-    for (int b = 0; b < SQ_BLOCKS; ++b) v += h[b];
+    for (int b = 0; e == cudaSuccess && b < SQ_BLOCKS; ++b) v += h[b];
     return e;
   };
   cudaError_t e = cudaMemcpyAsync(X, frames, sizeof(double) * nx, cudaMemcpyHostToDevice, st);
   double phi = 0.0, gg = 0.0;
-  if (e == cudaSuccess) e = eval(X, true, phi);
-  if (e == cudaSuccess) e = sq(gg);
+  if (e == cudaSuccess && nx > 0) k_adj_begin<<<gx_blocks, 256, 0, st>>>(a, X, nx);
+  if (e == cudaSuccess) e = eval(phi);
+  if (e == cudaSuccess) e = grad(gg);
   if (phi_hist) phi_hist[0] = phi;
   int accepted = 0;
   double eta = step;
@@ -379,9 +492,9 @@ int refine_frames(const AdjInput &in, double *frames, int n_iter, double step, d
     bool ok = false;
     // backtracking (Armijo): accept the first step that lowers Phi by at least 1e-4 eta |g|^2
     for (int bt = 0; bt < 40 && e == cudaSuccess && gg > 0.0; ++bt) {
-      k_descend<<<gx_blocks, 256, 0, st>>>(X, G, eta, Y, 3 * (size_t)ncv, nf);
+      k_descend<<<gx_blocks, 256, 0, st>>>(a, X, G, eta, Y, 3 * (size_t)ncv, nf);
       double phi_y = 0.0;
-      e = eval(Y, false, phi_y);
+      e = eval(phi_y);
       if (e != cudaSuccess) break;
       if (phi_y <= phi - 1e-4 * eta * gg) {
         std::swap(X, Y);
@@ -392,8 +505,9 @@ int refine_frames(const AdjInput &in, double *frames, int n_iter, double step, d
       eta *= 0.5;
     }
     if (e == cudaSuccess && ok) {
-      e = eval(X, true, phi);
-      if (e == cudaSuccess) e = sq(gg);
+      // the accepted path is the one evaluated last: its z, grad z and
+      // coefficients are in place
+      e = grad(gg);
       ++accepted;
       eta *= 2.0;
     }
@@ -405,29 +519,30 @@ int refine_frames(const AdjInput &in, double *frames, int n_iter, double step, d
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(frames, X, sizeof(double) * nx, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  freeall();
+  ws.trim();
   if (n_accepted) *n_accepted = accepted;
   if (e != cudaSuccess) { err = cudaGetErrorString(e); return SIM_ECUDA; }
   return SIM_OK;
 }
 
 int adjoint_coefficients(const double *z, const double *Q, int n, double c, double *coef, double *phi,
-                         cudaStream_t st, std::string &err) {
-  double *dz = nullptr, *dq = nullptr, *dc = nullptr, *dr = nullptr, *dp = nullptr;
-  size_t nb = sizeof(double) * (n > 0 ? n : 1);
-  if (cudaMalloc(&dz, nb) != cudaSuccess || cudaMalloc(&dq, nb) != cudaSuccess || cudaMalloc(&dc, 2 * nb) != cudaSuccess ||
-      cudaMalloc(&dr, nb) != cudaSuccess || cudaMalloc(&dp, sizeof(double)) != cudaSuccess) {
-    cudaFree(dz); cudaFree(dq); cudaFree(dc); cudaFree(dr); cudaFree(dp);
-    err = "cudaMalloc failed";
-    return SIM_ECUDA;
+                         AdjWorkspace &ws, cudaStream_t st, std::string &err) {
+  Carve size{nullptr};
+  for (int k = 0; k < 4; ++k) size.take<double>(n);
+  size.take<double>(1);
+  Carve a{(char *)ws.reserve(size.off)};
+  if (!a.base) { err = "cudaMalloc failed"; return SIM_ECUDA; }
+  double *dz = a.take<double>(n), *dq = a.take<double>(n), *dp = a.take<double>(1), *dc = a.take<double>(2 * (size_t)n);
+  cudaError_t e = cudaMemcpyAsync(dz, z, sizeof(double) * n, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(dq, Q, sizeof(double) * n, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) {
+    k_adj_scan<<<1, 256, 0, st>>>(dz, dq, n, c, dc, dp);
+    e = cudaGetLastError();
   }
-  cudaMemcpyAsync(dz, z, sizeof(double) * n, cudaMemcpyHostToDevice, st);
-  cudaMemcpyAsync(dq, Q, sizeof(double) * n, cudaMemcpyHostToDevice, st);
-  k_adj_scan<<<1, 32, 0, st>>>(dz, dq, n, c, dc, dr, dp);
-  cudaError_t e = cudaMemcpyAsync(coef, dc, sizeof(double) * 2 * n, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(coef, dc, sizeof(double) * 2 * n, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess && phi) e = cudaMemcpyAsync(phi, dp, sizeof(double), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  cudaFree(dz); cudaFree(dq); cudaFree(dc); cudaFree(dr); cudaFree(dp);
+  ws.trim();
   if (e != cudaSuccess) { err = cudaGetErrorString(e); return SIM_ECUDA; }
   return SIM_OK;
 }

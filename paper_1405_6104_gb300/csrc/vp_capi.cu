@@ -92,6 +92,8 @@ struct sim_handle {
   unsigned long long *d_count = nullptr;
   int *d_flag = nullptr;  // device flag of host-side checks done on the GPU
   int max_atoms = 0;
+  std::vector<double> zconst;  // per trial: sum of C~_nat^2 (fixed at creation)
+  AdjWorkspace adj_ws;         // device memory of the path-gradient calls
   // native structures (host copy, per system: first CV atom in native_all, CV atoms, min separation)
   std::vector<double> native_all;
   std::vector<int32_t> sys_nat0, sys_ncv, sys_minsep;
@@ -908,7 +910,6 @@ VP_API int sim_create(const sim_system *systems, int32_t n_systems, const int32_
   r |= dalloc(h, &d.gz, total_cv);
   r |= dalloc(h, &d.z_part, work.size());
   r |= upload(h, &d.asys, asys);
-  r |= upload(h, &d.gm, gm);
   {
     std::vector<double> igm(gm.size());
     for (size_t k = 0; k < gm.size(); ++k) igm[k] = std::isfinite(gm[k]) ? 1.0 / gm[k] : 0.0;
@@ -1006,6 +1007,10 @@ VP_API int sim_create(const sim_system *systems, int32_t n_systems, const int32_
                                        cudaGetErrorString(cudaGetLastError())));
   int fr = check_flags(h);
   if (fr) return bail(fr);
+  std::vector<TrialState> ts(total_trials);
+  if (cudaMemcpy(ts.data(), d.tstate, sizeof(TrialState) * ts.size(), cudaMemcpyDeviceToHost) != cudaSuccess)
+    return bail(fail(h, SIM_ECUDA, "cudaMemcpy trial states"));
+  for (const auto &S : ts) h->zconst.push_back(S.zconst);
   *out = h;
   return SIM_OK;
 }
@@ -1369,14 +1374,16 @@ AdjInput adj_input(sim_handle *h, int trial) {
   in.min_sep = h->c.cv_min_sep;
   in.n_tiles = T.n_work;
   in.tiles = h->d.tiles + T.systile0;
-  in.cnat = h->d.cnat + (size_t)T.systile0 * CV_T * CV_T;
-  in.gm = h->d.gm + T.sysatom0;
+  in.cnat = h->d.cnat_ff + (size_t)T.systile0 * CV_T * CV_T;
+  in.inv_gm = h->d.inv_gm + T.sysatom0;
+  in.n_sm = h->d.n_sm;
   in.L = T.box;
   in.iL = T.inv_box;
   const SimConst &c = h->c;
   in.k = CvConst{ff{c.cv_inv_r0sq_hi, c.cv_inv_r0sq_lo}, ff{c.cv_rs_hi, c.cv_rs_lo}, ff{c.cv_inv_w_hi, c.cv_inv_w_lo},
                  c.cv_rs2, c.cv_rc2_far};
   in.c = h->c.dt_d * h->c.kR_half_d * h->c.kR_half_d;
+  in.zconst = h->zconst[trial];
   return in;
 }
 }  // namespace
@@ -1386,19 +1393,15 @@ VP_API int phi_frames_adjoint(sim_handle *h, int32_t trial, const double *frames
   int r = enter(h);
   if (r) return r;
   if (trial < 0 || trial >= h->n_trials || n_frames < 1 || !frames) return fail(h, SIM_EINVAL, "bad arguments");
-  TrialState S;
-  CK(cudaMemcpyAsync(&S, h->d.tstate + trial, sizeof(S), cudaMemcpyDeviceToHost, h->stream));
-  CK(cudaStreamSynchronize(h->stream));
   AdjInput in = adj_input(h, trial);
   in.frames = frames;
   in.n_frames = n_frames;
-  in.zconst = S.zconst;
   in.coef = coef;
   in.phi = phi;
   in.z_out = z;
   in.grad = grad;
   std::string err;
-  r = adjoint_frames(in, h->stream, err);
+  r = adjoint_frames(in, h->adj_ws, h->stream, err);
   if (r) return fail(h, r, "phi_frames_adjoint: " + err);
   return SIM_OK;
 }
@@ -1409,15 +1412,11 @@ VP_API int phi_frames_refine(sim_handle *h, int32_t trial, double *frames, int32
   if (r) return r;
   if (trial < 0 || trial >= h->n_trials || n_frames < 2 || !frames || n_iter < 0 || !(step > 0.0))
     return fail(h, SIM_EINVAL, "bad refinement arguments");
-  TrialState S;
-  CK(cudaMemcpyAsync(&S, h->d.tstate + trial, sizeof(S), cudaMemcpyDeviceToHost, h->stream));
-  CK(cudaStreamSynchronize(h->stream));
   AdjInput in = adj_input(h, trial);
   in.n_frames = n_frames;
-  in.zconst = S.zconst;
   std::string err;
   int acc = 0;
-  r = refine_frames(in, frames, n_iter, step, phi_history, &acc, h->stream, err);
+  r = refine_frames(in, frames, n_iter, step, phi_history, &acc, h->adj_ws, h->stream, err);
   if (n_accepted) *n_accepted = acc;
   if (r) return fail(h, r, "phi_frames_refine: " + err);
   return SIM_OK;
@@ -1429,7 +1428,7 @@ VP_API int phi_adjoint_coefficients(sim_handle *h, const double *z, const double
   if (r) return r;
   if (n < 1 || !z || !Q || !coef) return fail(h, SIM_EINVAL, "bad arguments");
   std::string err;
-  r = adjoint_coefficients(z, Q, n, h->c.dt_d * h->c.kR_half_d * h->c.kR_half_d, coef, phi, h->stream, err);
+  r = adjoint_coefficients(z, Q, n, h->c.dt_d * h->c.kR_half_d * h->c.kR_half_d, coef, phi, h->adj_ws, h->stream, err);
   if (r) return fail(h, r, "phi_adjoint_coefficients: " + err);
   return SIM_OK;
 }
@@ -1977,6 +1976,7 @@ VP_API void sim_destroy(sim_handle *h) {
   if (h->d.rec) cudaFree(h->d.rec);
   if (h->frames) cudaFree(h->frames);
   if (h->dbuf) cudaFree(h->dbuf);
+  h->adj_ws.release();
   for (auto &t : h->timers)
     for (auto &pr : t.ev) { cudaEventDestroy(pr.first); cudaEventDestroy(pr.second); }
   if (h->entry_ev) cudaEventDestroy(h->entry_ev);

@@ -88,15 +88,16 @@ __global__ void __launch_bounds__(CV_WARPS * 32) k_cv(Dev d, SimConst c) {
   const int wib = threadIdx.x >> 5;
   const int wq = blockIdx.x * CV_WARPS + wib;
   if (wq >= d.total_work) return;
-  cv_tile(d, c, sh[wib], wq);
+  const CvItem W = d.cv_item[wq];
+  cv_tile(cv_item_tile(d, c, W), cv_const(c), sh[wib], CvSlotPos{d, W.atom0});
 }
 
-constexpr int CV_BLOCK_WARPS = 4;
 template <int NW>
 __global__ void __launch_bounds__(NW * 32) k_cv_block(Dev d, SimConst c) {
-  __shared__ CvBlockShared<NW> sh;
+  __shared__ CvBlockShared sh;
   PDL_WAIT();
-  cv_tile_block<NW>(d, c, sh, blockIdx.x);
+  const CvItem W = d.cv_item[blockIdx.x];
+  cv_tile_block<NW>(cv_item_tile(d, c, W), cv_const(c), sh, CvSlotPos{d, W.atom0});
 }
 
 // per trial: z, the ratchet amplitude a, z_m and Phi (Eqs. VR, VMDcondition).

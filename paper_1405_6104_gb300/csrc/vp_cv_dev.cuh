@@ -48,73 +48,144 @@ __device__ __forceinline__ bool cv_is_near(float dx, float dy, float dz, float L
   return dx * dx + dy * dy + dz * dz < rc2_far;
 }
 
-// the accumulated gradient of atom a (0..63) of the tile, into the trial's sums
+// the accumulated gradient of atom a (0..63) of the tile, into the sums at gx, gy, gz
 template <class SH>
-__device__ __forceinline__ void cv_flush_atom(const Dev &d, SH &sh, int a, int g) {
+__device__ __forceinline__ void cv_flush_atom(SH &sh, int a, long long *gx, long long *gy, long long *gz) {
   const long long a0 = gsum(sh.s_ghi[a][0], sh.s_glo[a][0]), a1 = gsum(sh.s_ghi[a][1], sh.s_glo[a][1]),
                   a2 = gsum(sh.s_ghi[a][2], sh.s_glo[a][2]);
-  if (a0 | a1 | a2) { red_add(d.gx + g, a0); red_add(d.gy + g, a1); red_add(d.gz + g, a2); }
+  if (a0 | a1 | a2) { red_add(gx, a0); red_add(gy, a1); red_add(gz, a2); }
 }
 
-// One warp's tile of the contact-pair triangle: the work item wq of the flat
-// (trial, tile) list, in the work order (costliest tiles first; the partial
-// sums of z keep their slots).
-__device__ __forceinline__ void cv_tile(const Dev &d, const SimConst &c, CvWarpShared &sh, int wq) {
-  auto &s_x = sh.s_x;
+// one tile of the contact-pair triangle of one configuration
+struct CvTile {
+  int n_cv, bi, bj, min_sep;
+  float L, iL, rc2_far;
+  const float2 *cn;         // the tile's C~_nat
+  long long *gx, *gy, *gz;  // the configuration's gradient sums (atom 0)
+  double *z_part;           // the tile's partial sum of z
+};
+
+// Whether no pair of the tile can be closer than the contact cut-off: the
+// periodic gap of the two 32-atom blocks' bounding boxes (lane l holds atom l
+// of either block).  Some 50 instructions that spare a far tile the 800 of its
+// distance tests.
+__device__ __forceinline__ bool cv_tile_far(const CvTile &t, bool iv, bool jv, float3 xi, float3 xj) {
+  float g2 = 0.f;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const float a = q == 0 ? xi.x : q == 1 ? xi.y : xi.z, b = q == 0 ? xj.x : q == 1 ? xj.y : xj.z;
+    const float al = warp_min(iv ? a : 3e38f), ah = warp_max(iv ? a : -3e38f);
+    const float bl = warp_min(jv ? b : 3e38f), bh = warp_max(jv ? b : -3e38f);
+    float dc = 0.5f * (bl + bh) - 0.5f * (al + ah);
+    dc = fabsf(dc - t.L * rintf(dc * t.iL)) - 0.5f * ((ah - al) + (bh - bl));
+    dc = fmaxf(dc, 0.f);
+    g2 += dc * dc;
+  }
+  return g2 > 1.001f * t.rc2_far;  // the margin covers every rounding
+}
+
+// The near pairs of the tile by one warp, in rotation-major order, into
+// s_near; returns their number.  Lane l holds atom l of either block.
+__device__ __forceinline__ int cv_near_list(const CvTile &t, unsigned short *s_near, float3 xi, float3 xj) {
   const int lane = threadIdx.x & 31;
-  const CvItem W = d.cv_item[wq];
-  const int ncv = W.n_cv, msep = c.cv_min_sep;
-  const float L = W.box, iL = W.inv_box;
-  const int i = W.bi * CV_T + lane;
-  const int jl = W.bj * CV_T + lane;
-  float3 xi = make_float3(0.f, 0.f, 0.f), xj = make_float3(0.f, 0.f, 0.f);
-  if (i < ncv) { float4 q = d.pos[d.slot_of[W.atom0 + i]]; xi = make_float3(q.x, q.y, q.z); }
-  if (jl < ncv) { float4 q = d.pos[d.slot_of[W.atom0 + jl]]; xj = make_float3(q.x, q.y, q.z); }
-  s_x[lane][0] = xi.x; s_x[lane][1] = xi.y; s_x[lane][2] = xi.z;
-  s_x[CV_T + lane][0] = xj.x; s_x[CV_T + lane][1] = xj.y; s_x[CV_T + lane][2] = xj.z;
+  const int i = t.bi * CV_T + lane;
+  int n_near = 0;
+  for (int k = 0; k < CV_T; ++k) {
+    const int jc = (lane + k) & (CV_T - 1);
+    const int j = t.bj * CV_T + jc;
+    const float xjx = __shfl_sync(0xffffffffu, xj.x, jc);
+    const float xjy = __shfl_sync(0xffffffffu, xj.y, jc);
+    const float xjz = __shfl_sync(0xffffffffu, xj.z, jc);
+    const bool near = i < t.n_cv && j < t.n_cv && j - i > t.min_sep &&
+                      cv_is_near(xjx - xi.x, xjy - xi.y, xjz - xi.z, t.L, t.iL, t.rc2_far);
+    const unsigned bal = __ballot_sync(0xffffffffu, near);
+    if (near) s_near[n_near + __popc(bal & ((1u << lane) - 1u))] = (unsigned short)(lane | (jc << 5));
+    n_near += __popc(bal);
+  }
+  return n_near;
+}
+
+// The same by a block of NW warps, the 32 rotations dealt out over them (the
+// atoms of both blocks in s_x; every thread of the block calls).
+template <int NW>
+__device__ __forceinline__ int cv_near_list_block(const CvTile &t, unsigned short *s_near, unsigned *s_bal,
+                                                  const float (*s_x)[3]) {
+  constexpr int KW = CV_T / NW;  // rotations per warp
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int i = t.bi * CV_T + lane;
+  const float3 xi = make_float3(s_x[lane][0], s_x[lane][1], s_x[lane][2]);
+  unsigned bal[KW];
+#pragma unroll
+  for (int q = 0; q < KW; ++q) {
+    const int jc = (lane + warp * KW + q) & (CV_T - 1);
+    const int j = t.bj * CV_T + jc;
+    const float *x = s_x[CV_T + jc];
+    const bool near = i < t.n_cv && j < t.n_cv && j - i > t.min_sep &&
+                      cv_is_near(x[0] - xi.x, x[1] - xi.y, x[2] - xi.z, t.L, t.iL, t.rc2_far);
+    bal[q] = __ballot_sync(0xffffffffu, near);
+    if (lane == 0) s_bal[warp * KW + q] = bal[q];
+  }
+  __syncthreads();
+  int incl = __popc(s_bal[lane]);
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, incl, off);
+    if (lane >= off) incl += v;
+  }
+#pragma unroll
+  for (int q = 0; q < KW; ++q) {
+    const int end = __shfl_sync(0xffffffffu, incl, warp * KW + q);
+    if ((bal[q] >> lane) & 1u)
+      s_near[end - __popc(bal[q]) + __popc(bal[q] & ((1u << lane) - 1u))] =
+          (unsigned short)(lane | (((lane + warp * KW + q) & (CV_T - 1)) << 5));
+  }
+  __syncthreads();
+  return __shfl_sync(0xffffffffu, incl, 31);
+}
+
+// One warp's tile: z partial sum and gradient.  pos(a): position of
+// reaction-coordinate atom a.
+template <class POS>
+__device__ __forceinline__ void cv_tile(const CvTile &t, const CvConst &k, CvWarpShared &sh, POS pos) {
+  const int lane = threadIdx.x & 31;
+  const int i = t.bi * CV_T + lane, j = t.bj * CV_T + lane;
+  const bool iv = i < t.n_cv, jv = j < t.n_cv;
+  float3 xi = make_float3(0.f, 0.f, 0.f), xj = xi;
+  if (iv) xi = pos(i);
+  if (jv) xj = pos(j);
+  if (cv_tile_far(t, iv, jv, xi, xj)) {
+    if (lane == 0) *t.z_part = 0.0;
+    return;
+  }
+  sh.s_x[lane][0] = xi.x; sh.s_x[lane][1] = xi.y; sh.s_x[lane][2] = xi.z;
+  sh.s_x[CV_T + lane][0] = xj.x; sh.s_x[CV_T + lane][1] = xj.y; sh.s_x[CV_T + lane][2] = xj.z;
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
     sh.s_ghi[lane][q] = 0; sh.s_ghi[CV_T + lane][q] = 0;
     sh.s_glo[lane][q] = 0u; sh.s_glo[CV_T + lane][q] = 0u;
   }
-  // ---- phase 1: near pairs of the tile ----
-  int n_near = 0;
-  for (int k = 0; k < CV_T; ++k) {
-    const int jc = (lane + k) & (CV_T - 1);
-    const int j = W.bj * CV_T + jc;
-    const float xjx = __shfl_sync(0xffffffffu, xj.x, jc);
-    const float xjy = __shfl_sync(0xffffffffu, xj.y, jc);
-    const float xjz = __shfl_sync(0xffffffffu, xj.z, jc);
-    const bool near = i < ncv && j < ncv && j - i > msep &&
-                      cv_is_near(xjx - xi.x, xjy - xi.y, xjz - xi.z, L, iL, c.cv_rc2_far);
-    const unsigned bal = __ballot_sync(0xffffffffu, near);
-    if (near) sh.s_near[n_near + __popc(bal & ((1u << lane) - 1u))] = (unsigned short)(lane | (jc << 5));
-    n_near += __popc(bal);
-  }
+  const int n_near = cv_near_list(t, sh.s_near, xi, xj);
   __syncwarp();
-  // ---- phase 2: the near pairs, densely ----
-  const CvConst k = cv_const(c);
-  const float2 *cn = d.cnat_ff + (size_t)W.tile * CV_T * CV_T;
+  // the near pairs, densely
   ff zacc = {0.f, 0.f};
   for (int base = 0; base < n_near; base += 32)
-    if (base + lane < n_near) zacc = ff_add(zacc, cv_near_pair(sh, k, cn, L, iL, sh.s_near[base + lane]));
+    if (base + lane < n_near) zacc = ff_add(zacc, cv_near_pair(sh, k, t.cn, t.L, t.iL, sh.s_near[base + lane]));
   __syncwarp();
   if (n_near > 0) {
-    if (i < ncv) cv_flush_atom(d, sh, lane, W.cv0 + i);
-    if (jl < ncv) cv_flush_atom(d, sh, CV_T + lane, W.cv0 + jl);
+    if (iv) cv_flush_atom(sh, lane, t.gx + i, t.gy + i, t.gz + i);
+    if (jv) cv_flush_atom(sh, CV_T + lane, t.gx + j, t.gy + j, t.gz + j);
   }
   double zl = ff_to_d(zacc);
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) zl += __shfl_xor_sync(0xffffffffu, zl, off);
-  if (lane == 0) d.z_part[W.w] = zl;
+  if (lane == 0) *t.z_part = zl;
 }
 
-// The same tile by a block of NW warps: the 32 rotations of phase 1 and the
-// chunks of 32 near pairs of phase 2 are dealt out over the warps.  The near
+// The same tile by a block of NW warps: the rotations of the distance tests
+// and the chunks of 32 near pairs are dealt out over the warps.  The near
 // pairs keep the order the one-warp form lists them in, and the z terms go
 // through shared memory so that each lane of the first warp adds them in that
 // order too: z and the gradient are the same bit for bit.
-template <int NW>
 struct CvBlockShared {
   unsigned short s_near[CV_T * CV_T];
   float s_x[2 * CV_T][3];
@@ -124,17 +195,15 @@ struct CvBlockShared {
   float2 s_term[CV_T * CV_T];
 };
 
-template <int NW>
-__device__ __forceinline__ void cv_tile_block(const Dev &d, const SimConst &c, CvBlockShared<NW> &sh, int wq) {
-  constexpr int KW = CV_T / NW;  // rotations per warp
+// positions of the tile's 64 atoms into s_x, its gradient sums cleared;
+// returns (in every thread) whether the tile is far
+template <int NW, class SH, class POS>
+__device__ __forceinline__ bool cv_block_begin(const CvTile &t, SH &sh, POS pos) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const CvItem W = d.cv_item[wq];
-  const int ncv = W.n_cv, msep = c.cv_min_sep;
-  const float L = W.box, iL = W.inv_box;
   if (threadIdx.x < 2 * CV_T) {
-    const int a = (warp == 0 ? W.bi : W.bj) * CV_T + lane;
-    float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (a < ncv) q = d.pos[d.slot_of[W.atom0 + a]];
+    const int a = (warp == 0 ? t.bi : t.bj) * CV_T + lane;
+    float3 q = make_float3(0.f, 0.f, 0.f);
+    if (a < t.n_cv) q = pos(a);
     sh.s_x[threadIdx.x][0] = q.x; sh.s_x[threadIdx.x][1] = q.y; sh.s_x[threadIdx.x][2] = q.z;
   }
   for (int q = threadIdx.x; q < 2 * CV_T * 3; q += NW * 32) {
@@ -142,40 +211,22 @@ __device__ __forceinline__ void cv_tile_block(const Dev &d, const SimConst &c, C
     (&sh.s_glo[0][0])[q] = 0u;
   }
   __syncthreads();
-  const int i = W.bi * CV_T + lane;
-  const float3 xi = make_float3(sh.s_x[lane][0], sh.s_x[lane][1], sh.s_x[lane][2]);
-  unsigned bal[KW];
-#pragma unroll
-  for (int q = 0; q < KW; ++q) {
-    const int jc = (lane + warp * KW + q) & (CV_T - 1);
-    const int j = W.bj * CV_T + jc;
-    const float *x = sh.s_x[CV_T + jc];
-    const bool near = i < ncv && j < ncv && j - i > msep &&
-                      cv_is_near(x[0] - xi.x, x[1] - xi.y, x[2] - xi.z, L, iL, c.cv_rc2_far);
-    bal[q] = __ballot_sync(0xffffffffu, near);
-    if (lane == 0) sh.s_bal[warp * KW + q] = bal[q];
+  return cv_tile_far(t, t.bi * CV_T + lane < t.n_cv, t.bj * CV_T + lane < t.n_cv,
+                     make_float3(sh.s_x[lane][0], sh.s_x[lane][1], sh.s_x[lane][2]),
+                     make_float3(sh.s_x[CV_T + lane][0], sh.s_x[CV_T + lane][1], sh.s_x[CV_T + lane][2]));
+}
+
+template <int NW, class POS>
+__device__ __forceinline__ void cv_tile_block(const CvTile &t, const CvConst &k, CvBlockShared &sh, POS pos) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (cv_block_begin<NW>(t, sh, pos)) {
+    if (threadIdx.x == 0) *t.z_part = 0.0;
+    return;
   }
-  __syncthreads();
-  int incl = __popc(sh.s_bal[lane]);
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const int v = __shfl_up_sync(0xffffffffu, incl, off);
-    if (lane >= off) incl += v;
-  }
-  const int n_near = __shfl_sync(0xffffffffu, incl, 31);
-#pragma unroll
-  for (int q = 0; q < KW; ++q) {
-    const int end = __shfl_sync(0xffffffffu, incl, warp * KW + q);
-    if ((bal[q] >> lane) & 1u)
-      sh.s_near[end - __popc(bal[q]) + __popc(bal[q] & ((1u << lane) - 1u))] =
-          (unsigned short)(lane | (((lane + warp * KW + q) & (CV_T - 1)) << 5));
-  }
-  __syncthreads();
-  const CvConst k = cv_const(c);
-  const float2 *cn = d.cnat_ff + (size_t)W.tile * CV_T * CV_T;
+  const int n_near = cv_near_list_block<NW>(t, sh.s_near, sh.s_bal, sh.s_x);
   for (int p = threadIdx.x; p < n_near; p += NW * 32) {
-    const ff t = cv_near_pair(sh, k, cn, L, iL, sh.s_near[p]);
-    sh.s_term[p] = make_float2(t.hi, t.lo);
+    const ff v = cv_near_pair(sh, k, t.cn, t.L, t.iL, sh.s_near[p]);
+    sh.s_term[p] = make_float2(v.hi, v.lo);
   }
   __syncthreads();
   if (warp == 0) {
@@ -184,12 +235,29 @@ __device__ __forceinline__ void cv_tile_block(const Dev &d, const SimConst &c, C
     double zl = ff_to_d(zacc);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) zl += __shfl_xor_sync(0xffffffffu, zl, off);
-    if (lane == 0) d.z_part[W.w] = zl;
+    if (lane == 0) *t.z_part = zl;
   } else if (warp <= 2 && n_near > 0) {
-    const int a = (warp == 1 ? W.bi : W.bj) * CV_T + lane;
-    if (a < ncv) cv_flush_atom(d, sh, (warp - 1) * CV_T + lane, W.cv0 + a);
+    const int a = (warp == 1 ? t.bi : t.bj) * CV_T + lane;
+    if (a < t.n_cv) cv_flush_atom(sh, (warp - 1) * CV_T + lane, t.gx + a, t.gy + a, t.gz + a);
   }
 }
+
+// the tile of work item wq of the batch's flat (trial, tile) list, in the
+// work order (costliest tiles first; the partial sums of z keep their slots)
+__device__ __forceinline__ CvTile cv_item_tile(const Dev &d, const SimConst &c, const CvItem &W) {
+  return CvTile{W.n_cv, W.bi, W.bj, c.cv_min_sep, W.box, W.inv_box, c.cv_rc2_far,
+                d.cnat_ff + (size_t)W.tile * CV_T * CV_T, d.gx + W.cv0, d.gy + W.cv0, d.gz + W.cv0, d.z_part + W.w};
+}
+
+// positions of a trial's reaction-coordinate atoms (caller order)
+struct CvSlotPos {
+  const Dev &d;
+  int atom0;
+  __device__ __forceinline__ float3 operator()(int a) const {
+    const float4 q = d.pos[d.slot_of[atom0 + a]];
+    return make_float3(q.x, q.y, q.z);
+  }
+};
 
 
 // The finaliser of trial t by one block of any size: the reduction runs over

@@ -43,7 +43,6 @@ struct Dev {
   double *z_part;                      // [total_work] per-tile partial sums of z
   // per system, caller-ordered
   AtomSys *asys;
-  double *gm;                          // gamma_i m_i
   double *inv_gm;                      // 1 / (gamma_i m_i) (0 without friction)
   int32_t *excl, *excl_n;              // [sys atoms * MAX_EXCL], counts
   int32_t *bt_start;                   // [total system atoms + 1] CSR of owner-computed bonded terms (energies)
@@ -125,6 +124,7 @@ struct CvWarpShared {
   int s_ghi[2 * CV_T][3];
   unsigned s_glo[2 * CV_T][3];
 };
+constexpr int CV_BLOCK_WARPS = 4;  // warps per tile of the block form
 constexpr int CVFIN_THREADS = 1024;  // the finaliser's reduction width (virtual threads)
 struct CvfinShared {
   double rz[CVFIN_THREADS], rq[CVFIN_THREADS];

@@ -183,6 +183,18 @@ __device__ __forceinline__ float3 normal3(uint32_t k0, uint32_t k1, uint32_t ato
   return make_float3(r01 * c1, r01 * s1, r23 * cospif(2.0f * u3));
 }
 
+// least and greatest of the warp's values (redux on FP32: one instruction)
+__device__ __forceinline__ float warp_min(float v) {
+  float r;
+  asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+  return r;
+}
+__device__ __forceinline__ float warp_max(float v) {
+  float r;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+  return r;
+}
+
 // ---------------------------------------------------------------------------
 // fixed point
 // ---------------------------------------------------------------------------

@@ -449,18 +449,6 @@ struct ListShared {
                                                // first words overwrite s_cand)
 };
 
-// least and greatest of the warp's values (redux on FP32: one instruction)
-__device__ __forceinline__ float warp_min(float v) {
-  float r;
-  asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
-  return r;
-}
-__device__ __forceinline__ float warp_max(float v) {
-  float r;
-  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
-  return r;
-}
-
 __device__ __forceinline__ void list_cluster(const Dev &d, const SimConst &c, float rl2_bbox, ListShared &sh, int t,
                                              int Il) {
   const int wib = threadIdx.x >> 5;

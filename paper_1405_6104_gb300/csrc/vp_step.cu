@@ -140,7 +140,8 @@ __global__ void __launch_bounds__(STEP_THREADS, MINB)
       if (lane == 0) got = atomicAdd(d.pair_next + 1, 1u);
       const int item = (int)__shfl_sync(0xffffffffu, got, 0);
       if (item < n_cv) {
-        cv_tile(d, c, sh.force.cv[wib], item);
+        const CvItem W = d.cv_item[item];
+        cv_tile(cv_item_tile(d, c, W), cv_const(c), sh.force.cv[wib], CvSlotPos{d, W.atom0});
       } else if (item < n_cv + n_pair) {
         pair_cluster_f2<1>(d, c, sh.force.pair, item - n_cv);
       } else if (item < n_cv + n_pair + n_bond) {
