@@ -104,12 +104,12 @@ __global__ void __launch_bounds__(FIN_THREADS) k_adj_fin(AdjDev a) {
 // Coefficients A_n, B_n and Phi from z and Q along the path (z_m starts at
 // z_0), one block.  Per SCAN frames: one warp forms the running minimum before
 // each frame (a scan of 32 at a time) and a = (z - z_m)_+; all threads write
-// the coefficients; then one thread sums Phi and another what the frames pass
-// on to the frame their running minimum sits at (those frames are
-// consecutive, so one running sum, put down when the minimum moves), both in
-// frame order.  The two sums are chains of one dependent operation per frame
-// on shared memory; one thread doing everything from global memory took 294
-// us for 501 frames.
+// the coefficients and the terms of the sums; then one warp adds up Phi and a
+// thread what the frames pass on to the frame their running minimum sits at
+// (those frames are consecutive, so one running sum, put down when the minimum
+// moves).  That last sum is the only chain of a dependent operation per frame
+// left, on shared memory; one thread doing everything from global memory took
+// 294 us for 501 frames.
 constexpr int SCAN = 1024;
 __global__ void __launch_bounds__(256) k_adj_scan(const double *z, const double *Q, int nf, double c, double *coef,
                                                   double *phi_out) {
@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(256) k_adj_scan(const double *z, const double 
   const double z0 = z[0];
   // a path that starts at NaN never compares below or above its minimum
   const bool dead = isnan(z0);
-  double Phi = 0.0, R = 0.0;  // thread 32, thread 64
+  double Phi = 0.0, R = 0.0;  // warp 1, thread 64
   int arg = 0;                // thread 64
   if (threadIdx.x == 0) {
     s_m = z0;
@@ -158,16 +158,18 @@ __global__ void __launch_bounds__(256) k_adj_scan(const double *z, const double 
     }
     __syncthreads();
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
-      const double a = s_a[k];
+      const double a = s_a[k], q = s_q[k];
       coef[2 * (f0 + k) + 1] = 2.0 * c * a * a;
-      coef[2 * (f0 + k)] = 2.0 * c * a * s_q[k];
+      coef[2 * (f0 + k)] = 2.0 * c * a * q;
+      s_a[k] = c * a * a * q;               // the frame's share of Phi ...
+      s_q[k] = a > 0.0 ? 2.0 * a * q : 0.0;  // ... and what it passes on
     }
     __syncthreads();
-    if (threadIdx.x == 32) {
-      for (int k = 0; k < n; ++k) Phi = fma(c * s_a[k] * s_a[k], s_q[k], Phi);
+    if (threadIdx.x >= 32 && threadIdx.x < 64) {
+      for (int k = threadIdx.x - 32; k < n; k += 32) Phi += s_a[k];
     } else if (threadIdx.x == 64) {
       for (int k = 0; k < n; ++k) {
-        if (s_a[k] > 0.0) R = fma(2.0 * s_a[k], s_q[k], R);
+        R += s_q[k];
         if (s_new[k]) {
           coef[2 * arg] = fma(-c, R, coef[2 * arg]);
           arg = f0 + k;
@@ -178,7 +180,11 @@ __global__ void __launch_bounds__(256) k_adj_scan(const double *z, const double 
     __syncthreads();  // the shared arrays are taken anew
   }
   if (threadIdx.x == 64) coef[2 * arg] = fma(-c, R, coef[2 * arg]);
-  if (threadIdx.x == 32 && phi_out) *phi_out = Phi;
+  if (threadIdx.x >= 32 && threadIdx.x < 64) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) Phi += __shfl_xor_sync(0xffffffffu, Phi, off);
+    if (threadIdx.x == 32 && phi_out) *phi_out = Phi;
+  }
 }
 
 // shared memory of a tile of H_z w
@@ -385,8 +391,10 @@ AdjDev adj_arrays(const AdjInput &in, Carve &c) {
   return a;
 }
 
-// few tiles: a block each (see launch_cv)
-bool block_form(const AdjInput &in) { return (long long)in.n_frames * in.n_tiles <= 16ll * in.n_sm; }
+// A block per tile up to 128 tiles per SM: these kernels run alone, so the
+// block form pays longer than beside the pair kernel (see launch_cv).  5576
+// tiles: z and grad z 72 -> 55 us, H_z w 68 -> 46; 84 303 tiles: 311 -> 350.
+bool block_form(const AdjInput &in) { return (long long)in.n_frames * in.n_tiles <= 128ll * in.n_sm; }
 
 void launch_adj_cv(const AdjInput &in, const AdjDev &a, cudaStream_t st) {
   const long long tiles = (long long)a.nf * a.n_tiles;
