@@ -370,7 +370,7 @@ int sim_philox_normals(uint64_t seed, int64_t step, uint32_t stream, int32_t n, 
  *   box: cubic side (rounded to FP32); params: cv_r0, cv_r_switch, cv_r_cut
  *   and cv_min_sep are read (host pointer);
  *   d_z [1] and d_grad [3*n_cv]: DEVICE pointers, written (FP64);
- *   cuda_stream: the stream the three launches go to (NULL: legacy stream);
+ *   cuda_stream: the stream the work goes to (NULL: legacy stream);
  *     the call returns after queueing them -- synchronise before reading;
  *   errbuf/errlen: optional host buffer for a message.
  * Scratch lives in a static device array of fixed size (112 KiB, held by every
