@@ -416,11 +416,11 @@ int sim_contact_times(sim_handle *h, int32_t trial, int64_t *times, int64_t cap)
  * read; a negative time: not formed, ordered after every formed contact),
  * pairs [2*n_pairs] path indices (HOST), s [n_pairs] (HOST, written):
  * s(pairs[2q], pairs[2q+1]).  Only the order of the times within a path
- * enters s, so the host replaces them by dense ranks.  A path pair whose
- * paths hold K_a and K_b distinct times with K_a K_b <= 4096 is counted from
- * the joint histogram of its ranks (every pair of contacts in one cell ties
- * in both paths, pairs of cells strictly below-left / above-right are
- * concordant); other pairs compare all ordered contact pairs.  Both counts
+ * enters s, so they are replaced by dense ranks.  A path pair whose paths hold
+ * K_a and K_b distinct times (at most 4096 each) with K_a K_b <= 53248 is
+ * counted from the joint histogram of its ranks (every pair of contacts in one
+ * cell ties in both paths, pairs of cells strictly below-left / above-right
+ * are concordant); other pairs compare all ordered contact pairs.  Both counts
  * are exact.  n_c < 2 gives 1 (no ordered pair); n_c <= 2^30.  At most 65535
  * pairs per call.  Returns SIM_OK, SIM_EINVAL or SIM_ECUDA. */
 int path_similarity(const int64_t *times, int32_t n_paths, int64_t n_c, const int32_t *pairs, int32_t n_pairs,

@@ -111,7 +111,7 @@ __device__ __forceinline__ double native_contact(double d2, const Consts &k) {
 // the native structure, and eight warps per tile to have their chains of
 // float-float operations side by side.  One warp per tile with the full FP64
 // contact per pair, and clearing and finishing kernels around it, took 103 us
-// (n_cv = 540); this one 14.
+// (n_cv = 540); this one 24.
 constexpr int NW = 8;
 struct TileShared {
   unsigned short s_near[CV_T * CV_T];
