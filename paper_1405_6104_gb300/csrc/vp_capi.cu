@@ -1207,19 +1207,25 @@ VP_API int sim_potential_device(sim_handle *h, const double *d_pos, double *d_en
   const Dev &d = h->d;
   int n = 0;
   for (const auto &T : h->tinfo) n += T.n_atoms;
-  // requests of earlier calls at this step number must not count again
-  CK(cudaMemsetAsync(d.rb, 0xff, 2 * sizeof(uint32_t) * (size_t)h->n_trials, s));
-  CK(cudaMemsetAsync(d.err, 0, sizeof(int), s));
-  CK(cudaMemsetAsync(d.fx, 0, sizeof(long long) * d.total_slots, s));
-  CK(cudaMemsetAsync(d.fy, 0, sizeof(long long) * d.total_slots, s));
-  CK(cudaMemsetAsync(d.fz, 0, sizeof(long long) * d.total_slots, s));
-  CK(cudaMemsetAsync(d.energy, 0, sizeof(long long) * 5 * (size_t)h->n_trials, s));
+  launch_potential_begin(d, s);
   launch_scatter_positions(d, h->c, d_pos, n, s);
   rebuild_cols(h, false);
+  // the bonded terms read only positions: beside the list build and the pair
+  // kernel, as in a step
+  const bool one_pass = d_energy && pair_energy_in_one_pass(h->c);
+  CK(cudaEventRecord(h->ev_fork, s));
+  CK(cudaStreamWaitEvent(h->bstream, h->ev_fork, 0));
+  launch_bonded(d, h->bstream);
+  if (one_pass) launch_bonded_energy(d, h->bstream);
+  CK(cudaEventRecord(h->ev_bjoin, h->bstream));
   rebuild_list(h);
-  launch_pair_hot(h, d, s);
-  launch_bonded(d, s);
-  launch_pair(d, h->c, true, -1, s);
+  if (one_pass) {
+    launch_pair_energy(d, h->c, s);
+  } else {
+    launch_pair_hot(h, d, s);
+    if (d_energy) launch_pair(d, h->c, true, -1, s);
+  }
+  CK(cudaStreamWaitEvent(s, h->ev_bjoin, 0));
   launch_potential_out(d, d_energy, d_forces, n, s);
   CK(cudaGetLastError());
   CK(cudaEventRecord(h->exit_ev, s));

@@ -174,6 +174,9 @@ void launch_pair(const Dev &d, const SimConst &c, bool energy, int32_t only_tria
                  const int *clist = nullptr, int n_items = 0);
 int default_pair_variant(const Dev &d, const SimConst &c);
 void launch_bonded(const Dev &d, cudaStream_t s);
+bool pair_energy_in_one_pass(const SimConst &c);
+void launch_pair_energy(const Dev &d, const SimConst &c, cudaStream_t s);
+void launch_bonded_energy(const Dev &d, cudaStream_t s);
 constexpr int PAIR_VARIANTS = 9;
 // reaction coordinate and functional (vp_cv.cu)
 void launch_cnat(const Dev &d, const SimConst &c, const double *native, const int32_t *sys_nat0, int32_t n_tiles_total,
@@ -192,6 +195,7 @@ void launch_gather_state(const Dev &d, int32_t trial, double *pos, double *vel, 
 void launch_check_finite(const double *x, size_t n, int *flag, cudaStream_t s);
 void launch_forces_out(const Dev &d, const SimConst &c, int32_t trial, double *out, int32_t n, cudaStream_t s);
 void launch_kinetic(const Dev &d, int32_t trial, cudaStream_t s);
+void launch_potential_begin(const Dev &d, cudaStream_t s);
 void launch_scatter_positions(const Dev &d, const SimConst &c, const double *pos, int32_t n, cudaStream_t s);
 void launch_potential_out(const Dev &d, double *energy, double *forces, int32_t n, cudaStream_t s);
 void launch_extract_pairs(const Dev &d, int32_t list_cap, int32_t trial, int32_t n_clus, int32_t *pairs,

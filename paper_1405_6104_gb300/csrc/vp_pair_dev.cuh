@@ -20,9 +20,19 @@ __device__ __forceinline__ float3 min_disp(float4 self, float4 other, float L, f
 constexpr int PF_WARPS = 4;
 constexpr float MASK_PEN = 1.0e30f;
 
-// shared memory of the packed pair kernel's warps
+// the energies' tables of a warp: {c12, c12', c6, c6'} (over r^12 and r^6) and the
+// potential at the cut-off per i-atom pair and type
+template <int NW, bool ENERGY>
+struct PairEnergyTables {
+  float4 s_e4[NW][CL / 2][SMALL_TYPES];
+  float2 s_ts[NW][CL / 2][SMALL_TYPES];
+};
 template <int NW>
-struct PairF2Shared {
+struct PairEnergyTables<NW, false> {};
+
+// shared memory of the packed pair kernel's warps
+template <int NW, bool ENERGY = false>
+struct PairF2Shared : PairEnergyTables<NW, ENERGY> {
   float4 s_c4[NW][CL / 2][SMALL_TYPES];
   float4 s_sh[NW][64];
   float4 s_ip[NW][CL / 2][2];
@@ -40,8 +50,11 @@ struct PairF2Shared {
 // against 20 us; U = 3 and 4, or U = 2 without the early loads, are slower).
 // Every accumulator takes its terms in the order of the groups either way:
 // the same forces bit for bit.
-template <int U, int NW>
-__device__ __forceinline__ void pair_cluster_f2(const Dev &d, const SimConst &c, PairF2Shared<NW> &sh, int I) {
+// ENERGY (U = 1): the Lennard-Jones and reaction-field energies too, each lane
+// adding its pairs' in the order of the entries and i-atoms.
+template <int U, int NW, bool ENERGY = false>
+__device__ __forceinline__ void pair_cluster_f2(const Dev &d, const SimConst &c, PairF2Shared<NW, ENERGY> &sh, int I) {
+  static_assert(!ENERGY || U == 1, "the energies' sums take one group at a time");
   constexpr int TS = SMALL_TYPES;
   auto &s_c4 = sh.s_c4;
   auto &s_sh = sh.s_sh;
@@ -94,6 +107,11 @@ __device__ __forceinline__ void pair_cluster_f2(const Dev &d, const SimConst &c,
       const int p = k / NT, tj = k - p * NT;
       const float2 c0 = d.ljtab[ty[r][0] * NT + tj], c1 = d.ljtab[ty[r][1] * NT + tj];
       s_c4[wib][p][tj] = make_float4(c0.y, c1.y, -c0.x, -c1.x);
+      if constexpr (ENERGY) {
+        sh.s_e4[wib][p][tj] = make_float4(__fmul_rn(c0.y, 1.0f / 12.0f), __fmul_rn(c1.y, 1.0f / 12.0f),
+                                          __fmul_rn(c0.x, 1.0f / 6.0f), __fmul_rn(c1.x, 1.0f / 6.0f));
+        sh.s_ts[wib][p][tj] = make_float2(d.ljshift[ty[r][0] * NT + tj], d.ljshift[ty[r][1] * NT + tj]);
+      }
     }
   }
   for (int k = lane; k < 64; k += 32) {
@@ -106,12 +124,24 @@ __device__ __forceinline__ void pair_cluster_f2(const Dev &d, const SimConst &c,
   for (int p = 0; p < CL / 2; ++p) fx[p] = fy[p] = fz[p] = make_float2(0.f, 0.f);
   const float2 m2krf = make_float2(-c.two_krf, -c.two_krf);
   const float rc2 = c.rc2;
+  float elj = 0.0f, erf = 0.0f;
+  // the energies of one pair inside the cut-off (hh: which i-atom of pair p)
+  auto add_energy = [&](int tj, int p, int hh, float rinv, float rinv6, float r2, float qq) {
+    if constexpr (ENERGY) {
+      const float4 e = sh.s_e4[wib][p][tj];
+      const float2 ts = sh.s_ts[wib][p][tj];
+      const float lj = __fmaf_rn(hh ? e.y : e.x, rinv6, -(hh ? e.w : e.z));
+      elj = __fadd_rn(elj, __fmaf_rn(rinv6, lj, -(hh ? ts.y : ts.x)));
+      erf = __fmaf_rn(qq, __fsub_rn(__fmaf_rn(c.krf, r2, rinv), c.crf), erf);
+    }
+  };
 
   // one pair of i-atoms (2p, 2p + 1) against this lane's j-atom (image
   // already applied): the i-forces into fx/fy/fz, the j-force into gx/gy/gz
   struct JAtom {
     float2 x, y, z, q;
     const float4 *row;
+    int tj;
     float2 gx, gy, gz;
   };
   auto j_atom = [&](float4 pj, int tj, uint32_t ent) {
@@ -123,6 +153,7 @@ __device__ __forceinline__ void pair_cluster_f2(const Dev &d, const SimConst &c,
     j.z = make_float2(zj, zj);
     j.q = make_float2(pj.w, pj.w);
     j.row = &s_c4[wib][0][tj];
+    j.tj = tj;
     j.gx = j.gy = j.gz = make_float2(0.f, 0.f);
     return j;
   };
@@ -147,8 +178,14 @@ __device__ __forceinline__ void pair_cluster_f2(const Dev &d, const SimConst &c,
     tt = __ffma2_rn(qq, rinv, tt);
     tt = __fmul2_rn(tt, rinv2);
     float2 f = __ffma2_rn(qq, m2krf, tt);
-    f.x = ((!MASKED || (mb & (1u << (2 * p)))) && r2.x < rc2) ? f.x : 0.0f;
-    f.y = ((!MASKED || (mb & (1u << (2 * p + 1)))) && r2.y < rc2) ? f.y : 0.0f;
+    const bool inx = (!MASKED || (mb & (1u << (2 * p)))) && r2.x < rc2,
+               iny = (!MASKED || (mb & (1u << (2 * p + 1)))) && r2.y < rc2;
+    f.x = inx ? f.x : 0.0f;
+    f.y = iny ? f.y : 0.0f;
+    if constexpr (ENERGY) {
+      if (inx) add_energy(j.tj, p, 0, rinv.x, rinv6.x, r2.x, qq.x);
+      if (iny) add_energy(j.tj, p, 1, rinv.y, rinv6.y, r2.y, qq.y);
+    }
     fx[p] = __ffma2_rn(f, dx, fx[p]);
     fy[p] = __ffma2_rn(f, dy, fy[p]);
     fz[p] = __ffma2_rn(f, dz, fz[p]);
@@ -198,6 +235,7 @@ __device__ __forceinline__ void pair_cluster_f2(const Dev &d, const SimConst &c,
           tt = __fmaf_rn(qq, rinv, tt);
           tt = __fmul_rn(tt, rinv2);
           float f = __fmaf_rn(qq, -c.two_krf, tt);
+          if (ENERGY && r2 < rc2) add_energy(j.tj, p, hh, rinv, rinv6, r2, qq);
           f = r2 < rc2 ? f : 0.0f;
           if (hh) { f2v.y = f; dx2.y = dx; dy2.y = dy; dz2.y = dz; }
           else { f2v.x = f; dx2.x = dx; dy2.x = dy; dz2.x = dz; }
@@ -305,6 +343,16 @@ __device__ __forceinline__ void pair_cluster_f2(const Dev &d, const SimConst &c,
     const int a = lane / 3, comp = lane - 3 * a;
     const long long val = fx_from(sum);
     if (val != 0) red_add((comp == 0 ? d.fx : comp == 1 ? d.fy : d.fz) + I * CL + a, val);
+  }
+  if constexpr (ENERGY) {
+    double e2[2] = {(double)elj, (double)erf};
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) e2[k] += __shfl_xor_sync(0xffffffffu, e2[k], off);
+    if (lane == 0)
+#pragma unroll
+      for (int k = 0; k < 2; ++k) red_add(d.energy + (size_t)t * 5 + k, __double2ll_rn(e2[k] * E_SCALE));
   }
 }
 

@@ -7,6 +7,8 @@
 // kick of one step and the opening half kick of the next are one kick of
 // dt (the device scalar `kick` is 0.5 at the first step of a call and 1.0
 // afterwards); a final half kick (UPD_FINAL) closes the call.
+#include <algorithm>
+
 #include "vp_dev.cuh"
 #include "vp_update_dev.cuh"
 
@@ -115,6 +117,17 @@ __global__ void k_forces_out(Dev d, SimConst c, int trial, double *out, int n) {
     F[2] += k * (double)d.gz[T.cv0 + o];
   }
   out[3 * o] = F[0]; out[3 * o + 1] = F[1]; out[3 * o + 2] = F[2];
+}
+
+// The accumulators of an evaluation of the potential cleared, and the rebuild
+// requests of earlier calls at this step number withdrawn (one launch instead
+// of six memsets)
+__global__ void __launch_bounds__(256) k_potential_begin(Dev d) {
+  const int k = blockIdx.x * 256 + threadIdx.x;
+  if (k < d.total_slots) { d.fx[k] = 0; d.fy[k] = 0; d.fz[k] = 0; }
+  if (k < 5 * d.n_trials) d.energy[k] = 0;
+  if (k < 2 * d.n_trials) d.rb[k] = 0xffffffffu;
+  if (k == 0) *d.err = 0;
 }
 
 // Positions of every trial from a device array (trials concatenated, caller
@@ -258,6 +271,10 @@ void launch_forces_out(const Dev &d, const SimConst &c, int32_t trial, double *o
   if (n > 0) k_forces_out<<<(n + 255) / 256, 256, 0, s>>>(d, c, trial, out, n);
 }
 void launch_kinetic(const Dev &d, int32_t trial, cudaStream_t s) { k_kinetic<<<1, 256, 0, s>>>(d, trial); }
+void launch_potential_begin(const Dev &d, cudaStream_t s) {
+  const int n = std::max(d.total_slots, 5 * d.n_trials);
+  k_potential_begin<<<(n + 255) / 256, 256, 0, s>>>(d);
+}
 void launch_scatter_positions(const Dev &d, const SimConst &c, const double *pos, int32_t n, cudaStream_t s) {
   if (n > 0) k_scatter_positions<<<(n + 255) / 256, 256, 0, s>>>(d, c, pos, n);
 }

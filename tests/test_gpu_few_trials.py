@@ -65,3 +65,28 @@ def test_lists_with_many_excluded_partners_are_bit_exact(per_atom):
         got = {tuple(x) for x in B.sim_pairlist(b.h, 0).tolist()}
     ref = {tuple(x) for x in O.pairlist(s, pos.astype(np.float32), p.r_cut + p.skin).tolist()}
     assert got == ref and len(ref) > 10 * s.n_atoms
+
+
+@pytest.mark.parametrize("n_solute,n_water", [(6, 430), (37, 420), (60, 440)])
+def test_one_pass_energies_match_the_general_kernel(n_solute, n_water):
+    """Energies of the one-pass force and energy kernel (device tensors) and
+    of the general energy kernel (energy_forces) on the same configuration and
+    lists, bonds and angles strained, in the smallest boxes (pair-by-pair
+    images): equal to the last bit of the fixed-point sums."""
+    import torch
+
+    from paper_1405_6104_gb300 import autograd as U
+
+    s, p = S.small_solvated(n_solute=n_solute, n_water=n_water)
+    rng = np.random.default_rng(n_solute)
+    ev = U.Evaluator(s, p, n_conf=2)
+    try:
+        for k in range(3):  # the lists of the first serve the second, the third needs new ones
+            x = s.pos[None] + 0.004 * rng.normal(size=(2, s.n_atoms, 3)) + (0.3 if k == 2 else 0.0)
+            x = x.astype(np.float32).astype(np.float64)
+            u, f = ev.device_energy_and_forces(torch.tensor(x, device="cuda"))
+            for t in range(2):
+                e, _ = ev.batch.energy_forces(t)
+                assert float(u[t]) == pytest.approx(e[:4].sum(), rel=1e-15)
+    finally:
+        ev.close()
