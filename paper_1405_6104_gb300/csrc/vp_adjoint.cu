@@ -54,11 +54,21 @@ __device__ __forceinline__ CvTile adj_tile(const AdjDev &a, const CvConst &k, in
 // (frame, tile): the tile routines of the batched kernel, which evaluate the
 // near pairs densely and leave a tile of far blocks at once.  One lane per i
 // and a loop over j, near or far, took 625 us for 51 frames of 1800 atoms.
+//
+// Two pairs per lane on the packed FP32 instructions, two warps per block at 64
+// registers: bound by issue (64% of the slots) and the FP32 latency of the 10
+// warps an SM holds on average, half of all tiles being far and gone at once.
+// 84 303 tiles of 51 frames of 1800 atoms: 311 -> 275 us, H_z w 340 -> 290 (one
+// pair per lane, four warps per block before; two warps alone -5 us, the
+// register limit another -5).
+constexpr int ADJ_WARPS = 2;  // tiles per block of the one-warp form
+constexpr int adj_threads(int nw) { return 32 * (nw == 1 ? ADJ_WARPS : nw); }
+constexpr int adj_blocks(int nw) { return nw == 1 ? 16 : 8; }  // 64 registers
 template <int NW>
-__global__ void __launch_bounds__(128) k_adj_cv(AdjDev a, CvConst k) {
+__global__ void __launch_bounds__(adj_threads(NW), adj_blocks(NW)) k_adj_cv(AdjDev a, CvConst k) {
   if constexpr (NW == 1) {
-    __shared__ CvWarpShared sh[4];
-    const int w = blockIdx.x * 4 + (threadIdx.x >> 5);
+    __shared__ CvWarpShared sh[ADJ_WARPS];
+    const int w = blockIdx.x * ADJ_WARPS + (threadIdx.x >> 5);
     if (w >= a.nf * a.n_tiles) return;
     const int f = w / a.n_tiles, t = w - f * a.n_tiles;
     cv_tile(adj_tile(a, k, f, t), k, sh[threadIdx.x >> 5], AdjFramePos{a.frames + (size_t)f * 3 * a.n_cv});
@@ -190,61 +200,46 @@ __global__ void __launch_bounds__(256) k_adj_scan(const double *z, const double 
 // shared memory of a tile of H_z w
 struct AdjHwShared {
   unsigned short s_near[CV_T * CV_T];
-  float s_x[2 * CV_T][3], s_w[2 * CV_T][3];
+  float4 s_x[2 * CV_T], s_w[2 * CV_T];
   int s_ghi[2 * CV_T][3];
-  unsigned s_glo[2 * CV_T][3];
+  int s_glo[2 * CV_T][3];
 };
 
-// One near pair of H_z w: it adds K (w_j - w_i) to atom j and subtracts it
-// from atom i, K v = f'' u (u.v) + (f'/r)(v - u (u.v)), f = (C~ - C~_nat)^2.
-// The sums are 64-bit fixed point, kept per tile as two 32-bit parts (see
-// CvWarpShared); a contribution too large for those goes straight to memory
-// (the sum is the same).
-__device__ __forceinline__ void adj_hw_pair(AdjHwShared &sh, const CvTile &t, const CvConst &k, unsigned e) {
-  const int il = e & 31, jc = e >> 5;
-  const float3 xi = make_float3(sh.s_x[il][0], sh.s_x[il][1], sh.s_x[il][2]);
-  ff dx, dy, dz;
-  cv_delta(xi, sh.s_x[CV_T + jc][0], sh.s_x[CV_T + jc][1], sh.s_x[CV_T + jc][2], t.L, t.iL, dx, dy, dz);
-  const float2 cv2 = t.cn[((jc - il) & (CV_T - 1)) * CV_T + il];
-  const ff r2 = ff_add(ff_add(ff_sqr(dx), ff_sqr(dy)), ff_sqr(dz));
-  const CvPair cp = cv_contact<true>(r2, k);
-  const float h = ff_add(cp.Ct, ff{-cv2.x, -cv2.y}).hi;
-  const float f1 = 2.0f * h * cp.dCt;
-  const float f2 = 2.0f * (cp.dCt * cp.dCt + h * cp.d2Ct);
-  const float ir = 1.0f / cp.r;
-  const float ux = dx.hi * ir, uy = dy.hi * ir, uz = dz.hi * ir;
-  const float vx = sh.s_w[CV_T + jc][0] - sh.s_w[il][0], vy = sh.s_w[CV_T + jc][1] - sh.s_w[il][1],
-              vz = sh.s_w[CV_T + jc][2] - sh.s_w[il][2];
-  const float uv = ux * vx + uy * vy + uz * vz;
-  const float q = f1 * ir;
-  const float kx = f2 * ux * uv + q * (vx - ux * uv);
-  const float ky = f2 * uy * uv + q * (vy - uy * uv);
-  const float kz = f2 * uz * uv + q * (vz - uz * uv);
-  const long long ev[3] = {fx_from(kx), fx_from(ky), fx_from(kz)};
-  long long *const gp[3] = {t.gx, t.gy, t.gz};
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const long long v = ev[c];
-    if (v == 0) continue;
-    if (v < (1ll << 49) && v > -(1ll << 49)) {
-      atomicAdd(&sh.s_ghi[il][c], (int)((-v) >> 24));
-      atomicAdd(&sh.s_glo[il][c], (unsigned)((-v) & 0xffffff));
-      atomicAdd(&sh.s_ghi[CV_T + jc][c], (int)(v >> 24));
-      atomicAdd(&sh.s_glo[CV_T + jc][c], (unsigned)(v & 0xffffff));
-    } else {
-      red_add(gp[c] + t.bi * CV_T + il, (long long)(0ull - (unsigned long long)v));
-      red_add(gp[c] + t.bj * CV_T + jc, v);
-    }
-  }
+// Two near pairs of H_z w (the second only when v1): a pair adds K (w_j - w_i)
+// to atom j and subtracts it from atom i, K v = f'' u (u.v) +
+// (f'/r)(v - u (u.v)), f = (C~ - C~_nat)^2.
+__device__ __forceinline__ void adj_hw_pairs(AdjHwShared &sh, const CvTile &t, const CvConst &k, unsigned e0, unsigned e1,
+                                             bool v1) {
+  const int il0 = e0 & 31, jc0 = e0 >> 5, il1 = e1 & 31, jc1 = e1 >> 5;
+  ff2 dx, dy, dz;
+  cv_delta2(sh.s_x[il0], sh.s_x[il1], sh.s_x[CV_T + jc0], sh.s_x[CV_T + jc1], t.L, t.iL, dx, dy, dz);
+  const float2 n0 = t.cn[((jc0 - il0) & (CV_T - 1)) * CV_T + il0], n1 = t.cn[((jc1 - il1) & (CV_T - 1)) * CV_T + il1];
+  const ff2 r2 = ff2_add(ff2_add(ff2_sqr(dx), ff2_sqr(dy)), ff2_sqr(dz));
+  const CvPair2 cp = cv_contact2<true>(r2, k);
+  const float2 h = ff2_sub(cp.Ct, ff2{make_float2(n0.x, n1.x), make_float2(n0.y, n1.y)}).hi;
+  const float2 f1 = __fmul2_rn(__fadd2_rn(h, h), cp.dCt);
+  const float2 fh = __ffma2_rn(cp.dCt, cp.dCt, __fmul2_rn(h, cp.d2Ct)), f2 = __fadd2_rn(fh, fh);
+  const float2 ir = f2_rcp(cp.r);
+  const float2 ux = __fmul2_rn(dx.hi, ir), uy = __fmul2_rn(dy.hi, ir), uz = __fmul2_rn(dz.hi, ir);
+  const float4 wi0 = sh.s_w[il0], wi1 = sh.s_w[il1], wj0 = sh.s_w[CV_T + jc0], wj1 = sh.s_w[CV_T + jc1];
+  const float2 vx = f2_sub(make_float2(wj0.x, wj1.x), make_float2(wi0.x, wi1.x)),
+               vy = f2_sub(make_float2(wj0.y, wj1.y), make_float2(wi0.y, wi1.y)),
+               vz = f2_sub(make_float2(wj0.z, wj1.z), make_float2(wi0.z, wi1.z));
+  const float2 uv = __ffma2_rn(uz, vz, __ffma2_rn(ux, vx, __fmul2_rn(uy, vy)));
+  const float2 q = __fmul2_rn(f1, ir);
+  const float2 g[3] = {__ffma2_rn(__fmul2_rn(f2, ux), uv, __fmul2_rn(q, f2_nma(ux, uv, vx))),
+                       __ffma2_rn(__fmul2_rn(f2, uy), uv, __fmul2_rn(q, f2_nma(uy, uv, vy))),
+                       __ffma2_rn(__fmul2_rn(f2, uz), uv, __fmul2_rn(q, f2_nma(uz, uv, vz)))};
+  cv_accumulate(sh, t, g, il0, jc0, il1, jc1, true, v1);
 }
 
 // H_z w per frame with a bias, a warp (NW = 1) or a block of NW warps per (frame, tile)
 template <int NW>
-__global__ void __launch_bounds__(128) k_adj_hw(AdjDev a, CvConst k) {
+__global__ void __launch_bounds__(adj_threads(NW), adj_blocks(NW)) k_adj_hw(AdjDev a, CvConst k) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  __shared__ AdjHwShared s_sh[NW == 1 ? 4 : 1];
+  __shared__ AdjHwShared s_sh[NW == 1 ? ADJ_WARPS : 1];
   __shared__ unsigned s_bal[CV_T];
-  const int w = NW == 1 ? blockIdx.x * 4 + warp : blockIdx.x;
+  const int w = NW == 1 ? blockIdx.x * ADJ_WARPS + warp : blockIdx.x;
   if (w >= a.nf * a.n_tiles) return;
   const int f = w / a.n_tiles;
   if (a.coef[2 * f + 1] == 0.0) return;  // no bias at this frame: no Hessian term
@@ -263,14 +258,14 @@ __global__ void __launch_bounds__(128) k_adj_hw(AdjDev a, CvConst k) {
     if (cv_tile_far(t, iv, jv, xi, xj)) return;
     n_near = cv_near_list(t, sh.s_near, xi, xj);
     if (n_near == 0) return;
-    const float x6[6] = {xi.x, xi.y, xi.z, xj.x, xj.y, xj.z}, w6[6] = {wi.x, wi.y, wi.z, wj.x, wj.y, wj.z};
+    sh.s_x[lane] = make_float4(xi.x, xi.y, xi.z, 0.f);
+    sh.s_x[CV_T + lane] = make_float4(xj.x, xj.y, xj.z, 0.f);
+    sh.s_w[lane] = make_float4(wi.x, wi.y, wi.z, 0.f);
+    sh.s_w[CV_T + lane] = make_float4(wj.x, wj.y, wj.z, 0.f);
 #pragma unroll
-    for (int q = 0; q < 6; ++q) {
-      const int row = lane + (q >= 3 ? CV_T : 0), c = q % 3;
-      sh.s_x[row][c] = x6[q];
-      sh.s_w[row][c] = w6[q];
-      sh.s_ghi[row][c] = 0;
-      sh.s_glo[row][c] = 0u;
+    for (int q = 0; q < 3; ++q) {
+      sh.s_ghi[lane][q] = 0; sh.s_ghi[CV_T + lane][q] = 0;
+      sh.s_glo[lane][q] = 0; sh.s_glo[CV_T + lane][q] = 0;
     }
     __syncwarp();
   } else {
@@ -279,11 +274,14 @@ __global__ void __launch_bounds__(128) k_adj_hw(AdjDev a, CvConst k) {
     if (threadIdx.x < 2 * CV_T) {
       const int q = (warp == 0 ? t.bi : t.bj) * CV_T + lane;
       const float3 v = q < t.n_cv ? wof(q) : make_float3(0.f, 0.f, 0.f);
-      sh.s_w[threadIdx.x][0] = v.x; sh.s_w[threadIdx.x][1] = v.y; sh.s_w[threadIdx.x][2] = v.z;
+      sh.s_w[threadIdx.x] = make_float4(v.x, v.y, v.z, 0.f);
     }
     n_near = cv_near_list_block<NW>(t, sh.s_near, s_bal, sh.s_x);
   }
-  for (int p = NW == 1 ? lane : (int)threadIdx.x; p < n_near; p += NW * 32) adj_hw_pair(sh, t, k, sh.s_near[p]);
+  for (int p = NW == 1 ? lane : (int)threadIdx.x; p < n_near; p += 2 * NW * 32) {
+    const bool two = p + NW * 32 < n_near;
+    adj_hw_pairs(sh, t, k, sh.s_near[p], sh.s_near[two ? p + NW * 32 : p], two);
+  }
   if constexpr (NW == 1) __syncwarp(); else __syncthreads();
   for (int q = NW == 1 ? lane : (int)threadIdx.x; q < 2 * CV_T; q += NW * 32) {
     const int atom = (q < CV_T ? t.bi : t.bj) * CV_T + (q & (CV_T - 1));
@@ -400,7 +398,7 @@ void launch_adj_cv(const AdjInput &in, const AdjDev &a, cudaStream_t st) {
   const long long tiles = (long long)a.nf * a.n_tiles;
   if (tiles > 0) {
     if (block_form(in)) k_adj_cv<CV_BLOCK_WARPS><<<(unsigned)tiles, 32 * CV_BLOCK_WARPS, 0, st>>>(a, in.k);
-    else k_adj_cv<1><<<(unsigned)((tiles + 3) / 4), 128, 0, st>>>(a, in.k);
+    else k_adj_cv<1><<<(unsigned)((tiles + ADJ_WARPS - 1) / ADJ_WARPS), 32 * ADJ_WARPS, 0, st>>>(a, in.k);
   }
   k_adj_fin<<<a.nf, FIN_THREADS, 0, st>>>(a);
 }
@@ -412,7 +410,7 @@ void launch_adj_grad(const AdjInput &in, const AdjDev &a, double *grad, cudaStre
   cudaMemsetAsync(a.hx, 0, sizeof(long long) * 3 * na, st);
   if (tiles > 0) {
     if (block_form(in)) k_adj_hw<CV_BLOCK_WARPS><<<(unsigned)tiles, 32 * CV_BLOCK_WARPS, 0, st>>>(a, in.k);
-    else k_adj_hw<1><<<(unsigned)((tiles + 3) / 4), 128, 0, st>>>(a, in.k);
+    else k_adj_hw<1><<<(unsigned)((tiles + ADJ_WARPS - 1) / ADJ_WARPS), 32 * ADJ_WARPS, 0, st>>>(a, in.k);
   }
   k_adj_out<<<(unsigned)((na + 255) / 256), 256, 0, st>>>(a, grad);
 }

@@ -7,37 +7,81 @@
 
 namespace vp {
 
-__device__ __forceinline__ long long gsum(int hi, unsigned lo) { return (long long)hi * 16777216ll + (long long)lo; }
+// one tile of the contact-pair triangle of one configuration
+struct CvTile {
+  int n_cv, bi, bj, min_sep;
+  float L, iL, rc2_far;
+  const float2 *cn;         // the tile's C~_nat
+  long long *gx, *gy, *gz;  // the configuration's gradient sums (atom 0)
+  double *z_part;           // the tile's partial sum of z
+};
 
-// The near pair (il, jc) of a tile: its z term, and its gradient contribution
-// into the tile's shared accumulators.  One definition for the warp and the
-// block form of a tile, so both give the same bits.
-template <class SH>
-__device__ __forceinline__ ff cv_near_pair(SH &sh, const CvConst &k, const float2 *cn, float L, float iL, unsigned e) {
-  const int il = e & 31, jc = e >> 5;
-  const float3 pi = make_float3(sh.s_x[il][0], sh.s_x[il][1], sh.s_x[il][2]);
-  ff dx, dy, dz;
-  cv_delta(pi, sh.s_x[CV_T + jc][0], sh.s_x[CV_T + jc][1], sh.s_x[CV_T + jc][2], L, iL, dx, dy, dz);
-  const float2 cv2 = cn[((jc - il) & (CV_T - 1)) * CV_T + il];
-  const ff cnat = {cv2.x, cv2.y};
-  const ff r2 = ff_add(ff_add(ff_sqr(dx), ff_sqr(dy)), ff_sqr(dz));
-  const CvPair cp = cv_contact<false>(r2, k);
-  const ff h = ff_add(cp.Ct, ff_neg(cnat));
-  // dz/dx_i = -w d, dz/dx_j = +w d with d = x_j - x_i, w = 2 h C~'(r)/r
-  const float wgt = 2.0f * h.hi * cp.dCt / cp.r;
-  if (wgt != 0.0f) {
-    const long long gx = fx_from(wgt * dx.hi), gy = fx_from(wgt * dy.hi), gz = fx_from(wgt * dz.hi);
-    const long long gv[3] = {gx, gy, gz};
+// a contribution too large for the tile's accumulators (the sum is the same)
+__device__ __forceinline__ void cv_add_large(const CvTile &t, float fx, float fy, float fz, int il, int jc) {
+  const long long v[3] = {fx_from(fx), fx_from(fy), fx_from(fz)};
+  long long *const gp[3] = {t.gx, t.gy, t.gz};
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      atomicAdd(&sh.s_ghi[il][q], (int)((-gv[q]) >> 24));
-      atomicAdd(&sh.s_glo[il][q], (unsigned)((-gv[q]) & 0xffffff));
-      atomicAdd(&sh.s_ghi[CV_T + jc][q], (int)(gv[q] >> 24));
-      atomicAdd(&sh.s_glo[CV_T + jc][q], (unsigned)(gv[q] & 0xffffff));
+  for (int c = 0; c < 3; ++c) {
+    red_add(gp[c] + t.bi * CV_T + il, (long long)(0ull - (unsigned long long)v[c]));
+    red_add(gp[c] + t.bj * CV_T + jc, v[c]);
+  }
+}
+
+// The two pairs' contributions f (per 1/2^32 after rounding, as fx_from rounds
+// them) into the tile's accumulators, or straight to memory when one is too
+// large for the split; pair 1 only when v1.  |f| < 512: f 2^(32 - CV_SPLIT) +
+// 1.5 2^23 is rounded to the high part, what is left of f 2^32 is exact and
+// rounds to the low one -- no 64-bit conversion, which the FP64 pipe does.
+template <class SH>
+__device__ __forceinline__ void cv_accumulate(SH &sh, const CvTile &t, const float2 (&f)[3], int il0, int jc0, int il1,
+                                              int jc1, bool v0, bool v1) {
+  const float big0 = fmaxf(fmaxf(fabsf(f[0].x), fabsf(f[1].x)), fabsf(f[2].x));
+  const float big1 = fmaxf(fmaxf(fabsf(f[0].y), fabsf(f[1].y)), fabsf(f[2].y));
+  if (v0 && !(big0 < 512.0f)) { cv_add_large(t, f[0].x, f[1].x, f[2].x, il0, jc0); v0 = false; }
+  if (v1 && !(big1 < 512.0f)) { cv_add_large(t, f[0].y, f[1].y, f[2].y, il1, jc1); v1 = false; }
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const float2 m = f2_all(12582912.0f);
+    const float2 th = __ffma2_rn(f[q], f2_all(4294967296.0f / (1 << CV_SPLIT)), m);
+    const float2 tl = __fadd2_rn(__ffma2_rn(f2_sub(th, m), f2_all(-(float)(1 << CV_SPLIT)), __fmul2_rn(f[q], f2_all(4294967296.0f))), m);
+    if (v0) {
+      const int hi = __float_as_int(th.x) - 0x4b400000, lo = __float_as_int(tl.x) - 0x4b400000;
+      atomicAdd(&sh.s_ghi[il0][q], hi);
+      atomicAdd(&sh.s_glo[il0][q], lo);
+      atomicAdd(&sh.s_ghi[CV_T + jc0][q], hi);
+      atomicAdd(&sh.s_glo[CV_T + jc0][q], lo);
+    }
+    if (v1) {
+      const int hi = __float_as_int(th.y) - 0x4b400000, lo = __float_as_int(tl.y) - 0x4b400000;
+      atomicAdd(&sh.s_ghi[il1][q], hi);
+      atomicAdd(&sh.s_glo[il1][q], lo);
+      atomicAdd(&sh.s_ghi[CV_T + jc1][q], hi);
+      atomicAdd(&sh.s_glo[CV_T + jc1][q], lo);
     }
   }
+}
+
+// The near pairs e0 and (when v1) e1 of a tile, entries il | jc << 5: their z
+// terms, and their gradient contributions into the tile's accumulators.  One
+// definition for the warp and the block form of a tile, so both give the same
+// bits.
+template <class SH>
+__device__ __forceinline__ ff2 cv_near_pairs(SH &sh, const CvConst &k, const CvTile &t, unsigned e0, unsigned e1, bool v1) {
+  const int il0 = e0 & 31, jc0 = e0 >> 5, il1 = e1 & 31, jc1 = e1 >> 5;
+  ff2 dx, dy, dz;
+  cv_delta2(sh.s_x[il0], sh.s_x[il1], sh.s_x[CV_T + jc0], sh.s_x[CV_T + jc1], t.L, t.iL, dx, dy, dz);
+  const float2 n0 = t.cn[((jc0 - il0) & (CV_T - 1)) * CV_T + il0], n1 = t.cn[((jc1 - il1) & (CV_T - 1)) * CV_T + il1];
+  const ff2 cnat = {make_float2(n0.x, n1.x), make_float2(n0.y, n1.y)};
+  const ff2 r2 = ff2_add(ff2_add(ff2_sqr(dx), ff2_sqr(dy)), ff2_sqr(dz));
+  const CvPair2 cp = cv_contact2<false>(r2, k);
+  const float2 h = ff2_sub(cp.Ct, cnat).hi;
+  // dz/dx_i = -w d, dz/dx_j = +w d with d = x_j - x_i, w = 2 h C~'(r)/r
+  const float2 w = f2_div(__fmul2_rn(__fadd2_rn(h, h), cp.dCt), cp.r, f2_rcp(cp.r));
+  const float2 g[3] = {__fmul2_rn(w, dx.hi), __fmul2_rn(w, dy.hi), __fmul2_rn(w, dz.hi)};
+  // coincident atoms (w not a number) pull nowhere
+  cv_accumulate(sh, t, g, il0, jc0, il1, jc1, w.x == w.x, v1 && w.y == w.y);
   // z term: C~ (C~ - 2 C~_nat) = (C~ - C~_nat)^2 - C~_nat^2
-  return ff_mul(cp.Ct, ff_add(cp.Ct, ff{-2.0f * cnat.hi, -2.0f * cnat.lo}));  // doubling is exact
+  return ff2_mul(cp.Ct, ff2_sub(cp.Ct, ff2{__fadd2_rn(cnat.hi, cnat.hi), __fadd2_rn(cnat.lo, cnat.lo)}));
 }
 
 // whether a pair at the (unimaged) FP32 difference (dx, dy, dz) is closer than the contact cut-off
@@ -51,19 +95,14 @@ __device__ __forceinline__ bool cv_is_near(float dx, float dy, float dz, float L
 // the accumulated gradient of atom a (0..63) of the tile, into the sums at gx, gy, gz
 template <class SH>
 __device__ __forceinline__ void cv_flush_atom(SH &sh, int a, long long *gx, long long *gy, long long *gz) {
-  const long long a0 = gsum(sh.s_ghi[a][0], sh.s_glo[a][0]), a1 = gsum(sh.s_ghi[a][1], sh.s_glo[a][1]),
-                  a2 = gsum(sh.s_ghi[a][2], sh.s_glo[a][2]);
-  if (a0 | a1 | a2) { red_add(gx, a0); red_add(gy, a1); red_add(gz, a2); }
+  long long g[3];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    g[q] = (long long)sh.s_ghi[a][q] * (1ll << CV_SPLIT) + (long long)sh.s_glo[a][q];
+    if (a < CV_T) g[q] = -g[q];
+  }
+  if (g[0] | g[1] | g[2]) { red_add(gx, g[0]); red_add(gy, g[1]); red_add(gz, g[2]); }
 }
-
-// one tile of the contact-pair triangle of one configuration
-struct CvTile {
-  int n_cv, bi, bj, min_sep;
-  float L, iL, rc2_far;
-  const float2 *cn;         // the tile's C~_nat
-  long long *gx, *gy, *gz;  // the configuration's gradient sums (atom 0)
-  double *z_part;           // the tile's partial sum of z
-};
 
 // Whether no pair of the tile can be closer than the contact cut-off: the
 // periodic gap of the two 32-atom blocks' bounding boxes (lane l holds atom l
@@ -109,19 +148,19 @@ __device__ __forceinline__ int cv_near_list(const CvTile &t, unsigned short *s_n
 // atoms of both blocks in s_x; every thread of the block calls).
 template <int NW>
 __device__ __forceinline__ int cv_near_list_block(const CvTile &t, unsigned short *s_near, unsigned *s_bal,
-                                                  const float (*s_x)[3]) {
+                                                  const float4 *s_x) {
   constexpr int KW = CV_T / NW;  // rotations per warp
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int i = t.bi * CV_T + lane;
-  const float3 xi = make_float3(s_x[lane][0], s_x[lane][1], s_x[lane][2]);
+  const float4 xi = s_x[lane];
   unsigned bal[KW];
 #pragma unroll
   for (int q = 0; q < KW; ++q) {
     const int jc = (lane + warp * KW + q) & (CV_T - 1);
     const int j = t.bj * CV_T + jc;
-    const float *x = s_x[CV_T + jc];
+    const float4 x = s_x[CV_T + jc];
     const bool near = i < t.n_cv && j < t.n_cv && j - i > t.min_sep &&
-                      cv_is_near(x[0] - xi.x, x[1] - xi.y, x[2] - xi.z, t.L, t.iL, t.rc2_far);
+                      cv_is_near(x.x - xi.x, x.y - xi.y, x.z - xi.z, t.L, t.iL, t.rc2_far);
     bal[q] = __ballot_sync(0xffffffffu, near);
     if (lane == 0) s_bal[warp * KW + q] = bal[q];
   }
@@ -157,19 +196,23 @@ __device__ __forceinline__ void cv_tile(const CvTile &t, const CvConst &k, CvWar
     if (lane == 0) *t.z_part = 0.0;
     return;
   }
-  sh.s_x[lane][0] = xi.x; sh.s_x[lane][1] = xi.y; sh.s_x[lane][2] = xi.z;
-  sh.s_x[CV_T + lane][0] = xj.x; sh.s_x[CV_T + lane][1] = xj.y; sh.s_x[CV_T + lane][2] = xj.z;
+  sh.s_x[lane] = make_float4(xi.x, xi.y, xi.z, 0.f);
+  sh.s_x[CV_T + lane] = make_float4(xj.x, xj.y, xj.z, 0.f);
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
     sh.s_ghi[lane][q] = 0; sh.s_ghi[CV_T + lane][q] = 0;
-    sh.s_glo[lane][q] = 0u; sh.s_glo[CV_T + lane][q] = 0u;
+    sh.s_glo[lane][q] = 0; sh.s_glo[CV_T + lane][q] = 0;
   }
   const int n_near = cv_near_list(t, sh.s_near, xi, xj);
   __syncwarp();
   // the near pairs, densely
   ff zacc = {0.f, 0.f};
-  for (int base = 0; base < n_near; base += 32)
-    if (base + lane < n_near) zacc = ff_add(zacc, cv_near_pair(sh, k, t.cn, t.L, t.iL, sh.s_near[base + lane]));
+  for (int p = lane; p < n_near; p += 64) {
+    const bool two = p + 32 < n_near;
+    const ff2 v = cv_near_pairs(sh, k, t, sh.s_near[p], sh.s_near[two ? p + 32 : p], two);
+    zacc = ff_add(zacc, ff{v.hi.x, v.lo.x});
+    if (two) zacc = ff_add(zacc, ff{v.hi.y, v.lo.y});
+  }
   __syncwarp();
   if (n_near > 0) {
     if (iv) cv_flush_atom(sh, lane, t.gx + i, t.gy + i, t.gz + i);
@@ -188,9 +231,9 @@ __device__ __forceinline__ void cv_tile(const CvTile &t, const CvConst &k, CvWar
 // order too: z and the gradient are the same bit for bit.
 struct CvBlockShared {
   unsigned short s_near[CV_T * CV_T];
-  float s_x[2 * CV_T][3];
+  float4 s_x[2 * CV_T];
   int s_ghi[2 * CV_T][3];
-  unsigned s_glo[2 * CV_T][3];
+  int s_glo[2 * CV_T][3];
   unsigned s_bal[CV_T];
   float2 s_term[CV_T * CV_T];
 };
@@ -204,16 +247,16 @@ __device__ __forceinline__ bool cv_block_begin(const CvTile &t, SH &sh, POS pos)
     const int a = (warp == 0 ? t.bi : t.bj) * CV_T + lane;
     float3 q = make_float3(0.f, 0.f, 0.f);
     if (a < t.n_cv) q = pos(a);
-    sh.s_x[threadIdx.x][0] = q.x; sh.s_x[threadIdx.x][1] = q.y; sh.s_x[threadIdx.x][2] = q.z;
+    sh.s_x[threadIdx.x] = make_float4(q.x, q.y, q.z, 0.f);
   }
   for (int q = threadIdx.x; q < 2 * CV_T * 3; q += NW * 32) {
     (&sh.s_ghi[0][0])[q] = 0;
-    (&sh.s_glo[0][0])[q] = 0u;
+    (&sh.s_glo[0][0])[q] = 0;
   }
   __syncthreads();
   return cv_tile_far(t, t.bi * CV_T + lane < t.n_cv, t.bj * CV_T + lane < t.n_cv,
-                     make_float3(sh.s_x[lane][0], sh.s_x[lane][1], sh.s_x[lane][2]),
-                     make_float3(sh.s_x[CV_T + lane][0], sh.s_x[CV_T + lane][1], sh.s_x[CV_T + lane][2]));
+                     make_float3(sh.s_x[lane].x, sh.s_x[lane].y, sh.s_x[lane].z),
+                     make_float3(sh.s_x[CV_T + lane].x, sh.s_x[CV_T + lane].y, sh.s_x[CV_T + lane].z));
 }
 
 template <int NW, class POS>
@@ -224,9 +267,12 @@ __device__ __forceinline__ void cv_tile_block(const CvTile &t, const CvConst &k,
     return;
   }
   const int n_near = cv_near_list_block<NW>(t, sh.s_near, sh.s_bal, sh.s_x);
-  for (int p = threadIdx.x; p < n_near; p += NW * 32) {
-    const ff v = cv_near_pair(sh, k, t.cn, t.L, t.iL, sh.s_near[p]);
-    sh.s_term[p] = make_float2(v.hi, v.lo);
+  for (int p = threadIdx.x; p < n_near; p += 2 * NW * 32) {
+    const int p1 = p + NW * 32;
+    const bool two = p1 < n_near;
+    const ff2 v = cv_near_pairs(sh, k, t, sh.s_near[p], sh.s_near[two ? p1 : p], two);
+    sh.s_term[p] = make_float2(v.hi.x, v.lo.x);
+    if (two) sh.s_term[p1] = make_float2(v.hi.y, v.lo.y);
   }
   __syncthreads();
   if (warp == 0) {

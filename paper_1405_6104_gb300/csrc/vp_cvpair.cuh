@@ -18,85 +18,177 @@ __device__ __forceinline__ CvConst cv_const(const SimConst &c) {
                  c.cv_rs2, c.cv_rc2_far};
 }
 
-__device__ __forceinline__ ff contact_ff(ff s) {
-  ff s2 = ff_sqr(s);
-  ff s3 = ff_mul(s2, s);
-  ff s4 = ff_sqr(s2);
-  ff N = ff_add(ff_add_f(s, 1.0f), s2);
-  ff D = ff_add(ff_add(N, s3), s4);
-  return ff_div(N, D);
+// Two near pairs per lane, on the packed FP32 instructions (two operations per
+// issue slot): the tile kernels are bound by instruction issue (79% of the
+// slots, with one pair per lane), most of it this arithmetic.
+__device__ __forceinline__ float2 f2_all(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 f2_neg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 f2_sub(float2 a, float2 b) { return __ffma2_rn(b, f2_all(-1.0f), a); }
+__device__ __forceinline__ float2 f2_nma(float2 a, float2 b, float2 c) { return __ffma2_rn(f2_neg(a), b, c); }  // c - a b
+
+struct ff2 { float2 hi, lo; };
+__device__ __forceinline__ ff2 ff2_all(ff a) { return {f2_all(a.hi), f2_all(a.lo)}; }
+__device__ __forceinline__ ff2 ff2_fast_two_sum(float2 a, float2 b) {
+  const float2 s = __fadd2_rn(a, b);
+  return {s, f2_sub(b, f2_sub(s, a))};
+}
+__device__ __forceinline__ ff2 ff2_two_sum(float2 a, float2 b) {
+  const float2 s = __fadd2_rn(a, b), bb = f2_sub(s, a);
+  return {s, __fadd2_rn(f2_sub(a, f2_sub(s, bb)), f2_sub(b, bb))};
+}
+__device__ __forceinline__ ff2 ff2_two_diff(float2 a, float2 b) {
+  const float2 s = f2_sub(a, b), bb = f2_sub(s, a);
+  return {s, f2_sub(f2_sub(a, f2_sub(s, bb)), __fadd2_rn(b, bb))};
+}
+__device__ __forceinline__ ff2 ff2_add(ff2 x, ff2 y) {
+  const ff2 s = ff2_two_sum(x.hi, y.hi);
+  return ff2_fast_two_sum(s.hi, __fadd2_rn(s.lo, __fadd2_rn(x.lo, y.lo)));
+}
+__device__ __forceinline__ ff2 ff2_sub(ff2 x, ff2 y) {
+  const ff2 s = ff2_two_diff(x.hi, y.hi);
+  return ff2_fast_two_sum(s.hi, __fadd2_rn(s.lo, f2_sub(x.lo, y.lo)));
+}
+__device__ __forceinline__ ff2 ff2_add_f(ff2 x, float2 y) {
+  const ff2 s = ff2_two_sum(x.hi, y);
+  return ff2_fast_two_sum(s.hi, __fadd2_rn(s.lo, x.lo));
+}
+__device__ __forceinline__ ff2 ff2_mul(ff2 x, ff2 y) {
+  const float2 p = __fmul2_rn(x.hi, y.hi);
+  const float2 e = __ffma2_rn(x.hi, y.hi, f2_neg(p));
+  return ff2_fast_two_sum(p, __ffma2_rn(x.hi, y.lo, __ffma2_rn(x.lo, y.hi, e)));
+}
+__device__ __forceinline__ ff2 ff2_mul_f(ff2 x, float2 y) {
+  const float2 p = __fmul2_rn(x.hi, y);
+  const float2 e = __ffma2_rn(x.hi, y, f2_neg(p));
+  return ff2_fast_two_sum(p, __ffma2_rn(x.lo, y, e));
+}
+__device__ __forceinline__ ff2 ff2_sqr(ff2 x) {
+  const float2 p = __fmul2_rn(x.hi, x.hi);
+  const float2 e = __ffma2_rn(x.hi, x.hi, f2_neg(p));
+  return ff2_fast_two_sum(p, __ffma2_rn(__fadd2_rn(x.hi, x.hi), x.lo, e));
+}
+__device__ __forceinline__ ff2 ff2_div(ff2 x, ff2 y) {
+  const float2 q = make_float2(__fdividef(x.hi.x, y.hi.x), __fdividef(x.hi.y, y.hi.y));
+  const ff2 r = ff2_sub(x, ff2_mul_f(y, q));
+  return ff2_fast_two_sum(q, make_float2(__fdividef(r.hi.x, y.hi.x), __fdividef(r.hi.y, y.hi.y)));
 }
 
-__device__ __forceinline__ float dcontact_ds(float s) {
-  float N = 1.0f + s + s * s;
-  float D = N + s * s * s + s * s * s * s;
-  float dN = 1.0f + 2.0f * s;
-  float dD = dN + 3.0f * s * s + 4.0f * s * s * s;
-  return (dN * D - N * dD) / (D * D);
+// Correctly rounded quotients and roots by Markstein's final step (IBM J. Res.
+// Dev. 34, 1990): a Newton step on the hardware's approximation gives the
+// correctly rounded reciprocal (every one of the 2^23 significands was
+// compared), and one on the quotient's (root's) remainder the correctly
+// rounded result.  For operands and results away from the range's ends.
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float rsqrt_approx(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float2 f2_rcp(float2 b) {
+  const float2 r = make_float2(rcp_approx(b.x), rcp_approx(b.y));
+  return __ffma2_rn(r, f2_nma(b, r, f2_all(1.0f)), r);
+}
+__device__ __forceinline__ float2 f2_div(float2 a, float2 b, float2 rb) {  // rb = f2_rcp(b)
+  const float2 q = __fmul2_rn(a, rb);
+  return __ffma2_rn(f2_nma(b, q, a), rb, q);
+}
+__device__ __forceinline__ float2 f2_sqrt(float2 x) {
+  const float2 y = make_float2(rsqrt_approx(x.x), rsqrt_approx(x.y));
+  const float2 g = __fmul2_rn(x, y), h = __fmul2_rn(y, f2_all(0.5f));
+  return __ffma2_rn(f2_nma(g, g, x), h, g);
 }
 
-// d^2 C / ds^2 of the rational contact function
-__device__ __forceinline__ float d2contact_ds2(float s) {
-  float N = 1.0f + s + s * s, D = N + s * s * s + s * s * s * s;
-  float N1 = 1.0f + 2.0f * s, D1 = N1 + 3.0f * s * s + 4.0f * s * s * s;
-  float D2 = 2.0f + 6.0f * s + 12.0f * s * s;
-  return ((2.0f * D - N * D2) * D - 2.0f * D1 * (N1 * D - N * D1)) / (D * D * D);
-}
-
-struct CvPair {
-  ff Ct;       // C~(r)
-  float dCt;   // dC~/dr
-  float d2Ct;  // d^2 C~/dr^2 (only with SECOND)
-  float r;
+struct CvPair2 {
+  ff2 Ct;
+  float2 dCt, d2Ct, r;
 };
 
-// C~, C~' (and C~'' when SECOND) at the squared distance r2 (float-float)
 template <bool SECOND>
-__device__ __forceinline__ CvPair cv_contact(ff r2, const CvConst &k) {
-  CvPair o;
-  const ff s = ff_mul(r2, k.inv_r0sq);
-  o.Ct = contact_ff(s);
-  o.r = sqrtf(r2.hi);
-  const float ds = 2.0f * o.r * k.inv_r0sq.hi;  // ds/dr
-  const float Cs = dcontact_ds(s.hi);
-  o.dCt = Cs * ds;
-  o.d2Ct = SECOND ? d2contact_ds2(s.hi) * ds * ds + Cs * 2.0f * k.inv_r0sq.hi : 0.0f;
-  if (r2.hi > k.rs2) {
-    const ff r = ff_sqrt(r2);
-    const ff x = ff_mul(ff_add(r, ff_neg(k.rs)), k.inv_w);
-    if (x.hi >= 1.0f) {
-      o.Ct = {0.f, 0.f};
-      o.dCt = 0.f;
-      o.d2Ct = 0.f;
-    } else {
-      // S = 1 - x^3 (10 - 15 x + 6 x^2)
-      ff p = ff_add_f(ff_mul_f(x, 6.0f), -15.0f);
-      p = ff_add_f(ff_mul(p, x), 10.0f);
-      const ff x3 = ff_mul(ff_sqr(x), x);
-      const ff S = ff_add_f(ff_neg(ff_mul(x3, p)), 1.0f);
-      const float xf = x.hi, iw = k.inv_w.hi;
-      const float S1 = -30.0f * xf * xf * (1.0f - xf) * (1.0f - xf) * iw;
-      if (SECOND) {
-        const float S2 = (-60.0f * xf + 180.0f * xf * xf - 120.0f * xf * xf * xf) * iw * iw;
-        o.d2Ct = o.d2Ct * S.hi + 2.0f * o.dCt * S1 + o.Ct.hi * S2;
-      }
-      o.dCt = o.dCt * S.hi + o.Ct.hi * S1;
-      o.Ct = ff_mul(o.Ct, S);
+__device__ __forceinline__ CvPair2 cv_contact2(ff2 r2, const CvConst &k) {
+  CvPair2 o;
+  const ff2 s = ff2_mul(r2, ff2_all(k.inv_r0sq));
+  {
+    const ff2 s2 = ff2_sqr(s), s3 = ff2_mul(s2, s), s4 = ff2_sqr(s2);
+    const ff2 N = ff2_add(ff2_add_f(s, f2_all(1.0f)), s2);
+    o.Ct = ff2_div(N, ff2_add(ff2_add(N, s3), s4));
+  }
+  o.r = f2_sqrt(r2.hi);
+  const float2 ds = __fmul2_rn(__fadd2_rn(o.r, o.r), f2_all(k.inv_r0sq.hi));
+  // C'(s), C''(s)
+  const float2 t = s.hi, t2 = __fmul2_rn(t, t), t3 = __fmul2_rn(t2, t);
+  const float2 N = __fadd2_rn(__fadd2_rn(t, f2_all(1.0f)), t2);
+  const float2 D = __ffma2_rn(t3, t, __fadd2_rn(N, t3));
+  const float2 N1 = __ffma2_rn(t, f2_all(2.0f), f2_all(1.0f));
+  const float2 D1 = __ffma2_rn(__fmul2_rn(__fmul2_rn(t, f2_all(4.0f)), t), t, __ffma2_rn(__fmul2_rn(t, f2_all(3.0f)), t, N1));
+  const float2 W = __ffma2_rn(N1, D, f2_neg(__fmul2_rn(N, D1))), DD = __fmul2_rn(D, D);
+  const float2 Cs = f2_div(W, DD, f2_rcp(DD));
+  o.dCt = __fmul2_rn(Cs, ds);
+  if (SECOND) {
+    const float2 D2 = __ffma2_rn(__fmul2_rn(t, f2_all(12.0f)), t, __ffma2_rn(t, f2_all(6.0f), f2_all(2.0f)));
+    const float2 A1 = f2_nma(N, D2, __fadd2_rn(D, D));
+    const float2 num = __ffma2_rn(A1, D, f2_neg(__fmul2_rn(__fadd2_rn(D1, D1), W)));
+    const float2 DDD = __fmul2_rn(DD, D);
+    const float2 d2 = f2_div(num, DDD, f2_rcp(DDD));
+    o.d2Ct = __ffma2_rn(__fadd2_rn(Cs, Cs), f2_all(k.inv_r0sq.hi), __fmul2_rn(__fmul2_rn(d2, ds), ds));
+  }
+  const bool sx = r2.hi.x > k.rs2, sy = r2.hi.y > k.rs2;
+  if (sx || sy) {
+    // ff_sqrt, from the root already there
+    const float2 y = o.r, yy = __fmul2_rn(y, y);
+    const ff2 rem = ff2_sub(r2, ff2{yy, __ffma2_rn(y, y, f2_neg(yy))});
+    const float2 y2 = __fadd2_rn(y, y);
+    const ff2 r = ff2_fast_two_sum(y, make_float2(__fdividef(rem.hi.x, y2.x), __fdividef(rem.hi.y, y2.y)));
+    const ff2 x = ff2_mul(ff2_add(r, ff2_all(ff_neg(k.rs))), ff2_all(k.inv_w));
+    ff2 p = ff2_add_f(ff2_mul_f(x, f2_all(6.0f)), f2_all(-15.0f));
+    p = ff2_add_f(ff2_mul(p, x), f2_all(10.0f));
+    const ff2 m = ff2_mul(ff2_mul(ff2_sqr(x), x), p);
+    // S = 1 - m
+    const float2 one = f2_all(1.0f), sh = f2_sub(one, m.hi), bb = __fadd2_rn(sh, m.hi);
+    const float2 se = f2_sub(f2_sub(one, bb), __fadd2_rn(m.hi, f2_sub(sh, bb)));
+    const ff2 S = ff2_fast_two_sum(sh, f2_sub(se, m.lo));
+    const float2 xf = x.hi, y1 = f2_sub(one, xf);
+    const float2 S1 = __fmul2_rn(
+        __fmul2_rn(__fmul2_rn(__fmul2_rn(__fmul2_rn(xf, f2_all(-30.0f)), xf), y1), y1), f2_all(k.inv_w.hi));
+    const float2 c1 = SECOND ? __ffma2_rn(o.Ct.hi, S1, __fmul2_rn(o.dCt, S.hi))
+                             : __ffma2_rn(o.dCt, S.hi, __fmul2_rn(o.Ct.hi, S1));
+    const ff2 cs = ff2_mul(o.Ct, S);
+    const bool zx = x.hi.x >= 1.0f, zy = x.hi.y >= 1.0f;
+    if (SECOND) {
+      const float2 iw = f2_all(k.inv_w.hi);
+      const float2 q = __ffma2_rn(__fmul2_rn(xf, f2_all(180.0f)), xf, __fmul2_rn(xf, f2_all(-60.0f)));
+      const float2 S2 = __fmul2_rn(
+          __fmul2_rn(f2_nma(__fmul2_rn(__fmul2_rn(xf, f2_all(120.0f)), xf), xf, q), iw), iw);
+      const float2 c2 = __ffma2_rn(o.Ct.hi, S2, __ffma2_rn(__fadd2_rn(o.dCt, o.dCt), S1, __fmul2_rn(o.d2Ct, S.hi)));
+      if (sx) o.d2Ct.x = zx ? 0.f : c2.x;
+      if (sy) o.d2Ct.y = zy ? 0.f : c2.y;
     }
+    if (sx) { o.dCt.x = zx ? 0.f : c1.x; o.Ct.hi.x = zx ? 0.f : cs.hi.x; o.Ct.lo.x = zx ? 0.f : cs.lo.x; }
+    if (sy) { o.dCt.y = zy ? 0.f : c1.y; o.Ct.hi.y = zy ? 0.f : cs.hi.y; o.Ct.lo.y = zy ? 0.f : cs.lo.y; }
   }
   return o;
 }
 
-// exact minimum-image difference x_j - x_i as float-float
-__device__ __forceinline__ void cv_delta(float3 xi, float xjx, float xjy, float xjz, float L, float iL, ff &dx, ff &dy,
-                                         ff &dz) {
-  dx = ff_diff(xjx, xi.x);
-  dy = ff_diff(xjy, xi.y);
-  dz = ff_diff(xjz, xi.z);
-  const float nx = rintf(dx.hi * iL), ny = rintf(dy.hi * iL), nz = rintf(dz.hi * iL);
-  if (nx != 0.f) dx = ff_add_f(dx, -L * nx);
-  if (ny != 0.f) dy = ff_add_f(dy, -L * ny);
-  if (nz != 0.f) dz = ff_add_f(dz, -L * nz);
+// exact minimum-image differences x_j - x_i as float-float
+__device__ __forceinline__ void cv_delta2(float4 xi0, float4 xi1, float4 xj0, float4 xj1, float L, float iL, ff2 &dx,
+                                          ff2 &dy, ff2 &dz) {
+  dx = ff2_two_diff(make_float2(xj0.x, xj1.x), make_float2(xi0.x, xi1.x));
+  dy = ff2_two_diff(make_float2(xj0.y, xj1.y), make_float2(xi0.y, xi1.y));
+  dz = ff2_two_diff(make_float2(xj0.z, xj1.z), make_float2(xi0.z, xi1.z));
+  // adding 1.5 2^23 and taking it away rounds to whole numbers (an image
+  // number of 2^22 would leave FP32 positions without a digit below the box)
+  const float2 il = f2_all(iL), m = f2_all(12582912.0f);
+  const float2 nx = f2_sub(__fadd2_rn(__fmul2_rn(dx.hi, il), m), m), ny = f2_sub(__fadd2_rn(__fmul2_rn(dy.hi, il), m), m),
+               nz = f2_sub(__fadd2_rn(__fmul2_rn(dz.hi, il), m), m);
+  if (nx.x != 0.f || nx.y != 0.f || ny.x != 0.f || ny.y != 0.f || nz.x != 0.f || nz.y != 0.f) {
+    const float2 l = f2_all(-L);
+    dx = ff2_add_f(dx, __fmul2_rn(l, nx));
+    dy = ff2_add_f(dy, __fmul2_rn(l, ny));
+    dz = ff2_add_f(dz, __fmul2_rn(l, nz));
+  }
 }
 
 }  // namespace vp

@@ -114,15 +114,18 @@ __device__ __forceinline__ void decide_rebuilds(const Dev &d, const SimConst &c,
 enum UpdateMode { UPD_DRIFT = 0, UPD_FINAL = 1 };
 
 // shared memory of one warp's reaction-coordinate tile
+constexpr int CV_SPLIT = 20;
 struct CvWarpShared {
   unsigned short s_near[CV_T * CV_T];
-  float s_x[2 * CV_T][3];
-  // gradient of the tile's 64 atoms: each fixed-point contribution c splits
-  // into c >> 24 (signed) and its low 24 bits, summed in 32-bit shared
+  float4 s_x[2 * CV_T];
+  // gradient of the tile's 64 atoms: each 64-bit fixed-point contribution is
+  // hi 2^CV_SPLIT + lo with both parts signed 32-bit, added up by 32-bit shared
   // atomics (native, unlike 64-bit ones); at most 32 contributions per entry
-  // keep both sums far from overflow, and (hi << 24) + lo is the exact sum
+  // keep both sums far from overflow, and the two give the exact sum.  A pair
+  // adds the same parts to both atoms; the rows of the i block are negated in
+  // the end.
   int s_ghi[2 * CV_T][3];
-  unsigned s_glo[2 * CV_T][3];
+  int s_glo[2 * CV_T][3];
 };
 constexpr int CV_BLOCK_WARPS = 4;  // warps per tile of the block form
 constexpr int CVFIN_THREADS = 1024;  // the finaliser's reduction width (virtual threads)

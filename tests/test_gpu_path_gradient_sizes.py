@@ -1,10 +1,11 @@
 """Sizes at which the kernels of the path gradient can go wrong: the scan of
 the coefficients at the edges of its warps and of its chunks of frames, and
 the tile kernels in their two forms (a block or a warp per tile), which must
-agree bit for bit."""
+agree bit for bit; contacts too steep for the tiles' 32-bit accumulators."""
 import numpy as np
 import pytest
 
+import oracle as O
 from paper_1405_6104_gb300 import binding as B
 from paper_1405_6104_gb300 import systems as S
 
@@ -63,10 +64,33 @@ def test_tiles_by_a_block_match_tiles_by_a_warp(n_solute):
     frames = np.stack([base * f for f in (0.4, 1.0, 2.5)]) + 0.01 * rng.normal(size=(3, n_solute, 3))
     coef = rng.normal(size=(3, 2))
     tiles = ((n_solute + 31) // 32) * ((n_solute + 31) // 32 + 1) // 2
-    reps = 16 * 160 // (3 * tiles) + 2
+    reps = 128 * 160 // (3 * tiles) + 2  # beyond 128 tiles per multiprocessor
     with B.TrialBatch(s, p, [1]) as b:
         _, z, g = B.phi_frames_adjoint(b.h, 0, frames, coef)
         _, zz, gg = B.phi_frames_adjoint(b.h, 0, np.concatenate([frames] * reps), np.concatenate([coef] * reps))
     assert np.abs(g).max() > 0.0
-    for k in range(reps):
-        assert np.array_equal(zz[3 * k:3 * k + 3], z) and np.array_equal(gg[3 * k:3 * k + 3], g)
+    assert (zz.reshape(reps, 3) == z).all() and (gg.reshape(reps, *g.shape) == g).all()
+
+
+@pytest.mark.parametrize("r0", [1e-3, 0.05])
+def test_steep_contacts(r0):
+    """Contacts so steep that a pair's gradient and Hessian terms pass the
+    range of the tiles' 32-bit accumulators, against the FP64 oracle; the
+    bounds are those of ordinary contacts (FP32 derivatives of C~).  r0 = 1e-3
+    nm: gradients of 1e3, checked through Phi = sum a^2 |grad z|^2 only, as the
+    Hessian products (1e10) leave the range +-2^31 of the 64-bit sums; r0 =
+    0.05 nm: Hessian products of 1e5."""
+    s, p = S.tiny_chain(0)
+    p.cv_r0 = r0
+    rng = np.random.default_rng(4)
+    frames = s.native_pos * np.array([1.0, 0.02, 0.01, 0.004])[:, None, None] * (r0 / 0.01)
+    frames = (frames + 0.3 * r0 * rng.normal(size=frames.shape)).astype(np.float32).astype(np.float64)
+    with B.TrialBatch(s, p, [1]) as b:
+        phi, z, G = B.phi_frames_adjoint(b.h, 0, frames)
+    phi_ref, G_ref = O.phi_frames_grad(s, p, frames)
+    _, z_ref, _, _ = O.phi_frames(s, p, frames)
+    assert phi_ref > 0
+    assert phi == pytest.approx(phi_ref, rel=1e-5)
+    assert np.allclose(z, z_ref, rtol=1e-11, atol=1e-11)
+    if r0 > 1e-3:
+        assert np.linalg.norm(G - G_ref) < 1e-4 * np.linalg.norm(G_ref)
