@@ -19,6 +19,8 @@ __device__ __forceinline__ float3 min_disp(float4 self, float4 other, float L, f
 // of a masked pair
 constexpr int PF_WARPS = 4;
 constexpr float MASK_PEN = 1.0e30f;
+// row of an i-force component's 32 partial sums: 16-byte loads without bank conflicts
+constexpr int RED_STRIDE = 36;
 
 // the energies' tables of a warp: {c12, c12', c6, c6'} (over r^12 and r^6) and the
 // potential at the cut-off per i-atom pair and type
@@ -36,7 +38,7 @@ struct PairF2Shared : PairEnergyTables<NW, ENERGY> {
   float4 s_c4[NW][CL / 2][SMALL_TYPES];
   float4 s_sh[NW][64];
   float4 s_ip[NW][CL / 2][2];
-  float s_red[NW][3 * CL * 33];
+  alignas(16) float s_red[NW][3 * CL * RED_STRIDE];
 };
 
 // The forces of one i-cluster I by the calling warp (packed arithmetic): one
@@ -46,14 +48,18 @@ struct PairF2Shared : PairEnergyTables<NW, ENERGY> {
 // evaluated, interleaves the two groups' arithmetic (two independent chains
 // per warp) and reads each i-atom pair from shared memory once for both: 96
 // registers, 20 warps per SM, and still faster at every batch size (64 x
-// 11 040 atoms 378 us against 419 with U = 1 and 24 warps; one trial 13
-// against 20 us; U = 3 and 4, or U = 2 without the early loads, are slower).
+// 11 040 atoms 371 us against 419 with U = 1 and 24 warps; one trial 13
+// against 20 us; U = 3 and 4, U = 2 without the early loads, or two iterations
+// unrolled (456 us: too much code for the instruction cache) are slower).  An
+// odd last group is taken by itself (an idle second one and the wider loads of
+// the i-force sums were 2.7% of the time).
 // Every accumulator takes its terms in the order of the groups either way:
 // the same forces bit for bit.
 // ENERGY (U = 1): the Lennard-Jones and reaction-field energies too, each lane
 // adding its pairs' in the order of the entries and i-atoms.
 template <int U, int NW, bool ENERGY = false>
 __device__ __forceinline__ void pair_cluster_f2(const Dev &d, const SimConst &c, PairF2Shared<NW, ENERGY> &sh, int I) {
+  static_assert(U <= 2, "an odd last group is the only remainder taken");
   static_assert(!ENERGY || U == 1, "the energies' sums take one group at a time");
   constexpr int TS = SMALL_TYPES;
   auto &s_c4 = sh.s_c4;
@@ -295,7 +301,8 @@ __device__ __forceinline__ void pair_cluster_f2(const Dev &d, const SimConst &c,
       const uint32_t em = e0 + lane < n ? w : d.idle_entry;
       masked_group(d.pos[em & J_MASK], d.type[em & J_MASK], em, e0 + lane < n ? segm[e0 + lane] : 0u);
     }
-    for (int e0 = e1; e0 < n; e0 += 32 * U) {
+    int e0 = e1;
+    for (; e0 + 32 < n; e0 += 32 * U) {
       float4 pj_n[U];
       int tj_n[U];
       uint32_t ent_nn[U];
@@ -323,25 +330,35 @@ __device__ __forceinline__ void pair_cluster_f2(const Dev &d, const SimConst &c,
         tj[u] = tj_n[u];
       }
     }
+    if (e0 < n) {  // an odd last group (the second one would hold idle entries only, which add nothing)
+      JAtom j = j_atom(pj[0], tj[0], ent[0]);
+#pragma unroll
+      for (int p = 0; p < CL / 2; ++p) pair2(std::false_type{}, j, p, s_ip[wib][p][0], s_ip[wib][p][1], 0u);
+      add_j(j, (int)(ent[0] & J_MASK));
+    }
   }
 
-  float fi[CL][3];
-#pragma unroll
-  for (int p = 0; p < CL / 2; ++p) {
-    fi[2 * p][0] = -fx[p].x; fi[2 * p][1] = -fy[p].x; fi[2 * p][2] = -fz[p].x;
-    fi[2 * p + 1][0] = -fx[p].y; fi[2 * p + 1][1] = -fy[p].y; fi[2 * p + 1][2] = -fz[p].y;
-  }
+  // the i-forces (minus these sums), added up in the order of the lanes
   float *r = s_red[wib];
 #pragma unroll
-  for (int a = 0; a < CL; ++a)
+  for (int p = 0; p < CL / 2; ++p) {
+    const float2 f3[3] = {fx[p], fy[p], fz[p]};
 #pragma unroll
-    for (int k = 0; k < 3; ++k) r[(3 * a + k) * 33 + lane] = fi[a][k];
+    for (int k = 0; k < 3; ++k) {
+      r[(6 * p + k) * RED_STRIDE + lane] = f3[k].x;
+      r[(6 * p + 3 + k) * RED_STRIDE + lane] = f3[k].y;
+    }
+  }
   __syncwarp();
   if (lane < 3 * CL) {
     float sum = 0.f;
-    for (int l = 0; l < 32; ++l) sum += r[lane * 33 + l];
+#pragma unroll
+    for (int l = 0; l < 32; l += 4) {
+      const float4 v = *reinterpret_cast<const float4 *>(r + lane * RED_STRIDE + l);
+      sum = __fadd_rn(__fadd_rn(__fadd_rn(__fadd_rn(sum, v.x), v.y), v.z), v.w);
+    }
     const int a = lane / 3, comp = lane - 3 * a;
-    const long long val = fx_from(sum);
+    const long long val = fx_from(-sum);
     if (val != 0) red_add((comp == 0 ? d.fx : comp == 1 ? d.fy : d.fz) + I * CL + a, val);
   }
   if constexpr (ENERGY) {
