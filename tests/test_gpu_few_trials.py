@@ -67,6 +67,28 @@ def test_lists_with_many_excluded_partners_are_bit_exact(per_atom):
     assert got == ref and len(ref) > 10 * s.n_atoms
 
 
+@pytest.mark.parametrize("crowd", [60, 127, 128, 129, 257, 512, 900])
+def test_crowded_columns_give_the_oracles_pairs(crowd):
+    """A grid column that holds about `crowd` atoms (below, at and beyond the
+    threads that sort it, up to its capacity of 1024), several of them at the
+    same height: the oracle's pair set, with the columns around nearly empty."""
+    import oracle as O
+
+    s, p = S.small_solvated(n_solute=24, n_water=432)
+    rng = np.random.default_rng(crowd)
+    pos = s.pos % s.box
+    who = rng.permutation(s.n_atoms)[:crowd]
+    pos[who, :2] = 0.5 * s.box + 0.02 * rng.random((crowd, 2))
+    pos[who, 2] = np.round(rng.random(crowd) * s.box, 2)
+    pos = pos.astype(np.float32).astype(np.float64)
+    with B.TrialBatch(s, p, [1], trial_seeds=[3]) as b:
+        b.set_state(0, pos, np.zeros_like(pos))
+        at = B.sim_list_positions(b.h, 0)
+        got = B.sim_pairlist(b.h, 0).tolist()
+    ref = {tuple(x) for x in O.pairlist(s, at.astype(np.float32), p.r_cut + p.skin).tolist()}
+    assert len(got) == len(ref) and {tuple(x) for x in got} == ref
+
+
 @pytest.mark.parametrize("n_solute,n_water", [(6, 430), (37, 420), (60, 440)])
 def test_one_pass_energies_match_the_general_kernel(n_solute, n_water):
     """Energies of the one-pass force and energy kernel (device tensors) and
