@@ -19,7 +19,7 @@ struct Dev {
   float4 *pos, *vel, *pos_b, *vel_b;   // pos.w = q*sqrt(f), vel.w = 1/m
   int32_t *orig, *type, *orig_b, *type_b;
   int32_t *slot_trial;                 // static: trial of every slot
-  int32_t *slot_col;                   // grid column of every slot at binning (-1: none)
+  int32_t *slot_col;                   // grid column (front kernel: and place in its bucket) of a slot at binning, -1: none
   long long *fx, *fy, *fz;             // fixed-point force accumulators per slot
   // clusters
   int32_t *clus_trial;                 // static: trial of every i-cluster

@@ -56,7 +56,7 @@ __global__ void k_rebuild_request(Dev d, int trial) {
 // ---------------------------------------------------------------------------
 // cond_a, cond_b (with set_cond): conditional nodes of a captured graph
 // around the later rebuild kernels, opened only when a trial rebuilds
-__global__ void __cluster_dims__(FRONT_CLUSTER, 1, 1) __launch_bounds__(FRONT_THREADS, 1)
+__global__ void __cluster_dims__(FRONT_CLUSTER, 1, 1) __launch_bounds__(FRONT_THREADS, 2)
     k_front(Dev d, SimConst c, float half_skin2, int strict, int forced_only, cudaGraphConditionalHandle cond_a,
             cudaGraphConditionalHandle cond_b, int set_cond) {
   __shared__ FrontShared sh;

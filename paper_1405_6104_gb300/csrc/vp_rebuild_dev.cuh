@@ -10,18 +10,17 @@
 
 namespace vp {
 
-// Slot `slot` of trial t, its position p already loaded (live: the slot
-// holds an atom): wrapped into the box, its grid column picked and recorded
-// in slot_col; returns the trial's column offset plus the column (the index
-// into the per-column arrays), or -1 for a slot without an atom.
+// Slot `slot` of trial t, its atom already loaded (live: the slot holds one):
+// wrapped into the box and staged in the sort buffers; returns its grid
+// column, or -1 for a slot without an atom.
 __device__ __forceinline__ int bin_loaded(const Dev &d, const SimConst &c, const TrialInfo &T, float half_skin2,
-                                          int strict, int t, int slot, bool live, int o, float4 p,
-                                          unsigned long long n) {
-  if (!live) { d.slot_col[slot] = -1; return -1; }
+                                          int strict, int t, int slot, bool live, int o, float4 p, float4 v,
+                                          int ty, unsigned long long n) {
+  if (!live) return -1;
   // the slot's atom is staged in the sort buffers (the column sort reads it
   // there and writes the new layout straight into the arrays themselves)
-  d.vel_b[slot] = d.vel[slot];
-  d.type_b[slot] = d.type[slot];
+  d.vel_b[slot] = v;
+  d.type_b[slot] = ty;
   d.orig_b[slot] = o;
   const float L = T.box, iL = T.inv_box;
   if (c.list_fixed && d.rb[d.n_trials + t] != (uint32_t)n) {
@@ -50,37 +49,29 @@ __device__ __forceinline__ int bin_loaded(const Dev &d, const SimConst &c, const
   d.pos_b[slot] = make_float4(x, y, z, p.w);
   int cx = max(0, min((int)(x * T.inv_col_w), T.ncol - 1));
   int cy = max(0, min((int)(y * T.inv_col_w), T.ncol - 1));
-  const int col = cx * T.ncol + cy;
-  d.slot_col[slot] = col;
-  return T.col0 + col;
+  return cx * T.ncol + cy;
 }
 
-// the same for slot `local` of the trial (loads included)
-__device__ __forceinline__ int bin_slot_col(const Dev &d, const SimConst &c, const TrialInfo &T, float half_skin2,
-                                            int strict, int t, int local, int n_clus, unsigned long long n) {
-  if (local >= T.max_clus * CL) return -1;
-  const int slot = T.slot0 + local;
-  const int o = d.orig[slot];
-  const bool live = local < n_clus * CL && o >= 0;
-  return bin_loaded(d, c, T, half_skin2, strict, t, slot, live, o,
-                    live ? d.pos[slot] : make_float4(0.f, 0.f, 0.f, 0.f), n);
-}
-
-// ... and counted in its column (global counters)
+// slot `local` of the trial, its column recorded in slot_col and counted (global counters)
 __device__ __forceinline__ void bin_slot(const Dev &d, const SimConst &c, float half_skin2, int strict, int t,
                                          int local, unsigned long long n) {
   const TrialInfo T = d.tinfo[t];
-  const int cg = bin_slot_col(d, c, T, half_skin2, strict, t, local, d.tstate[t].n_clus, n);
-  if (cg < 0) return;
+  if (local >= T.max_clus * CL) return;
+  const int slot = T.slot0 + local;
+  const int o = d.orig[slot];
+  const bool live = local < d.tstate[t].n_clus * CL && o >= 0;
+  const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
+  const int col = bin_loaded(d, c, T, half_skin2, strict, t, slot, live, o, live ? d.pos[slot] : none,
+                             live ? d.vel[slot] : none, live ? d.type[slot] : 0, n);
+  d.slot_col[slot] = col;
+  if (col < 0) return;
   // slots are in column order from the last rebuild, so a warp's atoms fall
   // into one or two columns: one atomic per column and warp
-  const unsigned peers = __match_any_sync(__activemask(), cg);
-  if ((threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&d.col_count[cg], __popc(peers));
+  const unsigned peers = __match_any_sync(__activemask(), col);
+  if ((threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&d.col_count[T.col0 + col], __popc(peers));
 }
 
-// STAMP: record this step as the trial's last rebuild here (the front kernel
-// leaves that to the column sort: its blocks still read the stamps to decide)
-template <int NT, bool STAMP = true>
+template <int NT>
 __device__ __forceinline__ void colscan_trial(const Dev &d, int (&s_a)[NT], int (&s_c)[NT], int t) {
   const TrialInfo T = d.tinfo[t];
   int nc = T.ncol * T.ncol;
@@ -123,7 +114,7 @@ __device__ __forceinline__ void colscan_trial(const Dev &d, int (&s_a)[NT], int 
   if (threadIdx.x == NT - 1) {
     d.tstate[t].n_clus = total;
     const uint32_t n32 = (uint32_t)*d.cur_step;
-    if (STAMP) d.last_rb[t] = n32;
+    d.last_rb[t] = n32;
     atomicAdd(reinterpret_cast<unsigned long long *>(d.diag + 1), 1ull);
     if (d.rb[t] == n32) atomicAdd(reinterpret_cast<unsigned long long *>(d.diag + 2), 1ull);
   }
@@ -160,91 +151,155 @@ __device__ __forceinline__ void colfill_slot(const Dev &d, int t, int local) {
 
 // The first part of trial t's rebuild by one thread-block cluster of
 // FRONT_CLUSTER blocks of FRONT_THREADS threads, in place of three grid-wide
-// kernels: binning (bin_loaded), the column scans (colscan_trial) and the
-// bucket fill.  The column counters live in the shared memory of the
-// cluster's first block; the others reach them through distributed shared
-// memory.  The order inside a column's bucket depends on timing (as with the
-// separate kernels), but the column sort orders every column by (z, atom
-// index), so the layout is the same.  Each thread issues the loads of
-// FRONT_UNROLL slots together.
-constexpr int FRONT_THREADS = 1024;
-constexpr int FRONT_CLUSTER = 4;
-constexpr int FRONT_UNROLL = 4;
+// kernels: binning, the column scans and the bucket fill.  The column counters
+// live in the shared memory of the cluster's first block; the others reach
+// them through distributed shared memory.  The order inside a column's bucket
+// depends on timing, but the column sort orders every column by (z, atom
+// index), so the layout is the same.
+// A chain of latencies, so: each thread's loads of FRONT_UNROLL slots go out
+// together, the counting atomic returns the atom's place in its bucket (no
+// second pass of atomics), column and place stay in registers (slot_col holds
+// them only for slots beyond the first FRONT_UNROLL of a thread), the scan
+// runs on the shared counters with one barrier, and eight blocks of 512 threads
+// spread a trial over eight SMs at 64 registers, two blocks per SM.  14 unequal
+// trials 27 -> 17 us per step, 64 trials of 11 040 atoms 20 -> 15, 10 trials of
+// 30 000 23 -> 16 (4 blocks of 1024 threads, two atomic passes before; 8 x 512
+// with four slots per thread 19 / 17, with two 21 / 18; 8 x 256 25 / 18).
+constexpr int FRONT_THREADS = 512;
+constexpr int FRONT_CLUSTER = 8;
+constexpr int FRONT_UNROLL = 3;
 constexpr int MAX_COLS = 64 * 64;  // columns per trial (the host caps the grid at 64 x 64)
+constexpr int COL_BITS = 12;
+static_assert(MAX_COLS <= 1 << COL_BITS && COL_CAP < 1 << (30 - COL_BITS), "column and place share a word");
 struct FrontShared {
-  int cnt[MAX_COLS];   // atoms per column (used in the cluster's first block)
-  int fill[MAX_COLS];  // places taken in each column's bucket (idem)
-  int a[FRONT_THREADS], c[FRONT_THREADS];
+  int cnt[MAX_COLS];  // atoms per column, then the column's first place, -1 beyond its capacity (the first block's)
+  int wa[32], wc[32];
+  int n_clus;         // clusters of the new layout (the first block's)
 };
+
+__device__ __forceinline__ void front_scan(const Dev &d, FrontShared &sh, const TrialInfo &T, int t) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nc = T.ncol * T.ncol;
+  const int per = (nc + FRONT_THREADS - 1) / FRONT_THREADS;
+  const int b = min((int)threadIdx.x * per, nc), e = min(b + per, nc);
+  int sa = 0, sc = 0;
+  for (int k = b; k < e; ++k) {
+    const int n = sh.cnt[k];
+    sa += n;
+    sc += (n + CL - 1) / CL;
+  }
+  int ia = sa, ic = sc;  // inclusive sums
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const int va = __shfl_up_sync(0xffffffffu, ia, off), vc = __shfl_up_sync(0xffffffffu, ic, off);
+    if (lane >= off) { ia += va; ic += vc; }
+  }
+  if (lane == 31) { sh.wa[warp] = ia; sh.wc[warp] = ic; }
+  __syncthreads();
+  int wa = 0, wc = 0, total = 0;
+  {
+    const int xa = lane < FRONT_THREADS / 32 ? sh.wa[lane] : 0, xc = lane < FRONT_THREADS / 32 ? sh.wc[lane] : 0;
+    wa = (int)__reduce_add_sync(0xffffffffu, (unsigned)(lane < warp ? xa : 0));
+    wc = (int)__reduce_add_sync(0xffffffffu, (unsigned)(lane < warp ? xc : 0));
+    total = (int)__reduce_add_sync(0xffffffffu, (unsigned)xc);
+  }
+  int pa = wa + ia - sa, pc = wc + ic - sc;
+  for (int k = b; k < e; ++k) {
+    const int n = sh.cnt[k];
+    d.col_count[T.col0 + k] = n;
+    d.col_start[T.col0 + k] = pa;
+    d.col_cstart[T.col0 + k] = pc;
+    if (n > COL_CAP) atomicOr(d.err, ERR_COL);
+    sh.cnt[k] = n > COL_CAP ? -1 : pa;
+    pa += n;
+    pc += (n + CL - 1) / CL;
+  }
+  if (threadIdx.x == 0) {
+    if (total > T.max_clus) {
+      atomicOr(d.err, ERR_CAPACITY);
+      total = T.max_clus;
+    }
+    sh.n_clus = total;
+    d.tstate[t].n_clus = total;
+    atomicAdd(reinterpret_cast<unsigned long long *>(d.diag + 1), 1ull);
+    if (d.rb[t] == (uint32_t)*d.cur_step) atomicAdd(reinterpret_cast<unsigned long long *>(d.diag + 2), 1ull);
+  }
+}
 
 __device__ __forceinline__ void front_trial(const Dev &d, const SimConst &c, float half_skin2, int strict,
                                             FrontShared &sh, int t, unsigned long long n) {
   namespace cgr = cooperative_groups;
   cgr::cluster_group cl = cgr::this_cluster();
-  const int rank = (int)cl.block_rank();
+  const int rank = (int)cl.block_rank(), lane = threadIdx.x & 31;
   int *cnt0 = cl.map_shared_rank(sh.cnt, 0);
-  int *fill0 = cl.map_shared_rank(sh.fill, 0);
   const TrialInfo T = d.tinfo[t];
-  const int nc = T.ncol * T.ncol;
-  const int n_clus = d.tstate[t].n_clus;
-  const int n_slots = T.max_clus * CL;
+  const int n_slots = T.max_clus * CL, n_used = d.tstate[t].n_clus * CL;
   constexpr int STRIDE = FRONT_CLUSTER * FRONT_THREADS;
   const int first = rank * FRONT_THREADS + threadIdx.x;
   if (rank == 0)
-    for (int k = threadIdx.x; k < nc; k += FRONT_THREADS) {
-      sh.cnt[k] = 0;
-      sh.fill[k] = 0;
-    }
+    for (int k = threadIdx.x; k < T.ncol * T.ncol; k += FRONT_THREADS) sh.cnt[k] = 0;
   cl.sync();
-  for (int base = first; base < n_slots; base += STRIDE * FRONT_UNROLL) {
-    int o[FRONT_UNROLL];
-    float4 p[FRONT_UNROLL];
+  int word[FRONT_UNROLL];  // column | place in its bucket << COL_BITS, or -1, of the thread's first slots
+  for (int base = first; base - lane < n_slots; base += STRIDE * FRONT_UNROLL) {
+    int o[FRONT_UNROLL], at[FRONT_UNROLL];
+    float4 p[FRONT_UNROLL], v[FRONT_UNROLL];
+    int ty[FRONT_UNROLL];
+    unsigned peers[FRONT_UNROLL];
 #pragma unroll
     for (int u = 0; u < FRONT_UNROLL; ++u) {
-      const int local = base + u * STRIDE;
-      o[u] = local < n_slots ? d.orig[T.slot0 + local] : -1;
-      p[u] = local < n_slots ? d.pos[T.slot0 + local] : make_float4(0.f, 0.f, 0.f, 0.f);
+      const int local = base + u * STRIDE, slot = T.slot0 + local;
+      const bool in = local < n_used;
+      o[u] = in ? d.orig[slot] : -1;
+      p[u] = in ? d.pos[slot] : make_float4(0.f, 0.f, 0.f, 0.f);
+      v[u] = in ? d.vel[slot] : make_float4(0.f, 0.f, 0.f, 0.f);
+      ty[u] = in ? d.type[slot] : 0;
+    }
+    // slots are in column order from the last rebuild, so a warp's atoms fall
+    // into one or two columns: one atomic per column and warp, the lanes of a
+    // column take consecutive places
+    int w[FRONT_UNROLL];
+#pragma unroll
+    for (int u = 0; u < FRONT_UNROLL; ++u) {
+      w[u] = bin_loaded(d, c, T, half_skin2, strict, t, T.slot0 + base + u * STRIDE, o[u] >= 0, o[u], p[u], v[u], ty[u], n);
+      peers[u] = __match_any_sync(0xffffffffu, w[u]);
+      at[u] = 0;
+      if (w[u] >= 0 && lane == __ffs(peers[u]) - 1) at[u] = atomicAdd(cnt0 + w[u], __popc(peers[u]));
     }
 #pragma unroll
     for (int u = 0; u < FRONT_UNROLL; ++u) {
+      const int place = __shfl_sync(0xffffffffu, at[u], __ffs(peers[u]) - 1) + __popc(peers[u] & ((1u << lane) - 1u));
+      if (w[u] >= 0) w[u] |= min(place, COL_CAP) << COL_BITS;
       const int local = base + u * STRIDE;
-      if (local < n_slots) {
-        const bool live = local < n_clus * CL && o[u] >= 0;
-        const int cg = bin_loaded(d, c, T, half_skin2, strict, t, T.slot0 + local, live, o[u], p[u], n);
-        if (cg >= 0) {
-          const unsigned peers = __match_any_sync(__activemask(), cg);
-          if ((threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(cnt0 + (cg - T.col0), __popc(peers));
-        }
-      }
+      if (base == first) word[u] = w[u];
+      else if (local < n_slots) d.slot_col[T.slot0 + local] = w[u];
     }
   }
   cl.sync();
-  if (rank == 0) {
-    for (int k = threadIdx.x; k < nc; k += FRONT_THREADS) d.col_count[T.col0 + k] = sh.cnt[k];
-    __syncthreads();
-    colscan_trial<FRONT_THREADS, false>(d, sh.a, sh.c, t);
-  }
-  cl.sync();  // the column starts are written (release and acquire at cluster scope)
+  if (rank == 0) front_scan(d, sh, T, t);
+  cl.sync();
+  const int n_new = *cl.map_shared_rank(&sh.n_clus, 0) * CL;
   for (int base = first; base < n_slots; base += STRIDE * FRONT_UNROLL) {
-    int col[FRONT_UNROLL];
+    if (base != first) {
 #pragma unroll
-    for (int u = 0; u < FRONT_UNROLL; ++u) {
-      const int local = base + u * STRIDE;
-      col[u] = local < n_slots ? d.slot_col[T.slot0 + local] : -1;
+      for (int u = 0; u < FRONT_UNROLL; ++u)
+        word[u] = base + u * STRIDE < n_slots ? d.slot_col[T.slot0 + base + u * STRIDE] : -1;
     }
+    int start[FRONT_UNROLL];
+#pragma unroll
+    for (int u = 0; u < FRONT_UNROLL; ++u) start[u] = word[u] >= 0 ? cnt0[word[u] & ((1 << COL_BITS) - 1)] : -1;
 #pragma unroll
     for (int u = 0; u < FRONT_UNROLL; ++u) {
-      if (col[u] >= 0) {
-        const unsigned act = __activemask();
-        const unsigned peers = __match_any_sync(act, col[u]);
-        const int lane = threadIdx.x & 31, leader = __ffs(peers) - 1;
-        int b = 0;
-        if (lane == leader) b = atomicAdd(fill0 + col[u], __popc(peers));
-        b = __shfl_sync(act, b, leader);
-        const int q = b + __popc(peers & ((1u << lane) - 1u));
-        const int cg = T.col0 + col[u];
-        if (q < COL_CAP && d.col_count[cg] <= COL_CAP)
-          d.bucket[T.atom0 + d.col_start[cg] + q] = T.slot0 + base + u * STRIDE;
+      const int place = word[u] >> COL_BITS, local = base + u * STRIDE, sl = T.slot0 + local;
+      if (start[u] >= 0 && place < COL_CAP) d.bucket[T.atom0 + start[u] + place] = sl;
+      // slots past the new clusters become empty (their atoms, if any, are
+      // staged in the sort buffers already; the column sort fills the others)
+      if (local >= n_new && local < n_slots) {
+        const float4 pad = pad_pos(sl);
+        d.orig[sl] = -1;
+        d.pos[sl] = pad;
+        d.ref_slot[sl] = pad;
+        d.vel[sl] = make_float4(0.f, 0.f, 0.f, 0.f);
+        d.type[sl] = 0;
       }
     }
   }

@@ -89,6 +89,25 @@ def test_crowded_columns_give_the_oracles_pairs(crowd):
     assert len(got) == len(ref) and {tuple(x) for x in got} == ref
 
 
+@pytest.mark.parametrize("n_water", [3900, 4400, 8300])
+def test_lists_of_trials_beyond_one_pass_of_the_binning(n_water):
+    """Trials of about as many atoms as the binning's threads take in one pass
+    (12 288), and two and three passes, beside a small trial: the oracle's pair
+    sets, after a rebuild that starts from a list's order."""
+    import oracle as O
+
+    big, p = S.small_solvated(n_solute=24, n_water=n_water)
+    small, _ = S.small_solvated(n_solute=24, n_water=432)
+    with B.TrialBatch([big, small], p, [1, 1], trial_seeds=[3, 4]) as b:
+        b.step(7)
+        for k, s in enumerate((big, small)):
+            pos = B.sim_list_positions(b.h, k).astype(np.float32)
+            got = B.sim_pairlist(b.h, k).astype(np.int64)
+            ref = O.pairlist(s, pos, p.r_cut + p.skin).astype(np.int64)
+            assert np.array_equal(np.sort(got[:, 0] * s.n_atoms + got[:, 1]),
+                                  np.sort(ref[:, 0] * s.n_atoms + ref[:, 1]))
+
+
 @pytest.mark.parametrize("n_solute,n_water", [(6, 430), (37, 420), (60, 440)])
 def test_one_pass_energies_match_the_general_kernel(n_solute, n_water):
     """Energies of the one-pass force and energy kernel (device tensors) and
