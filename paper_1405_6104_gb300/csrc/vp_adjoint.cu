@@ -278,9 +278,9 @@ __global__ void __launch_bounds__(adj_threads(NW), adj_blocks(NW)) k_adj_hw(AdjD
     }
     n_near = cv_near_list_block<NW>(t, sh.s_near, s_bal, sh.s_x);
   }
-  for (int p = NW == 1 ? lane : (int)threadIdx.x; p < n_near; p += 2 * NW * 32) {
-    const bool two = p + NW * 32 < n_near;
-    adj_hw_pairs(sh, t, k, sh.s_near[p], sh.s_near[two ? p + NW * 32 : p], two);
+  for (int p = (NW == 1 ? 0 : 64 * warp) + lane; p < n_near; p += 64 * NW) {
+    const bool two = p + 32 < n_near;
+    adj_hw_pairs(sh, t, k, sh.s_near[p], sh.s_near[two ? p + 32 : p], two);
   }
   if constexpr (NW == 1) __syncwarp(); else __syncthreads();
   for (int q = NW == 1 ? lane : (int)threadIdx.x; q < 2 * CV_T; q += NW * 32) {

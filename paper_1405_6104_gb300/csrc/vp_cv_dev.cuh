@@ -267,8 +267,9 @@ __device__ __forceinline__ void cv_tile_block(const CvTile &t, const CvConst &k,
     return;
   }
   const int n_near = cv_near_list_block<NW>(t, sh.s_near, sh.s_bal, sh.s_x);
-  for (int p = threadIdx.x; p < n_near; p += 2 * NW * 32) {
-    const int p1 = p + NW * 32;
+  // 64 pairs per warp at a time: warps without any leave their issue slots to the others
+  for (int p = 64 * warp + lane; p < n_near; p += 64 * NW) {
+    const int p1 = p + 32;
     const bool two = p1 < n_near;
     const ff2 v = cv_near_pairs(sh, k, t, sh.s_near[p], sh.s_near[two ? p1 : p], two);
     sh.s_term[p] = make_float2(v.hi.x, v.lo.x);
