@@ -113,6 +113,28 @@ __global__ void __launch_bounds__(LIST_WARPS * 32, 6) k_list(Dev d, SimConst c, 
   }
 }
 
+// The same with PARTS warps per cluster (at 96 registers), for batches so small
+// that every cluster of every trial can have that many at once: there a list is
+// one chain of latencies.  One trial of 11 040 atoms (1487 clusters) with two
+// warps per cluster: step 35.7 -> 33.3 us, of 1320 atoms (188) with four 35.2 ->
+// 29.2; with four for 1487 clusters, or two for 3975 (7950 warps on 3648), 0.4
+// and 0.5 us slower than with two and one.  Kept apart from k_list: one kernel
+// with both spills, and its loop of lists takes 152 instead of 138 us.
+constexpr int LIST_PARTS_BLOCKS = 5;
+template <int PARTS>
+__global__ void __launch_bounds__(LIST_WARPS * 32, LIST_PARTS_BLOCKS) k_list_parts(Dev d, SimConst c, float rl2_bbox) {
+  __shared__ ListShared sh;
+  PDL_WAIT();
+  constexpr int PER_BLOCK = LIST_WARPS / PARTS;
+  const int n_items = (int)d.rb_cnt[0] * d.max_trial_clus;
+  int turn = 0;
+  for (int item = (int)blockIdx.x * PER_BLOCK + (int)(threadIdx.x >> 5) / PARTS; item < n_items;
+       item += (int)gridDim.x * PER_BLOCK, ++turn) {
+    __syncwarp();  // the warp's shared arrays of its previous cluster are no longer read
+    list_cluster<PARTS>(d, c, rl2_bbox, sh, d.rb_list[item / d.max_trial_clus], item % d.max_trial_clus, turn);
+  }
+}
+
 // positions the current list of one trial was built from, caller order
 __global__ void k_list_positions(Dev d, int trial, double *out, int n) {
   const int o = blockIdx.x * blockDim.x + threadIdx.x;
@@ -152,8 +174,16 @@ void launch_colsort(const Dev &d, cudaStream_t s) {
   launch_pdl(k_colsort, dim3(rebuild_grid(d, 8, d.max_trial_cols)), dim3(128), s, d);
 }
 void launch_list(const Dev &d, const SimConst &c, float rl2_bbox, cudaStream_t s) {
-  launch_pdl(k_list, dim3(rebuild_grid(d, 6, (d.max_trial_clus + LIST_WARPS - 1) / LIST_WARPS)), dim3(LIST_WARPS * 32),
-             s, d, c, rl2_bbox);
+  const long long warps = (long long)LIST_PARTS_BLOCKS * d.n_sm * LIST_WARPS, clusters = (long long)d.max_trial_clus * d.n_trials;
+  if (4 * clusters <= warps)
+    launch_pdl(k_list_parts<4>, dim3(rebuild_grid(d, LIST_PARTS_BLOCKS, d.max_trial_clus)), dim3(LIST_WARPS * 32), s, d, c,
+               rl2_bbox);
+  else if (2 * clusters <= warps)
+    launch_pdl(k_list_parts<2>, dim3(rebuild_grid(d, LIST_PARTS_BLOCKS, (d.max_trial_clus + 1) / 2)), dim3(LIST_WARPS * 32),
+               s, d, c, rl2_bbox);
+  else
+    launch_pdl(k_list, dim3(rebuild_grid(d, 6, (d.max_trial_clus + LIST_WARPS - 1) / LIST_WARPS)), dim3(LIST_WARPS * 32),
+               s, d, c, rl2_bbox);
 }
 
 }  // namespace vp

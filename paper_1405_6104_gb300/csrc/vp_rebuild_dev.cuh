@@ -493,11 +493,17 @@ struct ListShared {
   unsigned s_dirty[LIST_WARPS][ENT_MAX / 32];  // entries whose j-atoms need the pair masks
   unsigned s_mask[LIST_WARPS][ENT_MAX];        // halves to test (phase 1), then the entries' masks (their
                                                // first words overwrite s_cand)
+  int4 s_part[2][LIST_WARPS];  // of the parts of a list: halves found, entries, masked and clean j-atoms
 };
 
+// PARTS > 1: that many consecutive warps of the block share the list, each
+// doing an equal share of the window's columns (turn counts their lists).  The
+// shares are consecutive in the list's order, so a warp only needs to know how
+// many j-atoms the shares before its own hold.
+template <int PARTS = 1>
 __device__ __forceinline__ void list_cluster(const Dev &d, const SimConst &c, float rl2_bbox, ListShared &sh, int t,
-                                             int Il) {
-  const int wib = threadIdx.x >> 5;
+                                             int Il, int turn = 0) {
+  const int wib = threadIdx.x >> 5, part = wib % PARTS;
   const int lane = threadIdx.x & 31;
   auto &s_xp = sh.s_xp[wib];
   auto &s_dirty = sh.s_dirty[wib];
@@ -566,7 +572,8 @@ __device__ __forceinline__ void list_cluster(const Dev &d, const SimConst &c, fl
   const float inv_wny = 1.0f / (float)wny;
   const float half_w = 0.5f * w, img_lim = 0.49999f * L;
   int xs = -1;  // slot of this lane's excluded partner
-  for (int cb = 0; cb < nwin; cb += 32) {
+  const int col_lo = nwin * part / PARTS, col_hi = nwin * (part + 1) / PARTS;
+  for (int cb = col_lo; cb < col_hi; cb += 32) {
     const int wi = cb + lane;
     // this lane's column: up to two ranges [a1, a1 + n1), [a2, a2 + n2) of
     // half indices (relative to the trial's first half) whose z-extent can
@@ -574,7 +581,7 @@ __device__ __forceinline__ void list_cluster(const Dev &d, const SimConst &c, fl
     // the column's xy gap, the ranges from the column's z-bin table, one bin
     // wider on each side than needed (every half in them is still tested)
     int a1 = 0, n1 = 0, a2 = 0, n2 = 0;
-    if (wi < nwin) {
+    if (wi < col_hi) {
       const int wr = (int)(((float)wi + 0.5f) * inv_wny);  // wi / wny (exact: wi < 2^12)
       const int cx = kth(wx0, wnx, row0 + wr), cy = kth(wy0, wny, wi - wr * wny);
       const int cc = cx * T.ncol + cy;
@@ -621,7 +628,7 @@ __device__ __forceinline__ void list_cluster(const Dev &d, const SimConst &c, fl
         }
       }
     }
-    if (cb == 0 && xa >= 0) xs = d.slot_of[T.atom0 + xa];
+    if (cb == col_lo && xa >= 0) xs = d.slot_of[T.atom0 + xa];
     const int cntc = n1 + n2;
     // inclusive scan of the per-column counts
     int incl = cntc;
@@ -667,7 +674,7 @@ __device__ __forceinline__ void list_cluster(const Dev &d, const SimConst &c, fl
       }
     }
   }
-  const bool overflow = n_cand > CAND_MAX;
+  int n_found = n_cand;
   n_cand = min(n_cand, CAND_MAX);
   __syncwarp();
   // ---- phase 2: one candidate 4-atom j-cluster per lane ----
@@ -777,9 +784,30 @@ __device__ __forceinline__ void list_cluster(const Dev &d, const SimConst &c, fl
     const int e = e0 + lane;
     n_dirty += __reduce_add_sync(0xffffffffu, e < n_ent && ((dw >> lane) & 1u) ? j_columns(s_mask[e]) : 0);
   }
+  int pd = 0, pc = n_dirty;  // where the next j-atoms of either kind go
+  if constexpr (PARTS > 1) {
+    int n_clean = 0;
+    for (int e = lane; e < n_ent; e += 32) n_clean += j_columns(s_mask[e]);
+    n_clean = (int)__reduce_add_sync(0xffffffffu, (unsigned)n_clean) - n_dirty;
+    const int w0 = wib - part;
+    if (lane == 0) sh.s_part[turn & 1][wib] = make_int4(n_found, cnt, n_dirty, n_clean);
+    // (constant barrier numbers: a block that may use all 16 leaves room for two on an SM)
+    if (PARTS == LIST_WARPS) __syncthreads();
+    else if (w0 == 0) asm volatile("bar.sync 1, %0;" ::"n"(32 * PARTS) : "memory");
+    else asm volatile("bar.sync 2, %0;" ::"n"(32 * PARTS) : "memory");
+    int before = 0;
+    n_found = cnt = n_dirty = 0;
+    for (int q = 0; q < PARTS; ++q) {
+      const int4 v = sh.s_part[turn & 1][w0 + q];
+      n_found += v.x;
+      cnt += v.y;
+      n_dirty += v.z;
+      if (q < part) { pd += v.z; before += v.w; }
+    }
+    pc = n_dirty + before;
+  }
   uint32_t *segw = d.list + (size_t)I * c.list_cap;
   uint8_t *segm = d.list_m + (size_t)I * c.list_cap;
-  int pd = 0, pc = n_dirty;  // where the next j-atoms of either kind go
   for (int e0 = 0; e0 < n_ent; e0 += 32) {
     const int e = e0 + lane;
     const unsigned m = e < n_ent ? s_mask[e] : 0u;
@@ -814,10 +842,10 @@ __device__ __forceinline__ void list_cluster(const Dev &d, const SimConst &c, fl
     pd += tot & 0xffff;
     pc += tot >> 16;
   }
-  if (lane == 0) {
+  if (lane == 0 && part == PARTS - 1) {
     d.list_n[I] = min(pc, c.list_cap);
     d.list_nm[I] = min(n_dirty, c.list_cap);
-    if (cnt > ENT_MAX || pc > c.list_cap || overflow) atomicOr(d.err, ERR_LIST);
+    if (cnt > ENT_MAX || pc > c.list_cap || n_found > CAND_MAX) atomicOr(d.err, ERR_LIST);
   }
 }
 

@@ -89,6 +89,21 @@ def test_crowded_columns_give_the_oracles_pairs(crowd):
     assert len(got) == len(ref) and {tuple(x) for x in got} == ref
 
 
+@pytest.mark.parametrize("n_water", [420, 1700, 2100, 3500, 4200])
+def test_lists_shared_by_warps_are_bit_exact(n_water):
+    """One trial's lists, each built by four warps (a few hundred clusters), by
+    two, or by one: the oracle's pair set, no pair twice."""
+    import oracle as O
+
+    s, p = S.small_solvated(n_solute=24, n_water=n_water)
+    with B.TrialBatch(s, p, [1], trial_seeds=[3]) as b:
+        b.step(7)
+        pos = B.sim_list_positions(b.h, 0).astype(np.float32)
+        got = B.sim_pairlist(b.h, 0).astype(np.int64)
+    ref = O.pairlist(s, pos, p.r_cut + p.skin).astype(np.int64)
+    assert np.array_equal(np.sort(got[:, 0] * s.n_atoms + got[:, 1]), np.sort(ref[:, 0] * s.n_atoms + ref[:, 1]))
+
+
 @pytest.mark.parametrize("n_water", [3900, 4400, 8300])
 def test_lists_of_trials_beyond_one_pass_of_the_binning(n_water):
     """Trials of about as many atoms as the binning's threads take in one pass
