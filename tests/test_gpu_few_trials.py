@@ -89,38 +89,33 @@ def test_crowded_columns_give_the_oracles_pairs(crowd):
     assert len(got) == len(ref) and {tuple(x) for x in got} == ref
 
 
-@pytest.mark.parametrize("n_water", [420, 1700, 2100, 3500, 4200])
-def test_lists_shared_by_warps_are_bit_exact(n_water):
-    """One trial's lists, each built by four warps (a few hundred clusters), by
-    two, or by one: the oracle's pair set, no pair twice."""
-    import oracle as O
-
-    s, p = S.small_solvated(n_solute=24, n_water=n_water)
-    with B.TrialBatch(s, p, [1], trial_seeds=[3]) as b:
+def _lists(systems, p, mode):
+    with B.TrialBatch(systems, p, [1] * len(systems), trial_seeds=list(range(3, 3 + len(systems)))) as b:
+        B.sim_set_step_mode(b.h, mode)
         b.step(7)
-        pos = B.sim_list_positions(b.h, 0).astype(np.float32)
-        got = B.sim_pairlist(b.h, 0).astype(np.int64)
-    ref = O.pairlist(s, pos, p.r_cut + p.skin).astype(np.int64)
-    assert np.array_equal(np.sort(got[:, 0] * s.n_atoms + got[:, 1]), np.sort(ref[:, 0] * s.n_atoms + ref[:, 1]))
+        pairs = [B.sim_pairlist(b.h, k).astype(np.int64) for k in range(len(systems))]  # in no fixed order
+        return [np.sort(x[:, 0] << 32 | x[:, 1]) for x in pairs], [b.get_state(k)[0] for k in range(len(systems))]
+
+
+@pytest.mark.parametrize("n_water", [420, 1700, 2100, 3500, 4200])
+def test_lists_shared_by_warps_match_lists_by_a_warp(n_water):
+    """One trial's lists, each built by four warps (a few hundred clusters), by
+    two, or by one: the one-kernel step's pairs, and its positions (the forces'
+    sums follow the lists' order)."""
+    s, p = S.small_solvated(n_solute=24, n_water=n_water)
+    x, y = _lists([s], p, 0), _lists([s], p, 1)
+    assert np.array_equal(x[0][0], y[0][0]) and np.array_equal(x[1][0], y[1][0])
 
 
 @pytest.mark.parametrize("n_water", [3900, 4400, 8300])
 def test_lists_of_trials_beyond_one_pass_of_the_binning(n_water):
-    """Trials of about as many atoms as the binning's threads take in one pass
-    (12 288), and two and three passes, beside a small trial: the oracle's pair
-    sets, after a rebuild that starts from a list's order."""
-    import oracle as O
-
+    """A trial of about as many atoms as the binning's threads take in one pass
+    (12 288), and in two and three, beside a small trial: the one-kernel step's
+    pairs and positions, after rebuilds that start from a list's order."""
     big, p = S.small_solvated(n_solute=24, n_water=n_water)
     small, _ = S.small_solvated(n_solute=24, n_water=432)
-    with B.TrialBatch([big, small], p, [1, 1], trial_seeds=[3, 4]) as b:
-        b.step(7)
-        for k, s in enumerate((big, small)):
-            pos = B.sim_list_positions(b.h, k).astype(np.float32)
-            got = B.sim_pairlist(b.h, k).astype(np.int64)
-            ref = O.pairlist(s, pos, p.r_cut + p.skin).astype(np.int64)
-            assert np.array_equal(np.sort(got[:, 0] * s.n_atoms + got[:, 1]),
-                                  np.sort(ref[:, 0] * s.n_atoms + ref[:, 1]))
+    for x, y in zip(_lists([big, small], p, 0), _lists([big, small], p, 1)):
+        assert all(np.array_equal(u, v) for u, v in zip(x, y))
 
 
 @pytest.mark.parametrize("n_solute,n_water", [(6, 430), (37, 420), (60, 440)])
