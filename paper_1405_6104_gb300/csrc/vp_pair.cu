@@ -492,10 +492,13 @@ void launch_bonded_energy(const Dev &d, cudaStream_t s) {
 // the types fit.  Up to 300 clusters per SM one warp per block is the faster
 // form (the MD step of one 11 040-atom trial 43.1 us against 51.2, of 16
 // trials 213 against 219, of ten 30 000-atom trials 352.2 against 352.9), in
-// larger batches the persistent one (64 trials 695 against 706 us).
+// larger batches the persistent one (64 trials 695 against 706 us).  Up to 50
+// clusters per SM 128 registers pay more than 20 warps: the step of one trial
+// of 1320 / 11 040 / 30 000 atoms 29.1 -> 28.4 / 33.0 -> 32.6 / 53.5 -> 52.2
+// us, of four of 11 040 68.3 -> 67.7, but of 16 (157 per SM) 171 -> 174.
 int default_pair_variant(const Dev &d, const SimConst &c) {
   if (c.n_types > SMALL_TYPES) return 0;
-  return d.total_clus <= 300 * d.n_sm ? 3 : 6;
+  return d.total_clus <= 50 * d.n_sm ? 4 : d.total_clus <= 300 * d.n_sm ? 3 : 6;
 }
 
 void launch_pair(const Dev &d, const SimConst &c, bool energy, int32_t only_trial, cudaStream_t s, int variant,
