@@ -973,6 +973,7 @@ VP_API int sim_create(const sim_system *systems, int32_t n_systems, const int32_
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h->device);
     d.n_sm = nsm > 0 ? nsm : 1;
   }
+  d.early_launch = few_clusters(d) ? 1 : 0;
   h->pair_variant = default_pair_variant(d, c);
   if (r) return bail(SIM_ECUDA);
   float half = 0.5f;

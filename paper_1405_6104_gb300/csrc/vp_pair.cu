@@ -427,6 +427,7 @@ __global__ void __launch_bounds__(PF_WARPS * 32, MINB) k_pair_f2(Dev d, SimConst
 template <int U, int MINB>
 __global__ void __launch_bounds__(32, MINB) k_pair_w(Dev d, SimConst c, const int *clist, int n_items) {
   __shared__ PairF2Shared<1> sh;
+  PDL_WAIT();
   const int item = blockIdx.x;
   pair_cluster_f2<U>(d, c, sh, clist ? clist[item] : item);
 }
@@ -517,8 +518,8 @@ void launch_pair(const Dev &d, const SimConst &c, bool energy, int32_t only_tria
   switch (variant) {
     case 1: k_pair_f<5><<<fb, PF_WARPS * 32, 0, s>>>(d, c, clist, n_items); break;
     case 2: k_pair_f<6><<<fb, PF_WARPS * 32, 0, s>>>(d, c, clist, n_items); break;
-    case 3: k_pair_w<2, 20><<<n_items, 32, 0, s>>>(d, c, clist, n_items); break;
-    case 4: k_pair_w<2, 16><<<n_items, 32, 0, s>>>(d, c, clist, n_items); break;
+    case 3: launch_pdl(k_pair_w<2, 20>, dim3(n_items), dim3(32), s, d, c, clist, n_items); break;
+    case 4: launch_pdl(k_pair_w<2, 16>, dim3(n_items), dim3(32), s, d, c, clist, n_items); break;
     case 5: case 6: case 7: case 8: {
       // persistent grid: as many blocks as can be resident, sized from the SM
       // count; the counter hands out the i-clusters

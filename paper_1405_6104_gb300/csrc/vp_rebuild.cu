@@ -60,6 +60,7 @@ __global__ void __cluster_dims__(FRONT_CLUSTER, 1, 1) __launch_bounds__(FRONT_TH
     k_front(Dev d, SimConst c, float half_skin2, int strict, int forced_only, cudaGraphConditionalHandle cond_a,
             cudaGraphConditionalHandle cond_b, int set_cond) {
   __shared__ FrontShared sh;
+  if (d.early_launch) PDL_TRIGGER();
   PDL_WAIT();
   const unsigned long long n = *d.cur_step;
   if (blockIdx.x == 0) {
@@ -87,6 +88,7 @@ __global__ void __cluster_dims__(FRONT_CLUSTER, 1, 1) __launch_bounds__(FRONT_TH
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(128) k_colsort(Dev d) {
   __shared__ ColsortShared sh;
+  if (d.early_launch) PDL_TRIGGER();
   PDL_WAIT();
   FOR_REBUILD_ITEMS(d.max_trial_cols, t, piece) {
     __syncthreads();  // the previous column's shared arrays are no longer read
@@ -100,6 +102,7 @@ __global__ void __launch_bounds__(128) k_colsort(Dev d) {
 // 16 trials of 11 040 atoms rebuilding)
 __global__ void __launch_bounds__(LIST_WARPS * 32, 6) k_list(Dev d, SimConst c, float rl2_bbox) {
   __shared__ ListShared sh;
+  if (d.early_launch) PDL_TRIGGER();
   PDL_WAIT();
   const int lane = threadIdx.x & 31;
   const int n_items = (int)d.rb_cnt[0] * d.max_trial_clus;
@@ -124,6 +127,7 @@ constexpr int LIST_PARTS_BLOCKS = 5;
 template <int PARTS>
 __global__ void __launch_bounds__(LIST_WARPS * 32, LIST_PARTS_BLOCKS) k_list_parts(Dev d, SimConst c, float rl2_bbox) {
   __shared__ ListShared sh;
+  if (d.early_launch) PDL_TRIGGER();
   PDL_WAIT();
   constexpr int PER_BLOCK = LIST_WARPS / PARTS;
   const int n_items = (int)d.rb_cnt[0] * d.max_trial_clus;
@@ -173,12 +177,15 @@ void launch_colsort(const Dev &d, cudaStream_t s) {
   // columns hold about 100 atoms: 128 threads keep every thread busy in the sort
   launch_pdl(k_colsort, dim3(rebuild_grid(d, 8, d.max_trial_cols)), dim3(128), s, d);
 }
+// warps that k_list_parts keeps resident
+static long long list_parts_warps(const Dev &d) { return (long long)LIST_PARTS_BLOCKS * d.n_sm * LIST_WARPS; }
+bool few_clusters(const Dev &d) { return 2ll * d.max_trial_clus * d.n_trials <= list_parts_warps(d); }
 void launch_list(const Dev &d, const SimConst &c, float rl2_bbox, cudaStream_t s) {
-  const long long warps = (long long)LIST_PARTS_BLOCKS * d.n_sm * LIST_WARPS, clusters = (long long)d.max_trial_clus * d.n_trials;
+  const long long warps = list_parts_warps(d), clusters = (long long)d.max_trial_clus * d.n_trials;
   if (4 * clusters <= warps)
     launch_pdl(k_list_parts<4>, dim3(rebuild_grid(d, LIST_PARTS_BLOCKS, d.max_trial_clus)), dim3(LIST_WARPS * 32), s, d, c,
                rl2_bbox);
-  else if (2 * clusters <= warps)
+  else if (few_clusters(d))
     launch_pdl(k_list_parts<2>, dim3(rebuild_grid(d, LIST_PARTS_BLOCKS, (d.max_trial_clus + 1) / 2)), dim3(LIST_WARPS * 32),
                s, d, c, rl2_bbox);
   else

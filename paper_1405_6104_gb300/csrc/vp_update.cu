@@ -21,6 +21,7 @@ namespace vp {
 // trips and needs every resident warp it can get.
 template <int MODE>
 __global__ void __launch_bounds__(256, 6) k_update(Dev d, SimConst c) {
+  if (d.early_launch) PDL_TRIGGER();
   update_slot<MODE>(d, c, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
