@@ -36,6 +36,8 @@ struct AdjDev {
   double *z, *Q;            // [nf]
   double *coef;             // [2 nf]: A_n, B_n
   double *phi;              // [1]
+  int *n_near;              // [nf][n_tiles] near pairs of each tile, and the ballots that list them: left by
+  unsigned *near;           // [nf][n_tiles][32] k_adj_cv for k_adj_hw (NULL: the lists are formed again)
 };
 
 struct AdjFramePos {
@@ -58,24 +60,27 @@ __device__ __forceinline__ CvTile adj_tile(const AdjDev &a, const CvConst &k, in
 // Two pairs per lane on the packed FP32 instructions, two warps per block at 64
 // registers: bound by issue (64% of the slots) and the FP32 latency of the 10
 // warps an SM holds on average, half of all tiles being far and gone at once.
-// 84 303 tiles of 51 frames of 1800 atoms: 311 -> 275 us, H_z w 340 -> 290 (one
-// pair per lane, four warps per block before; two warps alone -5 us, the
-// register limit another -5).
+// The distance tests, some 900 instructions per tile, are made once: this pass
+// keeps their ballots and H_z w reads them (132 bytes per tile).  51 frames of
+// 1800 atoms (84 303 tiles): call 821 -> 689 us, z and grad z 311 -> 277, H_z w
+// 340 -> 230 (one pair per lane, four warps per block, tests in both before).
 constexpr int ADJ_WARPS = 2;  // tiles per block of the one-warp form
 constexpr int adj_threads(int nw) { return 32 * (nw == 1 ? ADJ_WARPS : nw); }
 constexpr int adj_blocks(int nw) { return nw == 1 ? 16 : 8; }  // 64 registers
-template <int NW>
+template <int NW, bool KEEP>
 __global__ void __launch_bounds__(adj_threads(NW), adj_blocks(NW)) k_adj_cv(AdjDev a, CvConst k) {
   if constexpr (NW == 1) {
     __shared__ CvWarpShared sh[ADJ_WARPS];
     const int w = blockIdx.x * ADJ_WARPS + (threadIdx.x >> 5);
     if (w >= a.nf * a.n_tiles) return;
     const int f = w / a.n_tiles, t = w - f * a.n_tiles;
-    cv_tile(adj_tile(a, k, f, t), k, sh[threadIdx.x >> 5], AdjFramePos{a.frames + (size_t)f * 3 * a.n_cv});
+    cv_tile<KEEP>(adj_tile(a, k, f, t), k, sh[threadIdx.x >> 5], AdjFramePos{a.frames + (size_t)f * 3 * a.n_cv},
+                  a.n_near + w, a.near + (size_t)w * CV_T);
   } else {
     __shared__ CvBlockShared sh;
-    const int f = blockIdx.x / a.n_tiles, t = blockIdx.x - f * a.n_tiles;
-    cv_tile_block<NW>(adj_tile(a, k, f, t), k, sh, AdjFramePos{a.frames + (size_t)f * 3 * a.n_cv});
+    const int w = blockIdx.x, f = w / a.n_tiles, t = w - f * a.n_tiles;
+    cv_tile_block<NW, KEEP>(adj_tile(a, k, f, t), k, sh, AdjFramePos{a.frames + (size_t)f * 3 * a.n_cv}, a.n_near + w,
+                            a.near + (size_t)w * CV_T);
   }
 }
 
@@ -234,13 +239,14 @@ __device__ __forceinline__ void adj_hw_pairs(AdjHwShared &sh, const CvTile &t, c
 }
 
 // H_z w per frame with a bias, a warp (NW = 1) or a block of NW warps per (frame, tile)
-template <int NW>
+template <int NW, bool KEPT>
 __global__ void __launch_bounds__(adj_threads(NW), adj_blocks(NW)) k_adj_hw(AdjDev a, CvConst k) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   __shared__ AdjHwShared s_sh[NW == 1 ? ADJ_WARPS : 1];
   __shared__ unsigned s_bal[CV_T];
   const int w = NW == 1 ? blockIdx.x * ADJ_WARPS + warp : blockIdx.x;
   if (w >= a.nf * a.n_tiles) return;
+  if (KEPT && a.n_near[w] == 0) return;
   const int f = w / a.n_tiles;
   if (a.coef[2 * f + 1] == 0.0) return;  // no bias at this frame: no Hessian term
   CvTile t = adj_tile(a, k, f, w - f * a.n_tiles);
@@ -255,11 +261,9 @@ __global__ void __launch_bounds__(adj_threads(NW), adj_blocks(NW)) k_adj_hw(AdjD
     float3 xi = make_float3(0.f, 0.f, 0.f), xj = xi, wi = xi, wj = xi;
     if (iv) { xi = pos(i); wi = wof(i); }
     if (jv) { xj = pos(j); wj = wof(j); }
-    if (cv_tile_far(t, iv, jv, xi, xj)) return;
-    n_near = cv_near_list(t, sh.s_near, xi, xj);
-    if (n_near == 0) return;
-    sh.s_x[lane] = make_float4(xi.x, xi.y, xi.z, 0.f);
-    sh.s_x[CV_T + lane] = make_float4(xj.x, xj.y, xj.z, 0.f);
+    if (!KEPT && cv_tile_far(t, iv, jv, xi, xj)) return;
+    sh.s_x[lane] = cv_atom(iv, xi);
+    sh.s_x[CV_T + lane] = cv_atom(jv, xj);
     sh.s_w[lane] = make_float4(wi.x, wi.y, wi.z, 0.f);
     sh.s_w[CV_T + lane] = make_float4(wj.x, wj.y, wj.z, 0.f);
 #pragma unroll
@@ -267,6 +271,10 @@ __global__ void __launch_bounds__(adj_threads(NW), adj_blocks(NW)) k_adj_hw(AdjD
       sh.s_ghi[lane][q] = 0; sh.s_ghi[CV_T + lane][q] = 0;
       sh.s_glo[lane][q] = 0; sh.s_glo[CV_T + lane][q] = 0;
     }
+    __syncwarp();
+    if (KEPT) n_near = cv_near_list_kept(sh.s_near, a.near + (size_t)w * CV_T);
+    else n_near = cv_near_list<false>(t, sh.s_near, sh.s_x, nullptr);
+    if (n_near == 0) return;
     __syncwarp();
   } else {
     const bool far = cv_block_begin<NW>(t, sh, pos);
@@ -276,7 +284,13 @@ __global__ void __launch_bounds__(adj_threads(NW), adj_blocks(NW)) k_adj_hw(AdjD
       const float3 v = q < t.n_cv ? wof(q) : make_float3(0.f, 0.f, 0.f);
       sh.s_w[threadIdx.x] = make_float4(v.x, v.y, v.z, 0.f);
     }
-    n_near = cv_near_list_block<NW>(t, sh.s_near, s_bal, sh.s_x);
+    if (KEPT) {
+      if (warp == NW - 1) s_bal[lane] = a.near[(size_t)w * CV_T + lane];
+    } else {
+      cv_ballots_block<NW>(t, s_bal, sh.s_x);
+    }
+    __syncthreads();
+    n_near = cv_near_list_block<NW>(sh.s_near, s_bal);
   }
   for (int p = (NW == 1 ? 0 : 64 * warp) + lane; p < n_near; p += 64 * NW) {
     const bool two = p + 32 < n_near;
@@ -369,6 +383,10 @@ struct Carve {
   }
 };
 
+// Tiles up to which the near pairs are kept between the two passes (132 bytes
+// per tile: 66 MB); the block form stays far below.
+constexpr size_t KEEP_NEAR = 500000;
+
 // the arrays every evaluation needs (with base = nullptr only their size counts)
 AdjDev adj_arrays(const AdjInput &in, Carve &c) {
   const size_t na = (size_t)in.n_frames * in.n_cv;
@@ -386,19 +404,28 @@ AdjDev adj_arrays(const AdjInput &in, Carve &c) {
   a.Q = c.take<double>(in.n_frames);
   a.coef = c.take<double>(2 * (size_t)in.n_frames);
   a.phi = c.take<double>(1);
+  const size_t tiles = (size_t)in.n_frames * in.n_tiles;
+  if (tiles <= KEEP_NEAR) {
+    a.n_near = c.take<int>(tiles);
+    a.near = c.take<unsigned>(tiles * CV_T);
+  }
   return a;
 }
 
 // A block per tile up to 128 tiles per SM: these kernels run alone, so the
 // block form pays longer than beside the pair kernel (see launch_cv).  5576
 // tiles: z and grad z 72 -> 55 us, H_z w 68 -> 46; 84 303 tiles: 311 -> 350.
-bool block_form(const AdjInput &in) { return (long long)in.n_frames * in.n_tiles <= 128ll * in.n_sm; }
+bool block_form(const AdjInput &in) {
+  const long long tiles = (long long)in.n_frames * in.n_tiles;
+  return tiles <= 128ll * in.n_sm && tiles <= (long long)KEEP_NEAR;
+}
 
 void launch_adj_cv(const AdjInput &in, const AdjDev &a, cudaStream_t st) {
   const long long tiles = (long long)a.nf * a.n_tiles;
+  const unsigned grid = (unsigned)((tiles + ADJ_WARPS - 1) / ADJ_WARPS);
   if (tiles > 0) {
-    if (block_form(in)) k_adj_cv<CV_BLOCK_WARPS><<<(unsigned)tiles, 32 * CV_BLOCK_WARPS, 0, st>>>(a, in.k);
-    else k_adj_cv<1><<<(unsigned)((tiles + ADJ_WARPS - 1) / ADJ_WARPS), 32 * ADJ_WARPS, 0, st>>>(a, in.k);
+    if (block_form(in)) k_adj_cv<CV_BLOCK_WARPS, true><<<(unsigned)tiles, 32 * CV_BLOCK_WARPS, 0, st>>>(a, in.k);
+    else (a.near ? k_adj_cv<1, true> : k_adj_cv<1, false>)<<<grid, 32 * ADJ_WARPS, 0, st>>>(a, in.k);
   }
   k_adj_fin<<<a.nf, FIN_THREADS, 0, st>>>(a);
 }
@@ -408,9 +435,10 @@ void launch_adj_grad(const AdjInput &in, const AdjDev &a, double *grad, cudaStre
   const size_t na = (size_t)a.nf * a.n_cv;
   if (na == 0) return;
   cudaMemsetAsync(a.hx, 0, sizeof(long long) * 3 * na, st);
+  const unsigned grid = (unsigned)((tiles + ADJ_WARPS - 1) / ADJ_WARPS);
   if (tiles > 0) {
-    if (block_form(in)) k_adj_hw<CV_BLOCK_WARPS><<<(unsigned)tiles, 32 * CV_BLOCK_WARPS, 0, st>>>(a, in.k);
-    else k_adj_hw<1><<<(unsigned)((tiles + ADJ_WARPS - 1) / ADJ_WARPS), 32 * ADJ_WARPS, 0, st>>>(a, in.k);
+    if (block_form(in)) k_adj_hw<CV_BLOCK_WARPS, true><<<(unsigned)tiles, 32 * CV_BLOCK_WARPS, 0, st>>>(a, in.k);
+    else (a.near ? k_adj_hw<1, true> : k_adj_hw<1, false>)<<<grid, 32 * ADJ_WARPS, 0, st>>>(a, in.k);
   }
   k_adj_out<<<(unsigned)((na + 255) / 256), 256, 0, st>>>(a, grad);
 }

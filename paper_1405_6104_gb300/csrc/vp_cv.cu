@@ -77,7 +77,7 @@ __global__ void k_zconst(Dev d, const int32_t *sys_tile0, const int32_t *sys_nti
 // Two phases per (trial, tile) warp: (1) a cheap FP32 distance test of the
 // 1024 pairs of the tile lists the pairs closer than the contact cut-off in
 // shared memory; (2) the warp evaluates only those, 64 at a time (two per lane
-// on the packed FP32 instructions: 64 trials of 540 contact atoms 57 -> 50 us,
+// on the packed FP32 instructions: 64 trials of 540 contact atoms 57 -> 48 us,
 // 14 unequal trials 38 -> 30), in float-float, accumulating the gradient of the tile's 64 atoms with integer
 // shared-memory atomics (order-independent, so deterministic) and flushing it
 // once per tile.  Far pairs (C~ = 0) contribute only to the constant Z0.

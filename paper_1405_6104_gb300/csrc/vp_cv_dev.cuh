@@ -84,12 +84,19 @@ __device__ __forceinline__ ff2 cv_near_pairs(SH &sh, const CvConst &k, const CvT
   return ff2_mul(cp.Ct, ff2_sub(cp.Ct, ff2{__fadd2_rn(cnat.hi, cnat.hi), __fadd2_rn(cnat.lo, cnat.lo)}));
 }
 
-// whether a pair at the (unimaged) FP32 difference (dx, dy, dz) is closer than the contact cut-off
-__device__ __forceinline__ bool cv_is_near(float dx, float dy, float dz, float L, float iL, float rc2_far) {
-  dx -= L * rintf(dx * iL);
-  dy -= L * rintf(dy * iL);
-  dz -= L * rintf(dz * iL);
-  return dx * dx + dy * dy + dz * dz < rc2_far;
+// whether the pairs of atom xi with xj0 and with xj1 are closer than the contact
+// cut-off (FP32; a position that is not a number is near nothing)
+__device__ __forceinline__ void cv_are_near(float4 xi, float4 xj0, float4 xj1, float L, float iL, float rc2_far, bool &n0,
+                                            bool &n1) {
+  const float2 m = f2_all(12582912.0f), il = f2_all(iL), l = f2_all(-L);  // see cv_delta2
+  float2 dx = __fadd2_rn(make_float2(xj0.x, xj1.x), f2_all(-xi.x)), dy = __fadd2_rn(make_float2(xj0.y, xj1.y), f2_all(-xi.y)),
+         dz = __fadd2_rn(make_float2(xj0.z, xj1.z), f2_all(-xi.z));
+  dx = __ffma2_rn(l, f2_sub(__fadd2_rn(__fmul2_rn(dx, il), m), m), dx);
+  dy = __ffma2_rn(l, f2_sub(__fadd2_rn(__fmul2_rn(dy, il), m), m), dy);
+  dz = __ffma2_rn(l, f2_sub(__fadd2_rn(__fmul2_rn(dz, il), m), m), dz);
+  const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dx, dx, __fmul2_rn(dy, dy)));
+  n0 = r2.x < rc2_far;
+  n1 = r2.y < rc2_far;
 }
 
 // the accumulated gradient of atom a (0..63) of the tile, into the sums at gx, gy, gz
@@ -124,47 +131,72 @@ __device__ __forceinline__ bool cv_tile_far(const CvTile &t, bool iv, bool jv, f
 }
 
 // The near pairs of the tile by one warp, in rotation-major order, into
-// s_near; returns their number.  Lane l holds atom l of either block.
-__device__ __forceinline__ int cv_near_list(const CvTile &t, unsigned short *s_near, float3 xi, float3 xj) {
-  const int lane = threadIdx.x & 31;
-  const int i = t.bi * CV_T + lane;
+// s_near; returns their number.  s_x: the atoms of both blocks (not a number
+// beyond the last).  KEEP: the ballots of the 32 rotations go to kept.
+template <bool KEEP>
+__device__ __forceinline__ int cv_near_list(const CvTile &t, unsigned short *s_near, const float4 *s_x, unsigned *kept) {
+  const int lane = threadIdx.x & 31, sep = t.min_sep - (t.bj - t.bi) * CV_T + lane;
+  const float4 xi = s_x[lane];
+  const unsigned below = (1u << lane) - 1u;
   int n_near = 0;
-  for (int k = 0; k < CV_T; ++k) {
-    const int jc = (lane + k) & (CV_T - 1);
-    const int j = t.bj * CV_T + jc;
-    const float xjx = __shfl_sync(0xffffffffu, xj.x, jc);
-    const float xjy = __shfl_sync(0xffffffffu, xj.y, jc);
-    const float xjz = __shfl_sync(0xffffffffu, xj.z, jc);
-    const bool near = i < t.n_cv && j < t.n_cv && j - i > t.min_sep &&
-                      cv_is_near(xjx - xi.x, xjy - xi.y, xjz - xi.z, t.L, t.iL, t.rc2_far);
-    const unsigned bal = __ballot_sync(0xffffffffu, near);
-    if (near) s_near[n_near + __popc(bal & ((1u << lane) - 1u))] = (unsigned short)(lane | (jc << 5));
-    n_near += __popc(bal);
+#pragma unroll 2
+  for (int k = 0; k < CV_T; k += 2) {
+    const int j0 = (lane + k) & (CV_T - 1), j1 = (lane + k + 1) & (CV_T - 1);
+    bool n0, n1;
+    cv_are_near(xi, s_x[CV_T + j0], s_x[CV_T + j1], t.L, t.iL, t.rc2_far, n0, n1);
+    n0 = n0 && j0 > sep;
+    n1 = n1 && j1 > sep;
+    const unsigned b0 = __ballot_sync(0xffffffffu, n0), b1 = __ballot_sync(0xffffffffu, n1);
+    if (n0) s_near[n_near + __popc(b0 & below)] = (unsigned short)(lane | (j0 << 5));
+    n_near += __popc(b0);
+    if (n1) s_near[n_near + __popc(b1 & below)] = (unsigned short)(lane | (j1 << 5));
+    n_near += __popc(b1);
+    if (KEEP && lane == 0) *reinterpret_cast<uint2 *>(kept + k) = make_uint2(b0, b1);
   }
   return n_near;
 }
 
-// The same by a block of NW warps, the 32 rotations dealt out over them (the
-// atoms of both blocks in s_x; every thread of the block calls).
-template <int NW>
-__device__ __forceinline__ int cv_near_list_block(const CvTile &t, unsigned short *s_near, unsigned *s_bal,
-                                                  const float4 *s_x) {
-  constexpr int KW = CV_T / NW;  // rotations per warp
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int i = t.bi * CV_T + lane;
-  const float4 xi = s_x[lane];
-  unsigned bal[KW];
+// The same from kept ballots (in no particular order).
+__device__ __forceinline__ int cv_near_list_kept(unsigned short *s_near, const unsigned *kept) {
+  const int lane = threadIdx.x & 31;
+  unsigned m = kept[lane];  // lane k: rotation k
+  int incl = __popc(m);
 #pragma unroll
-  for (int q = 0; q < KW; ++q) {
-    const int jc = (lane + warp * KW + q) & (CV_T - 1);
-    const int j = t.bj * CV_T + jc;
-    const float4 x = s_x[CV_T + jc];
-    const bool near = i < t.n_cv && j < t.n_cv && j - i > t.min_sep &&
-                      cv_is_near(x.x - xi.x, x.y - xi.y, x.z - xi.z, t.L, t.iL, t.rc2_far);
-    bal[q] = __ballot_sync(0xffffffffu, near);
-    if (lane == 0) s_bal[warp * KW + q] = bal[q];
+  for (int off = 1; off < 32; off <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, incl, off);
+    if (lane >= off) incl += v;
   }
-  __syncthreads();
+  for (int p = incl - __popc(m); m; m &= m - 1u) {
+    const int i = __ffs(m) - 1;
+    s_near[p++] = (unsigned short)(i | (((i + lane) & (CV_T - 1)) << 5));
+  }
+  return __shfl_sync(0xffffffffu, incl, 31);
+}
+
+// The same by a block of NW warps, the 32 rotations dealt out over them: the
+// ballots into s_bal ...
+template <int NW>
+__device__ __forceinline__ void cv_ballots_block(const CvTile &t, unsigned *s_bal, const float4 *s_x) {
+  constexpr int KW = CV_T / NW;  // rotations per warp
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sep = t.min_sep - (t.bj - t.bi) * CV_T + lane;
+  const float4 xi = s_x[lane];
+#pragma unroll
+  for (int q = 0; q < KW; q += 2) {
+    const int k = warp * KW + q, j0 = (lane + k) & (CV_T - 1), j1 = (lane + k + 1) & (CV_T - 1);
+    bool n0, n1;
+    cv_are_near(xi, s_x[CV_T + j0], s_x[CV_T + j1], t.L, t.iL, t.rc2_far, n0, n1);
+    const unsigned b0 = __ballot_sync(0xffffffffu, n0 && j0 > sep), b1 = __ballot_sync(0xffffffffu, n1 && j1 > sep);
+    if (lane == 0) {
+      s_bal[k] = b0;
+      s_bal[k + 1] = b1;
+    }
+  }
+}
+// ... and the list from them (every thread of the block calls, after a barrier)
+template <int NW>
+__device__ __forceinline__ int cv_near_list_block(unsigned short *s_near, const unsigned *s_bal) {
+  constexpr int KW = CV_T / NW;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int incl = __popc(s_bal[lane]);
 #pragma unroll
   for (int off = 1; off < 32; off <<= 1) {
@@ -173,19 +205,28 @@ __device__ __forceinline__ int cv_near_list_block(const CvTile &t, unsigned shor
   }
 #pragma unroll
   for (int q = 0; q < KW; ++q) {
+    const unsigned bal = s_bal[warp * KW + q];
     const int end = __shfl_sync(0xffffffffu, incl, warp * KW + q);
-    if ((bal[q] >> lane) & 1u)
-      s_near[end - __popc(bal[q]) + __popc(bal[q] & ((1u << lane) - 1u))] =
+    if ((bal >> lane) & 1u)
+      s_near[end - __popc(bal) + __popc(bal & ((1u << lane) - 1u))] =
           (unsigned short)(lane | (((lane + warp * KW + q) & (CV_T - 1)) << 5));
   }
   __syncthreads();
   return __shfl_sync(0xffffffffu, incl, 31);
 }
 
+// an atom of a tile; one beyond the last is not a number, and so near nothing
+__device__ __forceinline__ float4 cv_atom(bool valid, float3 x) {
+  return valid ? make_float4(x.x, x.y, x.z, 0.f) : make_float4(NAN, NAN, NAN, 0.f);
+}
+
 // One warp's tile: z partial sum and gradient.  pos(a): position of
 // reaction-coordinate atom a.
-template <class POS>
-__device__ __forceinline__ void cv_tile(const CvTile &t, const CvConst &k, CvWarpShared &sh, POS pos) {
+// KEEP: the number of near pairs and the ballots that list them are left at
+// n_kept and kept, for a later pass over the same pairs.
+template <bool KEEP = false, class POS>
+__device__ __forceinline__ void cv_tile(const CvTile &t, const CvConst &k, CvWarpShared &sh, POS pos,
+                                        int *n_kept = nullptr, unsigned *kept = nullptr) {
   const int lane = threadIdx.x & 31;
   const int i = t.bi * CV_T + lane, j = t.bj * CV_T + lane;
   const bool iv = i < t.n_cv, jv = j < t.n_cv;
@@ -194,16 +235,19 @@ __device__ __forceinline__ void cv_tile(const CvTile &t, const CvConst &k, CvWar
   if (jv) xj = pos(j);
   if (cv_tile_far(t, iv, jv, xi, xj)) {
     if (lane == 0) *t.z_part = 0.0;
+    if (KEEP && lane == 0) *n_kept = 0;
     return;
   }
-  sh.s_x[lane] = make_float4(xi.x, xi.y, xi.z, 0.f);
-  sh.s_x[CV_T + lane] = make_float4(xj.x, xj.y, xj.z, 0.f);
+  sh.s_x[lane] = cv_atom(iv, xi);
+  sh.s_x[CV_T + lane] = cv_atom(jv, xj);
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
     sh.s_ghi[lane][q] = 0; sh.s_ghi[CV_T + lane][q] = 0;
     sh.s_glo[lane][q] = 0; sh.s_glo[CV_T + lane][q] = 0;
   }
-  const int n_near = cv_near_list(t, sh.s_near, xi, xj);
+  __syncwarp();
+  const int n_near = cv_near_list<KEEP>(t, sh.s_near, sh.s_x, kept);
+  if (KEEP && lane == 0) *n_kept = n_near;
   __syncwarp();
   // the near pairs, densely
   ff zacc = {0.f, 0.f};
@@ -247,7 +291,7 @@ __device__ __forceinline__ bool cv_block_begin(const CvTile &t, SH &sh, POS pos)
     const int a = (warp == 0 ? t.bi : t.bj) * CV_T + lane;
     float3 q = make_float3(0.f, 0.f, 0.f);
     if (a < t.n_cv) q = pos(a);
-    sh.s_x[threadIdx.x] = make_float4(q.x, q.y, q.z, 0.f);
+    sh.s_x[threadIdx.x] = cv_atom(a < t.n_cv, q);
   }
   for (int q = threadIdx.x; q < 2 * CV_T * 3; q += NW * 32) {
     (&sh.s_ghi[0][0])[q] = 0;
@@ -259,14 +303,22 @@ __device__ __forceinline__ bool cv_block_begin(const CvTile &t, SH &sh, POS pos)
                      make_float3(sh.s_x[CV_T + lane].x, sh.s_x[CV_T + lane].y, sh.s_x[CV_T + lane].z));
 }
 
-template <int NW, class POS>
-__device__ __forceinline__ void cv_tile_block(const CvTile &t, const CvConst &k, CvBlockShared &sh, POS pos) {
+template <int NW, bool KEEP = false, class POS>
+__device__ __forceinline__ void cv_tile_block(const CvTile &t, const CvConst &k, CvBlockShared &sh, POS pos,
+                                              int *n_kept = nullptr, unsigned *kept = nullptr) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (cv_block_begin<NW>(t, sh, pos)) {
     if (threadIdx.x == 0) *t.z_part = 0.0;
+    if (KEEP && threadIdx.x == 0) *n_kept = 0;
     return;
   }
-  const int n_near = cv_near_list_block<NW>(t, sh.s_near, sh.s_bal, sh.s_x);
+  cv_ballots_block<NW>(t, sh.s_bal, sh.s_x);
+  __syncthreads();
+  const int n_near = cv_near_list_block<NW>(sh.s_near, sh.s_bal);
+  if (KEEP && warp == NW - 1) {
+    kept[lane] = sh.s_bal[lane];
+    if (lane == 0) *n_kept = n_near;
+  }
   // 64 pairs per warp at a time: warps without any leave their issue slots to the others
   for (int p = 64 * warp + lane; p < n_near; p += 64 * NW) {
     const int p1 = p + 32;

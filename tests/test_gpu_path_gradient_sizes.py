@@ -72,6 +72,22 @@ def test_tiles_by_a_block_match_tiles_by_a_warp(n_solute):
     assert (zz.reshape(reps, 3) == z).all() and (gg.reshape(reps, *g.shape) == g).all()
 
 
+@pytest.mark.parametrize("n_solute", [12, 33])
+def test_near_pairs_kept_match_near_pairs_listed_again(n_solute):
+    """Beyond 500 000 tiles the second pass lists the near pairs itself: equal
+    bits with a short call, whose first pass keeps them."""
+    s, p = S.small_solvated(n_solute=n_solute, n_water=430 + n_solute)
+    rng = np.random.default_rng(n_solute)
+    frames = s.native_pos * np.array([0.4, 1.0, 2.5])[:, None, None] + 0.01 * rng.normal(size=(3, n_solute, 3))
+    coef = rng.normal(size=(3, 2))
+    reps = 500_000 // (3 * (1 if n_solute <= 32 else 3)) + 2
+    with B.TrialBatch(s, p, [1]) as b:
+        _, z, g = B.phi_frames_adjoint(b.h, 0, frames, coef)
+        _, zz, gg = B.phi_frames_adjoint(b.h, 0, np.concatenate([frames] * reps), np.concatenate([coef] * reps))
+    assert np.abs(g).max() > 0.0
+    assert (zz.reshape(reps, 3) == z).all() and (gg.reshape(reps, *g.shape) == g).all()
+
+
 @pytest.mark.parametrize("r0", [1e-3, 0.05])
 def test_steep_contacts(r0):
     """Contacts so steep that a pair's gradient and Hessian terms pass the
