@@ -432,8 +432,9 @@ __global__ void __launch_bounds__(32, MINB) k_pair_w(Dev d, SimConst c, const in
   pair_cluster_f2<U>(d, c, sh, clist ? clist[item] : item);
 }
 
-// Forces and nonbonded energies in one pass over the lists (24 warps per SM: 163
-// us for 16 configurations of 11 040 atoms; 20: 203, 28: 174).
+// Forces and nonbonded energies in one pass over the lists (24 warps per SM: 132
+// us for 16 configurations of 11 040 atoms, 162 with the energy terms scalar and
+// behind a branch per pair; 16 warps 150, 20: 138, 28: 161).
 __global__ void __launch_bounds__(32, 24) k_pair_e(Dev d, SimConst c) {
   __shared__ PairF2Shared<1, true> sh;
   pair_cluster_f2<1, 1, true>(d, c, sh, blockIdx.x);

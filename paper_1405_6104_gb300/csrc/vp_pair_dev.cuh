@@ -22,8 +22,8 @@ constexpr float MASK_PEN = 1.0e30f;
 // row of an i-force component's 32 partial sums: 16-byte loads without bank conflicts
 constexpr int RED_STRIDE = 36;
 
-// the energies' tables of a warp: {c12, c12', c6, c6'} (over r^12 and r^6) and the
-// potential at the cut-off per i-atom pair and type
+// the energies' tables of a warp: {c12, c12', -c6, -c6'} (over r^12 and r^6) and
+// minus the potential at the cut-off per i-atom pair and type
 template <int NW, bool ENERGY>
 struct PairEnergyTables {
   float4 s_e4[NW][CL / 2][SMALL_TYPES];
@@ -115,8 +115,8 @@ __device__ __forceinline__ void pair_cluster_f2(const Dev &d, const SimConst &c,
       s_c4[wib][p][tj] = make_float4(c0.y, c1.y, -c0.x, -c1.x);
       if constexpr (ENERGY) {
         sh.s_e4[wib][p][tj] = make_float4(__fmul_rn(c0.y, 1.0f / 12.0f), __fmul_rn(c1.y, 1.0f / 12.0f),
-                                          __fmul_rn(c0.x, 1.0f / 6.0f), __fmul_rn(c1.x, 1.0f / 6.0f));
-        sh.s_ts[wib][p][tj] = make_float2(d.ljshift[ty[r][0] * NT + tj], d.ljshift[ty[r][1] * NT + tj]);
+                                          -__fmul_rn(c0.x, 1.0f / 6.0f), -__fmul_rn(c1.x, 1.0f / 6.0f));
+        sh.s_ts[wib][p][tj] = make_float2(-d.ljshift[ty[r][0] * NT + tj], -d.ljshift[ty[r][1] * NT + tj]);
       }
     }
   }
@@ -131,14 +131,18 @@ __device__ __forceinline__ void pair_cluster_f2(const Dev &d, const SimConst &c,
   const float2 m2krf = make_float2(-c.two_krf, -c.two_krf);
   const float rc2 = c.rc2;
   float elj = 0.0f, erf = 0.0f;
-  // the energies of one pair inside the cut-off (hh: which i-atom of pair p)
-  auto add_energy = [&](int tj, int p, int hh, float rinv, float rinv6, float r2, float qq) {
+  // the energies of the pairs inside the cut-off of i-atom pair p, added in the
+  // order of the i-atoms (a pair that is left out may be inf or NaN)
+  auto add_energies = [&](int tj, int p, float2 rinv, float2 rinv6, float2 r2, float2 qq, bool inx, bool iny) {
     if constexpr (ENERGY) {
       const float4 e = sh.s_e4[wib][p][tj];
-      const float2 ts = sh.s_ts[wib][p][tj];
-      const float lj = __fmaf_rn(hh ? e.y : e.x, rinv6, -(hh ? e.w : e.z));
-      elj = __fadd_rn(elj, __fmaf_rn(rinv6, lj, -(hh ? ts.y : ts.x)));
-      erf = __fmaf_rn(qq, __fsub_rn(__fmaf_rn(c.krf, r2, rinv), c.crf), erf);
+      const float2 lj = __ffma2_rn(make_float2(e.x, e.y), rinv6, make_float2(e.z, e.w));
+      const float2 el = __ffma2_rn(rinv6, lj, sh.s_ts[wib][p][tj]);
+      const float2 rf = __fadd2_rn(__ffma2_rn(make_float2(c.krf, c.krf), r2, rinv), make_float2(-c.crf, -c.crf));
+      elj = inx ? __fadd_rn(elj, el.x) : elj;
+      erf = inx ? __fmaf_rn(qq.x, rf.x, erf) : erf;
+      elj = iny ? __fadd_rn(elj, el.y) : elj;
+      erf = iny ? __fmaf_rn(qq.y, rf.y, erf) : erf;
     }
   };
 
@@ -188,10 +192,7 @@ __device__ __forceinline__ void pair_cluster_f2(const Dev &d, const SimConst &c,
                iny = (!MASKED || (mb & (1u << (2 * p + 1)))) && r2.y < rc2;
     f.x = inx ? f.x : 0.0f;
     f.y = iny ? f.y : 0.0f;
-    if constexpr (ENERGY) {
-      if (inx) add_energy(j.tj, p, 0, rinv.x, rinv6.x, r2.x, qq.x);
-      if (iny) add_energy(j.tj, p, 1, rinv.y, rinv6.y, r2.y, qq.y);
-    }
+    add_energies(j.tj, p, rinv, rinv6, r2, qq, inx, iny);
     fx[p] = __ffma2_rn(f, dx, fx[p]);
     fy[p] = __ffma2_rn(f, dy, fy[p]);
     fz[p] = __ffma2_rn(f, dz, fz[p]);
@@ -220,7 +221,7 @@ __device__ __forceinline__ void pair_cluster_f2(const Dev &d, const SimConst &c,
       for (int p = 0; p < CL / 2; ++p) {
         const float4 i0 = s_ip[wib][p][0], i1 = s_ip[wib][p][1];
         const float4 cc = j.row[p * TS];
-        float2 f2v, dx2, dy2, dz2;
+        float2 f2v, dx2, dy2, dz2, rinv_2, rinv6_2, r2_2, qq_2;
 #pragma unroll
         for (int hh = 0; hh < 2; ++hh) {
           const float pen = (mb & (1u << (2 * p + hh))) ? 0.0f : MASK_PEN;
@@ -241,11 +242,11 @@ __device__ __forceinline__ void pair_cluster_f2(const Dev &d, const SimConst &c,
           tt = __fmaf_rn(qq, rinv, tt);
           tt = __fmul_rn(tt, rinv2);
           float f = __fmaf_rn(qq, -c.two_krf, tt);
-          if (ENERGY && r2 < rc2) add_energy(j.tj, p, hh, rinv, rinv6, r2, qq);
           f = r2 < rc2 ? f : 0.0f;
-          if (hh) { f2v.y = f; dx2.y = dx; dy2.y = dy; dz2.y = dz; }
-          else { f2v.x = f; dx2.x = dx; dy2.x = dy; dz2.x = dz; }
+          if (hh) { f2v.y = f; dx2.y = dx; dy2.y = dy; dz2.y = dz; rinv_2.y = rinv; rinv6_2.y = rinv6; r2_2.y = r2; qq_2.y = qq; }
+          else { f2v.x = f; dx2.x = dx; dy2.x = dy; dz2.x = dz; rinv_2.x = rinv; rinv6_2.x = rinv6; r2_2.x = r2; qq_2.x = qq; }
         }
+        add_energies(j.tj, p, rinv_2, rinv6_2, r2_2, qq_2, r2_2.x < rc2, r2_2.y < rc2);
         fx[p] = __ffma2_rn(f2v, dx2, fx[p]);
         fy[p] = __ffma2_rn(f2v, dy2, fy[p]);
         fz[p] = __ffma2_rn(f2v, dz2, fz[p]);
