@@ -48,11 +48,12 @@ struct PairF2Shared : PairEnergyTables<NW, ENERGY> {
 // evaluated, interleaves the two groups' arithmetic (two independent chains
 // per warp) and reads each i-atom pair from shared memory once for both: 96
 // registers, 20 warps per SM, and still faster at every batch size (64 x
-// 11 040 atoms 371 us against 419 with U = 1 and 24 warps; one trial 13
+// 11 040 atoms 366 us against 419 with U = 1 and 24 warps; one trial 13
 // against 20 us; U = 3 and 4, U = 2 without the early loads, or two iterations
 // unrolled (456 us: too much code for the instruction cache) are slower).  An
 // odd last group is taken by itself (an idle second one and the wider loads of
-// the i-force sums were 2.7% of the time).
+// the i-force sums were 2.7% of the time, loading the masked groups' j-atoms when
+// they are due another 1.3%).
 // Every accumulator takes its terms in the order of the groups either way:
 // the same forces bit for bit.
 // ENERGY (U = 1): the Lennard-Jones and reaction-field energies too, each lane
@@ -283,6 +284,19 @@ __device__ __forceinline__ void pair_cluster_f2(const Dev &d, const SimConst &c,
   } else {
     const int e1 = (min(nm, n) + 31) & ~31;  // the groups from here on need no masks
     auto entry = [&](int e) { return e < n ? __ldcs(seg + e) : d.idle_entry; };
+    // the masked groups' j-atoms are loaded a group ahead
+    uint32_t em_n = 0u;
+    float4 pm_n = make_float4(0.f, 0.f, 0.f, 0.f);
+    int tm_n = 0;
+    unsigned mb_n = 0u;
+    auto masked_load = [&](int e0) {
+      const uint32_t w = e0 == 0 ? raw0 : e0 == 32 ? raw1 : entry(e0 + lane);
+      em_n = e0 + lane < n ? w : d.idle_entry;
+      pm_n = d.pos[em_n & J_MASK];
+      tm_n = d.type[em_n & J_MASK];
+      mb_n = e0 + lane < n ? segm[e0 + lane] : 0u;
+    };
+    if (e1 > 0) masked_load(0);
     // the first U clean groups' j-atoms and the next ones' entries are in
     // flight while the masked groups are evaluated
     uint32_t ent[U], ent_n[U];
@@ -298,9 +312,12 @@ __device__ __forceinline__ void pair_cluster_f2(const Dev &d, const SimConst &c,
       tj[u] = d.type[ent[u] & J_MASK];
     }
     for (int e0 = 0; e0 < e1; e0 += 32) {
-      const uint32_t w = e0 == 0 ? raw0 : e0 == 32 ? raw1 : entry(e0 + lane);
-      const uint32_t em = e0 + lane < n ? w : d.idle_entry;
-      masked_group(d.pos[em & J_MASK], d.type[em & J_MASK], em, e0 + lane < n ? segm[e0 + lane] : 0u);
+      const uint32_t em = em_n;
+      const float4 pm = pm_n;
+      const int tm = tm_n;
+      const unsigned mb = mb_n;
+      if (e0 + 32 < e1) masked_load(e0 + 32);
+      masked_group(pm, tm, em, mb);
     }
     int e0 = e1;
     for (; e0 + 32 < n; e0 += 32 * U) {
