@@ -289,7 +289,7 @@ int sim_diagnostics(sim_handle *h, int64_t *out);
  * one warp per block, two groups of list entries at a time, 20 or 16 warps
  * per SM; 5, 6: persistent blocks, two groups at a time, 4 or 5 blocks per
  * SM; 7, 8: one group at a time, 6 or 7 blocks; all give bit-identical
- * forces; an untuned batch takes 0, 3 or 6 by its types and size) and of the
+ * forces; an untuned batch takes 0, 3, 4 or 6 by its types and size) and of the
  * reaction-coordinate kernel
  * (2, 4 or 8 warps per block) on this batch, reps launches each, into scratch
  * accumulators (the state is untouched), and uses the fastest from then on.
