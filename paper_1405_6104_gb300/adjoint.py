@@ -139,8 +139,8 @@ def trajectory_adjoint(batch, trial: int, n_steps: int, every: int = 50, keep_fr
         lo = 0 if s == 0 else 1
         frames = seg_frames[lo:]
         rows = slice(s * every + lo, s * every + every + 1)
-        _, _, G = B.phi_frames_adjoint(h, trial, frames, coef=coef[rows])
-        grad[rows] = G
+        # straight into the result: an array of its own per segment would be fresh memory each time
+        B.phi_frames_adjoint(h, trial, frames, coef=coef[rows], out=grad[rows])
         if keep_frames:
             replayed[rows] = frames
 

@@ -309,14 +309,19 @@ def sim_trial_seed(h, trial: int) -> int:
     return int(v.value)
 
 
-def phi_frames_adjoint(h, trial: int, frames, coef=None):
-    """(Phi or None, z per frame, dPhi/dframes) for frames (n_frames, n_cv, 3)."""
+def phi_frames_adjoint(h, trial: int, frames, coef=None, out=None):
+    """(Phi or None, z per frame, dPhi/dframes) for frames (n_frames, n_cv, 3);
+    out: where the gradient goes (FP64, C-contiguous, the frames' shape), or a
+    new array."""
     F = np.ascontiguousarray(np.asarray(frames, np.float64))
     nf, ncv = F.shape[0], F.shape[1]
     Cf = None if coef is None else np.ascontiguousarray(np.asarray(coef, np.float64).reshape(-1))
     phi = np.zeros(1)
     z = np.zeros(nf)
-    G = np.zeros((nf, ncv, 3))
+    if out is not None and (out.shape != (nf, ncv, 3) or out.dtype != np.float64 or not out.flags.c_contiguous
+                            or not out.flags.writeable):
+        raise ValueError(f"out must be a writeable C-contiguous float64 array of shape {(nf, ncv, 3)}")
+    G = np.zeros((nf, ncv, 3)) if out is None else out
     _check(h, load().phi_frames_adjoint(h, int(trial), F.ctypes.data, nf, _ptr(Cf), phi.ctypes.data, z.ctypes.data,
                                         G.ctypes.data))
     return (None if coef is not None else float(phi[0])), z, G
