@@ -414,7 +414,8 @@ AdjDev adj_arrays(const AdjInput &in, Carve &c) {
 
 // A block per tile up to 128 tiles per SM: these kernels run alone, so the
 // block form pays longer than beside the pair kernel (see launch_cv).  5576
-// tiles: z and grad z 72 -> 55 us, H_z w 68 -> 46; 84 303 tiles: 311 -> 350.
+// tiles: z and grad z 62 -> 50 us, H_z w 56 -> 37; 84 303 tiles: 277 -> 332 and
+// 230 -> 261.
 bool block_form(const AdjInput &in) {
   const long long tiles = (long long)in.n_frames * in.n_tiles;
   return tiles <= 128ll * in.n_sm && tiles <= (long long)KEEP_NEAR;
