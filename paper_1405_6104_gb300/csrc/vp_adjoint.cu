@@ -235,9 +235,9 @@ __device__ __forceinline__ void adj_hw_pairs(AdjHwShared &sh, const CvTile &t, c
                vz = f2_sub(make_float2(wj0.z, wj1.z), make_float2(wi0.z, wi1.z));
   const float2 uv = __ffma2_rn(uz, vz, __ffma2_rn(ux, vx, __fmul2_rn(uy, vy)));
   const float2 q = __fmul2_rn(f1, ir);
-  const float2 g[3] = {__ffma2_rn(__fmul2_rn(f2, ux), uv, __fmul2_rn(q, f2_nma(ux, uv, vx))),
-                       __ffma2_rn(__fmul2_rn(f2, uy), uv, __fmul2_rn(q, f2_nma(uy, uv, vy))),
-                       __ffma2_rn(__fmul2_rn(f2, uz), uv, __fmul2_rn(q, f2_nma(uz, uv, vz)))};
+  const float2 g[3] = {__ffma2_rn(q, f2_nma(ux, uv, vx), __fmul2_rn(__fmul2_rn(f2, ux), uv)),
+                       __ffma2_rn(q, f2_nma(uy, uv, vy), __fmul2_rn(__fmul2_rn(f2, uy), uv)),
+                       __ffma2_rn(q, f2_nma(uz, uv, vz), __fmul2_rn(__fmul2_rn(f2, uz), uv))};
   cv_accumulate(sh, t, g, il0, jc0, il1, jc1, true, v1);
 }
 
