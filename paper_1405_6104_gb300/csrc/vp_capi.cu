@@ -573,6 +573,7 @@ VP_API int sim_create(const sim_system *systems, int32_t n_systems, const int32_
   ff_split(1.0 / (p.cv_r_cut - p.cv_r_switch), c.cv_inv_w_hi, c.cv_inv_w_lo);
   c.cv_rs2 = (float)(p.cv_r_switch * p.cv_r_switch);
   c.cv_rc2_far = (float)(p.cv_r_cut * p.cv_r_cut * (1.0 + 1e-4));
+  c.cv_steep = p.cv_r_cut * p.cv_r_cut > 1000.0 * p.cv_r0 * p.cv_r0;
   c.cv_r0_d = p.cv_r0;
   c.cv_rs_d = p.cv_r_switch;
   c.cv_rc_d = p.cv_r_cut;
@@ -1393,7 +1394,7 @@ AdjInput adj_input(sim_handle *h, int trial) {
   in.iL = T.inv_box;
   const SimConst &c = h->c;
   in.k = CvConst{ff{c.cv_inv_r0sq_hi, c.cv_inv_r0sq_lo}, ff{c.cv_rs_hi, c.cv_rs_lo}, ff{c.cv_inv_w_hi, c.cv_inv_w_lo},
-                 c.cv_rs2, c.cv_rc2_far};
+                 c.cv_rs2, c.cv_rc2_far, c.cv_steep};
   in.c = h->c.dt_d * h->c.kR_half_d * h->c.kR_half_d;
   in.zconst = h->zconst[trial];
   return in;

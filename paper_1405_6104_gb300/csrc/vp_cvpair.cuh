@@ -11,11 +11,12 @@ namespace vp {
 struct CvConst {
   ff inv_r0sq, rs, inv_w;
   float rs2, rc2_far;
+  int steep;  // a near pair may have s > 1000: its D^3 may leave the FP32 range
 };
 
 __device__ __forceinline__ CvConst cv_const(const SimConst &c) {
   return CvConst{ff{c.cv_inv_r0sq_hi, c.cv_inv_r0sq_lo}, ff{c.cv_rs_hi, c.cv_rs_lo}, ff{c.cv_inv_w_hi, c.cv_inv_w_lo},
-                 c.cv_rs2, c.cv_rc2_far};
+                 c.cv_rs2, c.cv_rc2_far, c.cv_steep};
 }
 
 // Two near pairs per lane, on the packed FP32 instructions (two operations per
@@ -75,9 +76,15 @@ __device__ __forceinline__ ff2 ff2_div(ff2 x, ff2 y) {
 
 // Correctly rounded quotients and roots by Markstein's final step (IBM J. Res.
 // Dev. 34, 1990): a Newton step on the hardware's approximation gives the
-// correctly rounded reciprocal (every one of the 2^23 significands was
-// compared), and one on the quotient's (root's) remainder the correctly
-// rounded result.  For operands and results away from the range's ends.
+// correctly rounded reciprocal, and one on the quotient's (root's) remainder the
+// correctly rounded result.  The hardware's approximations are not specified
+// closely enough to prove that, so the tests compare every significand of
+// reciprocals and roots, and quotients next to a midpoint, with the operators.  For
+// numbers away from the range's ends: a denominator lies below RCP_TOP (from there
+// on its reciprocal is denormal, which the approximation flushes, and an infinite
+// one gives NaN), a radicand or dividend not below 2^-100 (its remainder would be
+// denormal; smaller dividends occur in terms far below the sums' unit of 2^-32).
+constexpr float RCP_TOP = 8.507059e37f;  // 2^126
 __device__ __forceinline__ float rcp_approx(float x) {
   float y;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -107,6 +114,18 @@ struct CvPair2 {
   float2 dCt, d2Ct, r;
 };
 
+// C'(s) and (SECOND) C''(s) without the powers of D, whose FP32 range ends at
+// r = 255 r0 (D^2) and 40 r0 (D^3): every quotient is over D itself.  Beside the
+// usual form, for the pairs that need it: the usual one takes a third of the
+// quotients, and its results stay what they were.
+template <bool SECOND>
+__device__ __forceinline__ float2 cv_far_slopes(float t) {
+  const float N = 1.0f + t + t * t, D = N + t * t * t + t * t * t * t;
+  const float n = N / D, n1 = (1.0f + 2.0f * t) / D, d1 = (1.0f + 2.0f * t + 3.0f * t * t + 4.0f * t * t * t) / D;
+  const float Cs = n1 - n * d1;
+  return make_float2(Cs, SECOND ? 2.0f / D - n * ((2.0f + 6.0f * t + 12.0f * t * t) / D) - 2.0f * d1 * Cs : 0.0f);
+}
+
 template <bool SECOND>
 __device__ __forceinline__ CvPair2 cv_contact2(ff2 r2, const CvConst &k) {
   CvPair2 o;
@@ -125,16 +144,22 @@ __device__ __forceinline__ CvPair2 cv_contact2(ff2 r2, const CvConst &k) {
   const float2 N1 = __ffma2_rn(t, f2_all(2.0f), f2_all(1.0f));
   const float2 D1 = __ffma2_rn(__fmul2_rn(__fmul2_rn(t, f2_all(4.0f)), t), t, __ffma2_rn(__fmul2_rn(t, f2_all(3.0f)), t, N1));
   const float2 W = __ffma2_rn(N1, D, f2_neg(__fmul2_rn(N, D1))), DD = __fmul2_rn(D, D);
-  const float2 Cs = f2_div(W, DD, f2_rcp(DD));
-  o.dCt = __fmul2_rn(Cs, ds);
+  float2 Cs = f2_div(W, DD, f2_rcp(DD));
+  float2 d2 = f2_all(0.0f), top = DD;  // top: the largest denominator
   if (SECOND) {
     const float2 D2 = __ffma2_rn(__fmul2_rn(t, f2_all(12.0f)), t, __ffma2_rn(t, f2_all(6.0f), f2_all(2.0f)));
     const float2 A1 = f2_nma(N, D2, __fadd2_rn(D, D));
     const float2 num = __ffma2_rn(A1, D, f2_neg(__fmul2_rn(__fadd2_rn(D1, D1), W)));
-    const float2 DDD = __fmul2_rn(DD, D);
-    const float2 d2 = f2_div(num, DDD, f2_rcp(DDD));
-    o.d2Ct = __ffma2_rn(__fadd2_rn(Cs, Cs), f2_all(k.inv_r0sq.hi), __fmul2_rn(__fmul2_rn(d2, ds), ds));
+    top = __fmul2_rn(DD, D);
+    d2 = f2_div(num, top, f2_rcp(top));
   }
+  if (k.steep) {
+    if (!(top.x < RCP_TOP)) { const float2 v = cv_far_slopes<SECOND>(t.x); Cs.x = v.x; d2.x = v.y; }
+    if (!(top.y < RCP_TOP)) { const float2 v = cv_far_slopes<SECOND>(t.y); Cs.y = v.x; d2.y = v.y; }
+  }
+  o.dCt = __fmul2_rn(Cs, ds);
+  if (SECOND)
+    o.d2Ct = __ffma2_rn(__fadd2_rn(Cs, Cs), f2_all(k.inv_r0sq.hi), __fmul2_rn(__fmul2_rn(d2, ds), ds));
   const bool sx = r2.hi.x > k.rs2, sy = r2.hi.y > k.rs2;
   if (sx || sy) {
     // ff_sqrt, from the root already there

@@ -140,6 +140,7 @@ struct SimConst {
   float cv_rs_hi, cv_rs_lo;               // switching start as float-float
   float cv_inv_w_hi, cv_inv_w_lo;         // 1/(r_cut^cv - r_switch) as float-float
   float cv_rs2, cv_rc2_far;   // switching start^2, far threshold on r^2
+  int32_t cv_steep;    // r_cut > 31 r0: see CvConst
   double cv_r0_d, cv_rs_d, cv_rc_d;
   int32_t cv_min_sep;
   int32_t rec_cap;
