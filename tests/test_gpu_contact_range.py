@@ -1,5 +1,6 @@
 """Contact parameters and frames at the ends of what the path gradient takes:
-pairs at distances far beyond a small contact radius, against the FP64 oracle."""
+pairs at distances far beyond a small contact radius, or next to none, against
+the FP64 oracle."""
 import numpy as np
 import pytest
 
@@ -46,3 +47,20 @@ def test_pairs_far_beyond_the_contact_radius(r0):
     d = np.linalg.norm(frames[1, :6, None] - frames[1, None, 6:], axis=2)
     assert ((d > 0.9) & (d < 1.2) & (d > 40 * r0)).sum() > 5
     _check(s, p, frames)
+
+
+def test_atoms_that_all_but_coincide():
+    """1e-20 nm apart (r^2 below the normal FP32 range): the oracle's gradient;
+    exactly at one place: the same, C' and C'' vanish there."""
+    s, p = S.tiny_chain(0)
+    rng = np.random.default_rng(6)
+    frames = np.stack([s.native_pos * f for f in (1.0, 0.7, 0.8)]) + 0.02 * rng.normal(size=(3, s.n_cv, 3))
+    frames = frames.astype(np.float32).astype(np.float64)
+    frames[1, [0, 6]] = 0.0
+    frames[1, 6, 1] = 1e-20
+    _check(s, p, frames)
+    with B.TrialBatch(s, p, [1]) as b:
+        _, z, G = B.phi_frames_adjoint(b.h, 0, frames)
+        frames[1, 6, 1] = 0.0
+        _, z0, G0 = B.phi_frames_adjoint(b.h, 0, frames)
+    assert np.array_equal(z, z0) and np.array_equal(G, G0)
