@@ -240,7 +240,7 @@ int sim_get_frames(sim_handle *h, double *out, int64_t out_len);
  *   frames [n_frames][n_cv][3] host; coef [2*n_frames] host (A_n, B_n) or NULL
  *   to derive them from these frames with z_m starting at frame 0 (then *phi,
  *   if not NULL, receives Phi along them); z [n_frames] (may be NULL) receives
- *   z(X_n); grad [n_frames][n_cv][3] host output. */
+ *   z(X_n); grad [n_frames][n_cv][3] host output (may be frames itself). */
 int phi_frames_adjoint(sim_handle *h, int32_t trial, const double *frames, int32_t n_frames, const double *coef,
                        double *phi, double *z, double *grad);
 

@@ -311,8 +311,8 @@ def sim_trial_seed(h, trial: int) -> int:
 
 def phi_frames_adjoint(h, trial: int, frames, coef=None, out=None):
     """(Phi or None, z per frame, dPhi/dframes) for frames (n_frames, n_cv, 3);
-    out: where the gradient goes (FP64, C-contiguous, the frames' shape), or a
-    new array."""
+    out: where the gradient goes (FP64, C-contiguous, the frames' shape; may be
+    frames itself), or a new array."""
     F = np.ascontiguousarray(np.asarray(frames, np.float64))
     nf, ncv = F.shape[0], F.shape[1]
     Cf = None if coef is None else np.ascontiguousarray(np.asarray(coef, np.float64).reshape(-1))

@@ -480,9 +480,13 @@ int adjoint_frames(const AdjInput &in, AdjWorkspace &ws, cudaStream_t st, std::s
   }
   // The copy back is several times slower into memory that no one has touched
   // yet (a fresh array of 2 MB: 1.1 ms a call against 0.35): its pages are
-  // touched here, while the kernels run.
-  if (e == cudaSuccess && in.grad)
-    for (size_t k = 0; k < nx; k += 4096 / sizeof(double)) *(volatile double *)(in.grad + k) = 0.0;
+  // touched here, while the kernels run.  Every byte keeps its value: grad may be
+  // frames itself, whose copy to the device, from page-locked memory, may not have
+  // read it yet.
+  if (e == cudaSuccess && in.grad) {
+    volatile char *g = reinterpret_cast<volatile char *>(in.grad);
+    for (size_t k = 0; k < nx * sizeof(double); k += 4096) g[k] = g[k];
+  }
   if (e == cudaSuccess && in.grad) e = cudaMemcpyAsync(in.grad, dgrad, sizeof(double) * nx, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess && in.z_out) e = cudaMemcpyAsync(in.z_out, a.z, sizeof(double) * nf, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess && in.Q_out) e = cudaMemcpyAsync(in.Q_out, a.Q, sizeof(double) * nf, cudaMemcpyDeviceToHost, st);
