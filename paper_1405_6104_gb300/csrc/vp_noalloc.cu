@@ -118,7 +118,7 @@ struct TileShared {
   float s_x[2 * CV_T][3];
   float s_nf[2 * CV_T][3];
   double s_n[2 * CV_T][3];
-  int s_ghi[2 * CV_T][3];   // as in CvWarpShared: c >> 24 and the low 24 bits of each contribution
+  int s_ghi[2 * CV_T][3];   // c >> 24 and the low 24 bits of each contribution c
   unsigned s_glo[2 * CV_T][3];
   unsigned s_bal[CV_T];
   double s_z[NW];
@@ -244,13 +244,25 @@ __global__ void __launch_bounds__(NW * 32) k_eval(const float *__restrict__ pos,
       const ff h = ff_add(Ct, ff_neg(cnat));
       zacc = ff_add(zacc, ff_mul(Ct, ff_add(Ct, ff_neg(ff_mul_f(cnat, 2.0f)))));
       const float wgt = 2.0f * h.hi * dCt / rf;
-      const long long gv[3] = {fx_from(wgt * dx.hi), fx_from(wgt * dy.hi), fx_from(wgt * dz.hi)};
+      const float g[3] = {wgt * dx.hi, wgt * dy.hi, wgt * dz.hi};
+      // 32 contributions below 2^16 stay within the 32-bit halves; a larger one
+      // goes straight to the sums (contacts of a radius or switching range below
+      // some 1e-5 nm).  Coincident atoms (wgt not a number) pull nowhere.
+      const bool large = !(fmaxf(fmaxf(fabsf(g[0]), fabsf(g[1])), fabsf(g[2])) < 65536.0f);
+      if (wgt != wgt) continue;
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        atomicAdd(&sh.s_ghi[il][c], (int)((-gv[c]) >> 24));
-        atomicAdd(&sh.s_glo[il][c], (unsigned)((-gv[c]) & 0xffffff));
-        atomicAdd(&sh.s_ghi[CV_T + jc][c], (int)(gv[c] >> 24));
-        atomicAdd(&sh.s_glo[CV_T + jc][c], (unsigned)(gv[c] & 0xffffff));
+        const long long v = fx_from(g[c]);
+        if (large) {
+          long long *sum = c == 0 ? sc.gx : c == 1 ? sc.gy : sc.gz;
+          red_add(sum + bi * CV_T + il, (long long)(0ull - (unsigned long long)v));
+          red_add(sum + bj * CV_T + jc, v);
+          continue;
+        }
+        atomicAdd(&sh.s_ghi[il][c], (int)((-v) >> 24));
+        atomicAdd(&sh.s_glo[il][c], (unsigned)((-v) & 0xffffff));
+        atomicAdd(&sh.s_ghi[CV_T + jc][c], (int)(v >> 24));
+        atomicAdd(&sh.s_glo[CV_T + jc][c], (unsigned)(v & 0xffffff));
       }
     }
     zl = ff_to_d(zacc) + z0;
