@@ -54,3 +54,34 @@ def test_steep_contacts(r0):
     nat = 3.0 * rng.random((40, 3))
     _, g = _check(pos, nat, 8.0, S.Params(cv_r0=r0, cv_min_sep=2))
     assert np.abs(g).max() > 0.5 / r0
+
+
+@pytest.mark.parametrize("min_sep", [3, 30, 31, 32, 35, 63, 64])
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 36, 37, 64, 65, 97, 540])
+def test_tile_edges(n, min_sep):
+    """Tile diagonals without a pair left out, partial last tiles, no tile at
+    all; 60 atoms per nm^3 (many pairs near)."""
+    rng = np.random.default_rng(n)
+    pos = (2.0 + (max(n, 30) / 60.0) ** (1.0 / 3.0) * rng.random((n, 3))).astype(np.float32).astype(np.float64)
+    z, _ = _check(pos, pos + 0.1 * rng.normal(size=pos.shape), 8.0, S.Params(cv_min_sep=min_sep))
+    assert (z > 0.0) == (n > min_sep + 1)
+
+
+def test_no_atom():
+    z, g = _eval(np.zeros((0, 3)), np.zeros((0, 3)), 8.0, S.Params())
+    assert z == 0.0 and g.shape == (0, 3)
+
+
+@pytest.mark.parametrize("shift", [0.0, 1000.0])
+def test_native_pairs_around_the_cut_off(shift):
+    """Native distances within 3e-3 nm of the cut-off (the FP32 test of the
+    native structure passes pairs up to 4e-3 nm beyond), the structure far
+    from the origin; a narrow switch, so that C~ is visible next to it."""
+    rng = np.random.default_rng(11)
+    p = S.Params(cv_min_sep=2, cv_r_switch=1.19)
+    nat = np.zeros((70, 3))
+    nat[:35] = 0.05 * rng.normal(size=(35, 3))
+    u = rng.normal(size=(35, 3))
+    nat[35:] = nat[:35] + (p.cv_r_cut + 3e-3 * rng.uniform(-1, 1, (35, 1))) * u / np.linalg.norm(u, axis=1)[:, None]
+    pos = (3.0 + 0.4 * rng.normal(size=(70, 3))).astype(np.float32).astype(np.float64)
+    _check(pos, nat + shift, 8.0, p)
