@@ -298,6 +298,7 @@ int sim_diagnostics(sim_handle *h, int64_t *out);
  * class's clusters alone, and one launch per class with its own variant is
  * used instead of the single launch when that sequence is faster.
  * cache_path (may be NULL): a text file of "size-class variant variant" lines
+ * (the size class names the version of the variants' numbering as well)
  * consulted first and appended to (batches of one class).  choice[2] (may be
  * NULL) receives the picked variants (the single launch's pair variant). */
 int sim_autotune(sim_handle *h, int32_t reps, const char *cache_path, int32_t *choice);

@@ -1454,6 +1454,11 @@ VP_API int phi_adjoint_coefficients(sim_handle *h, const double *z, const double
 // ---------------------------------------------------------------------------
 namespace {
 
+// Raised whenever a variant number comes to mean another kernel: entries of
+// cache files written before are then tuned anew.  1 (no prefix): pair variants
+// 3-5 scalar, 6-8 packed with one group of entries at a time.
+constexpr int TUNE_VERSION = 2;
+
 std::string tune_key(const sim_handle *h) {
   long long atoms = 0;
   double vol = 0.0;
@@ -1465,7 +1470,7 @@ std::string tune_key(const sim_handle *h) {
   const int lg_trials = (int)std::lround(std::log2((double)std::max(1, h->n_trials)));
   const int dens = (int)std::lround(atoms / std::max(vol, 1e-9) / 10.0);
   char buf[96];
-  std::snprintf(buf, sizeof(buf), "a%d_t%d_d%d_nt%d", lg_atoms, lg_trials, dens, h->c.n_types);
+  std::snprintf(buf, sizeof(buf), "v%d_a%d_t%d_d%d_nt%d", TUNE_VERSION, lg_atoms, lg_trials, dens, h->c.n_types);
   return buf;
 }
 
