@@ -3,9 +3,9 @@
 // list is due.
 //
 // Every kernel here runs in every step and works only on the trials whose
-// list is due in that step: the front kernel (one block per trial) decides,
-// bins, scans and fills per trial and lists the rebuilding trials in
-// d.rb_list; the later kernels take their work items (columns, slot chunks,
+// list is due in that step: the front kernel (one cluster of eight blocks per
+// trial) decides, bins, scans and fills per trial and lists the rebuilding
+// trials in d.rb_list; the later kernels take their work items (columns,
 // clusters) from that list.  A trial's list is due when one of its atoms has moved
 // farther than skin/2 - 1e-5 nm from where its list was built (the update
 // kernel requests it), after nstlist steps, or on request from the host
@@ -129,14 +129,10 @@ __global__ void __launch_bounds__(LIST_WARPS * 32, LIST_PARTS_BLOCKS) k_list_par
   __shared__ ListShared sh;
   if (d.early_launch) PDL_TRIGGER();
   PDL_WAIT();
-  constexpr int PER_BLOCK = LIST_WARPS / PARTS;
-  const int n_items = (int)d.rb_cnt[0] * d.max_trial_clus;
-  int turn = 0;
-  for (int item = (int)blockIdx.x * PER_BLOCK + (int)(threadIdx.x >> 5) / PARTS; item < n_items;
-       item += (int)gridDim.x * PER_BLOCK, ++turn) {
-    __syncwarp();  // the warp's shared arrays of its previous cluster are no longer read
-    list_cluster<PARTS>(d, c, rl2_bbox, sh, d.rb_list[item / d.max_trial_clus], item % d.max_trial_clus, turn);
-  }
+  // one list per group of warps: the grid covers every cluster of every trial
+  const int item = (int)blockIdx.x * (LIST_WARPS / PARTS) + (int)(threadIdx.x >> 5) / PARTS;
+  if (item < (int)d.rb_cnt[0] * d.max_trial_clus)
+    list_cluster<PARTS>(d, c, rl2_bbox, sh, d.rb_list[item / d.max_trial_clus], item % d.max_trial_clus);
 }
 
 // positions the current list of one trial was built from, caller order
@@ -183,11 +179,9 @@ bool few_clusters(const Dev &d) { return 2ll * d.max_trial_clus * d.n_trials <= 
 void launch_list(const Dev &d, const SimConst &c, float rl2_bbox, cudaStream_t s) {
   const long long warps = list_parts_warps(d), clusters = (long long)d.max_trial_clus * d.n_trials;
   if (4 * clusters <= warps)
-    launch_pdl(k_list_parts<4>, dim3(rebuild_grid(d, LIST_PARTS_BLOCKS, d.max_trial_clus)), dim3(LIST_WARPS * 32), s, d, c,
-               rl2_bbox);
+    launch_pdl(k_list_parts<4>, dim3((unsigned)clusters), dim3(LIST_WARPS * 32), s, d, c, rl2_bbox);
   else if (few_clusters(d))
-    launch_pdl(k_list_parts<2>, dim3(rebuild_grid(d, LIST_PARTS_BLOCKS, (d.max_trial_clus + 1) / 2)), dim3(LIST_WARPS * 32),
-               s, d, c, rl2_bbox);
+    launch_pdl(k_list_parts<2>, dim3((unsigned)((clusters + 1) / 2)), dim3(LIST_WARPS * 32), s, d, c, rl2_bbox);
   else
     launch_pdl(k_list, dim3(rebuild_grid(d, 6, (d.max_trial_clus + LIST_WARPS - 1) / LIST_WARPS)), dim3(LIST_WARPS * 32),
                s, d, c, rl2_bbox);

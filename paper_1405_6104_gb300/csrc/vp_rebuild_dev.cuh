@@ -493,16 +493,16 @@ struct ListShared {
   unsigned s_dirty[LIST_WARPS][ENT_MAX / 32];  // entries whose j-atoms need the pair masks
   unsigned s_mask[LIST_WARPS][ENT_MAX];        // halves to test (phase 1), then the entries' masks (their
                                                // first words overwrite s_cand)
-  int4 s_part[2][LIST_WARPS];  // of the parts of a list: halves found, entries, masked and clean j-atoms
+  int4 s_part[LIST_WARPS];  // of the parts of a list: halves found, entries, masked and clean j-atoms
 };
 
 // PARTS > 1: that many consecutive warps of the block share the list, each
-// doing an equal share of the window's columns (turn counts their lists).  The
-// shares are consecutive in the list's order, so a warp only needs to know how
-// many j-atoms the shares before its own hold.
+// doing an equal share of the window's columns.  The shares are consecutive in the
+// list's order, so a warp only needs to know how many j-atoms the shares before
+// its own hold.  Once per block: s_part holds one list's numbers.
 template <int PARTS = 1>
 __device__ __forceinline__ void list_cluster(const Dev &d, const SimConst &c, float rl2_bbox, ListShared &sh, int t,
-                                             int Il, int turn = 0) {
+                                             int Il) {
   const int wib = threadIdx.x >> 5, part = wib % PARTS;
   const int lane = threadIdx.x & 31;
   auto &s_xp = sh.s_xp[wib];
@@ -790,7 +790,7 @@ __device__ __forceinline__ void list_cluster(const Dev &d, const SimConst &c, fl
     for (int e = lane; e < n_ent; e += 32) n_clean += j_columns(s_mask[e]);
     n_clean = (int)__reduce_add_sync(0xffffffffu, (unsigned)n_clean) - n_dirty;
     const int w0 = wib - part;
-    if (lane == 0) sh.s_part[turn & 1][wib] = make_int4(n_found, cnt, n_dirty, n_clean);
+    if (lane == 0) sh.s_part[wib] = make_int4(n_found, cnt, n_dirty, n_clean);
     // (constant barrier numbers: a block that may use all 16 leaves room for two on an SM)
     if (PARTS == LIST_WARPS) __syncthreads();
     else if (w0 == 0) asm volatile("bar.sync 1, %0;" ::"n"(32 * PARTS) : "memory");
@@ -798,7 +798,7 @@ __device__ __forceinline__ void list_cluster(const Dev &d, const SimConst &c, fl
     int before = 0;
     n_found = cnt = n_dirty = 0;
     for (int q = 0; q < PARTS; ++q) {
-      const int4 v = sh.s_part[turn & 1][w0 + q];
+      const int4 v = sh.s_part[w0 + q];
       n_found += v.x;
       cnt += v.y;
       n_dirty += v.z;
