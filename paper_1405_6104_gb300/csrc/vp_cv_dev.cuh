@@ -341,8 +341,7 @@ __device__ __forceinline__ void cv_tile_block(const CvTile &t, const CvConst &k,
   }
 }
 
-// the tile of work item wq of the batch's flat (trial, tile) list, in the
-// work order (costliest tiles first; the partial sums of z keep their slots)
+// the tile of work item W (the partial sum of z goes to the item's slot)
 __device__ __forceinline__ CvTile cv_item_tile(const Dev &d, const SimConst &c, const CvItem &W) {
   return CvTile{W.n_cv, W.bi, W.bj, c.cv_min_sep, W.box, W.inv_box, c.cv_rc2_far,
                 d.cnat_ff + (size_t)W.tile * CV_T * CV_T, d.gx + W.cv0, d.gy + W.cv0, d.gz + W.cv0, d.z_part + W.w};

@@ -62,16 +62,14 @@ __device__ __forceinline__ void bonded_energy(const Dev &d, const TrialInfo &T, 
   }
 }
 
-// the 8 pairs of one lane: j-atom (xj, yj, zj, qj, type row tj) against the
-// warp's 8 i-atoms.  Explicit round-to-nearest intrinsics pin the operation
-// count (3 FADD, 6 FMUL, 12 FFMA, 1 RSQ, 1 LDS, 1 FSEL per pair).
-template <bool EXACT, bool ENERGY>
-__device__ __forceinline__ void pair_block(const float (&xi)[CL], const float (&yi)[CL], const float (&zi)[CL],
-                                           const float (&qi)[CL], const int (&tio)[CL], float xj, float yj,
-                                           float zj, float qj, int tj, unsigned mb, float L, float iL,
-                                           const SimConst &c, const float2 *tab, const float *tshift,
-                                           float (&fi)[CL][3], float &fjx, float &fjy, float &fjz, float &elj,
-                                           float &erf) {
+// the energies of the 8 pairs of one lane: j-atom (xj, yj, zj, qj, type row tj)
+// against the warp's 8 i-atoms, distances rounded as the force kernels round them
+template <bool EXACT>
+__device__ __forceinline__ void pair_energies(const float (&xi)[CL], const float (&yi)[CL], const float (&zi)[CL],
+                                              const float (&qi)[CL], const int (&tio)[CL], float xj, float yj,
+                                              float zj, float qj, int tj, unsigned mb, float L, float iL,
+                                              const SimConst &c, const float2 *tab, const float *tshift, float &elj,
+                                              float &erf) {
 #pragma unroll
   for (int a = 0; a < CL; ++a) {
     float dx = __fsub_rn(xj, xi[a]), dy = __fsub_rn(yj, yi[a]), dz = __fsub_rn(zj, zi[a]);
@@ -87,35 +85,23 @@ __device__ __forceinline__ void pair_block(const float (&xi)[CL], const float (&
     const float rinv6 = __fmul_rn(__fmul_rn(rinv2, rinv2), rinv2);
     const float2 cc = tab[tio[a] + tj];
     const float qq = __fmul_rn(qi[a], qj);
-    float t = __fmaf_rn(cc.y, rinv6, -cc.x);
-    t = __fmul_rn(t, rinv6);
-    t = __fmaf_rn(qq, rinv, t);
-    t = __fmul_rn(t, rinv2);
-    float f = __fmaf_rn(-qq, c.two_krf, t);
-    f = in ? f : 0.0f;
-    fi[a][0] = __fmaf_rn(-f, dx, fi[a][0]);
-    fi[a][1] = __fmaf_rn(-f, dy, fi[a][1]);
-    fi[a][2] = __fmaf_rn(-f, dz, fi[a][2]);
-    fjx = __fmaf_rn(f, dx, fjx);
-    fjy = __fmaf_rn(f, dy, fjy);
-    fjz = __fmaf_rn(f, dz, fjz);
-    if (ENERGY && in) {
+    if (in) {
       elj += rinv6 * (cc.y * (1.0f / 12.0f) * rinv6 - cc.x * (1.0f / 6.0f)) - tshift[tio[a] + tj];
       erf += qq * (rinv + c.krf * r2 - c.crf);
     }
   }
 }
 
-template <bool ENERGY, int MINB>
-__global__ void __launch_bounds__(128, MINB) k_pair(Dev d, SimConst c, int only_trial) {
+// Energies (nonbonded and bonded) of one trial, or of all, any number of types:
+// one warp per i-cluster.
+__global__ void __launch_bounds__(128, 4) k_pair(Dev d, SimConst c, int only_trial) {
   extern __shared__ float2 smem_tab[];
-  __shared__ float s_red[ENERGY ? 1 : 4][ENERGY ? 1 : 3 * CL * 33];
   float2 *tab = smem_tab;
   float *tshift = reinterpret_cast<float *>(smem_tab + c.n_types * c.n_types);
   const int nt2 = c.n_types * c.n_types;
   for (int k = threadIdx.x; k < nt2; k += blockDim.x) {
     tab[k] = d.ljtab[k];
-    if (ENERGY) tshift[k] = d.ljshift[k];
+    tshift[k] = d.ljshift[k];
   }
   __syncthreads();
   const int I = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -135,9 +121,6 @@ __global__ void __launch_bounds__(128, MINB) k_pair(Dev d, SimConst c, int only_
     xi[a] = p.x; yi[a] = p.y; zi[a] = p.z; qi[a] = p.w;
     tio[a] = d.type[I * CL + a] * c.n_types;
   }
-  float fi[CL][3];
-#pragma unroll
-  for (int a = 0; a < CL; ++a) fi[a][0] = fi[a][1] = fi[a][2] = 0.0f;
   float elj = 0.0f, erf = 0.0f;
 
   const int n = d.list_n[I];
@@ -155,28 +138,15 @@ __global__ void __launch_bounds__(128, MINB) k_pair(Dev d, SimConst c, int only_
     const int sj_n = (int)(ent_n & J_MASK);
     const float4 pj_n = d.pos[sj_n];
     const int tj_n = d.type[sj_n];
-    const int sj = (int)(ent & J_MASK);
     const unsigned sh = ent >> J_BITS;
     const float xj = pj.x - L * (float)((int)(sh & 3u) - 1);
     const float yj = pj.y - L * (float)((int)((sh >> 2) & 3u) - 1);
     const float zj = pj.z - L * (float)((int)((sh >> 4) & 3u) - 1);
     const unsigned mb = e0 + lane < n ? segm[e0 + lane] : 0u;
-    const bool exact = (ent & E_EXACT) != 0u;
-    float fjx = 0.f, fjy = 0.f, fjz = 0.f;
-    if (!__any_sync(0xffffffffu, exact))
-      pair_block<false, ENERGY>(xi, yi, zi, qi, tio, xj, yj, zj, pj.w, tj, mb, L, iL, c, tab, tshift, fi, fjx, fjy,
-                                fjz, elj, erf);
-    else if (exact)
-      pair_block<true, ENERGY>(xi, yi, zi, qi, tio, xj, yj, zj, pj.w, tj, mb, L, iL, c, tab, tshift, fi, fjx, fjy,
-                               fjz, elj, erf);
+    if (ent & E_EXACT)
+      pair_energies<true>(xi, yi, zi, qi, tio, xj, yj, zj, pj.w, tj, mb, L, iL, c, tab, tshift, elj, erf);
     else
-      pair_block<false, ENERGY>(xi, yi, zi, qi, tio, xj, yj, zj, pj.w, tj, mb, L, iL, c, tab, tshift, fi, fjx, fjy,
-                                fjz, elj, erf);
-    if (!ENERGY && (fjx != 0.f || fjy != 0.f || fjz != 0.f)) {
-      red_add(d.fx + sj, fx_from(fjx));
-      red_add(d.fy + sj, fx_from(fjy));
-      red_add(d.fz + sj, fx_from(fjz));
-    }
+      pair_energies<false>(xi, yi, zi, qi, tio, xj, yj, zj, pj.w, tj, mb, L, iL, c, tab, tshift, elj, erf);
     ent = ent_n;
     ent_n = ent_nn;
     pj = pj_n;
@@ -196,31 +166,14 @@ __global__ void __launch_bounds__(128, MINB) k_pair(Dev d, SimConst c, int only_
     }
   }
 
-  if (!ENERGY) {
-    // i-forces: column sums of the 32 lanes' partials in a fixed order
-    float *r = s_red[threadIdx.x >> 5];
+  double e4[4] = {(double)elj, (double)erf, (double)eb, (double)ea};
 #pragma unroll
-    for (int a = 0; a < CL; ++a)
+  for (int k = 0; k < 4; ++k)
 #pragma unroll
-      for (int k = 0; k < 3; ++k) r[(3 * a + k) * 33 + lane] = fi[a][k];
-    __syncwarp();
-    if (lane < 3 * CL) {
-      float sum = 0.f;
-      for (int l = 0; l < 32; ++l) sum += r[lane * 33 + l];
-      const int a = lane / 3, comp = lane - 3 * a;
-      const long long val = fx_from(sum);
-      if (val != 0) red_add((comp == 0 ? d.fx : comp == 1 ? d.fy : d.fz) + I * CL + a, val);
-    }
-  } else {
-    double e4[4] = {(double)elj, (double)erf, (double)eb, (double)ea};
+    for (int off = 16; off > 0; off >>= 1) e4[k] += __shfl_xor_sync(0xffffffffu, e4[k], off);
+  if (lane == 0)
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) e4[k] += __shfl_xor_sync(0xffffffffu, e4[k], off);
-    if (lane == 0)
-#pragma unroll
-      for (int k = 0; k < 4; ++k) red_add(d.energy + (size_t)t * 5 + k, __double2ll_rn(e4[k] * E_SCALE));
-  }
+    for (int k = 0; k < 4; ++k) red_add(d.energy + (size_t)t * 5 + k, __double2ll_rn(e4[k] * E_SCALE));
 }
 
 
@@ -509,7 +462,7 @@ void launch_pair(const Dev &d, const SimConst &c, bool energy, int32_t only_tria
   unsigned blocks = (unsigned)((threads + 127) / 128);
   const size_t nt2 = (size_t)c.n_types * c.n_types;
   if (energy || only_trial >= 0) {
-    k_pair<true, 4><<<blocks, 128, nt2 * (sizeof(float2) + sizeof(float)), s>>>(d, c, only_trial);
+    k_pair<<<blocks, 128, nt2 * (sizeof(float2) + sizeof(float)), s>>>(d, c, only_trial);
     return;
   }
   if (!clist) n_items = d.total_clus;

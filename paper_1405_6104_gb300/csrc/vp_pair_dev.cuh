@@ -396,11 +396,9 @@ __device__ __forceinline__ void pair_cluster_f2(const Dev &d, const SimConst &c,
 // a water's angle and bonds form one group): every term's forces are
 // converted to fixed point and summed per atom, exactly, so the group issues
 // one reduction per atom and component (exact action-reaction: a bond's
-// second atom and an angle's vertex take minus the others' forces).  The
-// arithmetic of a term is that of bonded_force for the bond's first atom and
-// for the angle's vertex.  A kernel of its own, beside the pair kernel: inside
-// the pair kernel's warps the per-atom term loops ran on 8 of 32 lanes behind
-// chains of dependent loads.
+// second atom and an angle's vertex take minus the others' forces).  A kernel of
+// its own, beside the pair kernel: inside the pair kernel's warps the per-atom
+// term loops ran on 8 of 32 lanes behind chains of dependent loads.
 __device__ __forceinline__ void add3(long long (&F)[3][3], int m, long long x, long long y, long long z) {
 #pragma unroll
   for (int q = 0; q < 3; ++q)
