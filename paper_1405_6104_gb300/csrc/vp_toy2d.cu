@@ -579,11 +579,16 @@ extern "C" __attribute__((visibility("default"))) int toy2d_run(const toy2d_para
   // (an eighth of all draws at a time, between 1 and 64 MB, but 16 steps at least)
   const double total = (double)n * (double)n_steps;
   const long long want = (long long)std::min<double>(TOY_DRAWS, std::max<double>(1 << 16, total / 8.0));
-  const long long draws =
+  long long draws =
       (long long)n * std::max<long long>(1, std::min<long long>(n_steps, std::max<long long>(16, want / (long long)n)));
   double *buf = nullptr, *dpath = nullptr, *tables = nullptr;
-  bool ok = ck(cudaMalloc(&buf, (2 * (size_t)draws + n * 12 + 1) * sizeof(double)), "cudaMalloc") &&
-            (!path || ck(cudaMalloc(&dpath, (size_t)n_rec * 2 * n * sizeof(double)), "cudaMalloc"));
+  bool ok = !path || ck(cudaMalloc(&dpath, (size_t)n_rec * 2 * n * sizeof(double)), "cudaMalloc");
+  // with little memory left the draws of fewer steps at a time, down to one
+  for (; ok && cudaMalloc(&buf, (2 * (size_t)draws + n * 12 + 1) * sizeof(double)) != cudaSuccess;) {
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaErrorMemoryAllocation || draws == (long long)n) ok = ck(e, "cudaMalloc");
+    draws = std::max<long long>(n, draws / 4);
+  }
   double2 *dnoise = (double2 *)buf;
   double *dk = buf + 2 * draws;
   unsigned long long *dseed = (unsigned long long *)(dk + n);

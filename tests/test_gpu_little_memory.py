@@ -1,0 +1,63 @@
+"""Calls whose scratch has a size of choice, with almost all device memory
+taken by another allocator: less scratch, the same results.  (In a process of
+its own: the memory that is taken is given back with it.)"""
+import os
+import subprocess
+import sys
+
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+CHILD = r"""
+import sys
+import numpy as np, torch
+from paper_1405_6104_gb300 import binding as B, systems as S
+
+rng = np.random.default_rng(1)
+tp = S.Toy2dParams()
+ks, seeds = rng.choice([0.5, 4.0], 20000), rng.integers(1, 2 ** 60, 20000).astype(np.uint64)
+times = rng.integers(0, 40, (64, 40000)) * 10
+pairs = [(a, b) for a in range(64) for b in range(a)]
+s, p = S.small_solvated(n_solute=300, n_water=900)
+frames = s.native_pos * rng.uniform(0.4, 2.0, (750, 1, 1))
+
+
+def calls(h):
+    return [lambda: B.toy2d_run(tp, ks, seeds, 2000)[:3], lambda: B.path_similarity(times, pairs),
+            lambda: B.phi_frames_adjoint(h, 0, frames),
+            lambda: B.phi_frames_refine(h, 0, frames[:540], 2, 1e-4)]  # each takes more than 24 MB, given it
+
+
+def flat(x):
+    return [np.asarray(v) for v in (x if isinstance(x, (tuple, list)) else [x])]
+
+
+which = int(sys.argv[1])
+with B.TrialBatch(s, p, [1]) as b:
+    ref = flat(calls(b.h)[which]())
+b = B.TrialBatch(s, p, [1])  # its workspace is not taken yet
+torch.cuda.synchronize()
+room, hold = torch.empty(24 << 20, dtype=torch.uint8, device="cuda"), []
+for size in (1 << 33, 1 << 30, 1 << 27, 1 << 24, 1 << 21):  # the rest of the memory
+    try:
+        while True:
+            hold.append(torch.empty(size, dtype=torch.uint8, device="cuda"))
+    except torch.cuda.OutOfMemoryError:
+        pass
+del room
+torch.cuda.empty_cache()
+got = flat(calls(b.h)[which]())
+assert len(got) == len(ref) and all(np.array_equal(x, y, equal_nan=True) for x, y in zip(got, ref))
+print("same")
+"""
+
+
+@pytest.mark.parametrize("call", range(1), ids=["toy2d_run"])
+def test_results_with_little_memory_left(call):
+    from paper_1405_6104_gb300 import build
+    build.build()
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", CHILD, str(call)], cwd=root, capture_output=True, text=True, timeout=300,
+                       env={**os.environ, "PYTHONPATH": root})
+    assert r.returncode == 0 and "same" in r.stdout, r.stdout + r.stderr
