@@ -405,21 +405,38 @@ extern "C" __attribute__((visibility("default"))) int path_similarity(const int6
     return e == cudaSuccess;
   };
   // one allocation: the 16-bit ranks, and for a group of paths at a time their
-  // times, sets and sorted distinct times
-  const int32_t group = (int32_t)std::max<int64_t>(1, std::min<int64_t>({(int64_t)n_paths, 256, ((int64_t)1 << 27) / n_c}));
+  // times, sets and sorted distinct times (smaller groups with little memory left)
+  int32_t group = (int32_t)std::max<int64_t>(1, std::min<int64_t>({(int64_t)n_paths, 256, ((int64_t)1 << 27) / n_c}));
   const long long ld16 = ((long long)n_c + 7) & ~7ll;  // row length of the 16-bit ranks: rows start on 16 bytes
-  size_t total = 0;
-  auto part = [&](size_t bytes) {
-    const size_t off = total;
-    total += (bytes + 255) & ~(size_t)255;
-    return off;
-  };
-  const size_t o_times = part((size_t)group * (size_t)n_c * 8), o_set = part((size_t)group * SET_SLOTS * 8),
-               o_cnt = part((size_t)group * 4), o_sorted = part((size_t)group * DISTINCT_CAP * 8),
-               o_k = part((size_t)n_paths * 4), o_r16 = part((size_t)n_paths * (size_t)ld16 * 2), o_pp = part(np * 8),
-               o_list = part(2 * np * 4), o_all = part(np * 8), o_count = part(np * 8), o_call = part(np * 8);
+  size_t o_times, o_set, o_cnt, o_sorted, o_k, o_r16, o_pp, o_list, o_all, o_count, o_call;
   char *buf = nullptr;
-  bool ok = ck(cudaMalloc(&buf, total), "cudaMalloc");
+  bool ok = true;
+  for (;;) {
+    size_t total = 0;
+    auto part = [&](size_t bytes) {
+      const size_t off = total;
+      total += (bytes + 255) & ~(size_t)255;
+      return off;
+    };
+    o_times = part((size_t)group * (size_t)n_c * 8);
+    o_set = part((size_t)group * SET_SLOTS * 8);
+    o_cnt = part((size_t)group * 4);
+    o_sorted = part((size_t)group * DISTINCT_CAP * 8);
+    o_k = part((size_t)n_paths * 4);
+    o_r16 = part((size_t)n_paths * (size_t)ld16 * 2);
+    o_pp = part(np * 8);
+    o_list = part(2 * np * 4);
+    o_all = part(np * 8);
+    o_count = part(np * 8);
+    o_call = part(np * 8);
+    if (cudaMalloc(&buf, total) == cudaSuccess) break;
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaErrorMemoryAllocation || group == 1) {
+      ok = ck(e, "cudaMalloc");
+      break;
+    }
+    group /= 2;
+  }
   long long *d_times = (long long *)(buf + o_times), *d_sorted = (long long *)(buf + o_sorted);
   unsigned long long *d_sets = (unsigned long long *)(buf + o_set);
   int *d_cnt = (int *)(buf + o_cnt), *d_k = (int *)(buf + o_k), *d_list = (int *)(buf + o_list);

@@ -53,7 +53,7 @@ print("same")
 """
 
 
-@pytest.mark.parametrize("call", range(1), ids=["toy2d_run"])
+@pytest.mark.parametrize("call", range(2), ids=["toy2d_run", "path_similarity"])
 def test_results_with_little_memory_left(call):
     from paper_1405_6104_gb300 import build
     build.build()
