@@ -394,8 +394,9 @@ struct Carve {
 // per tile: 66 MB); the block form stays far below.
 constexpr size_t KEEP_NEAR = 500000;
 
-// the arrays every evaluation needs (with base = nullptr only their size counts)
-AdjDev adj_arrays(const AdjInput &in, Carve &c) {
+// the arrays every evaluation needs (with base = nullptr only their size
+// counts); keep: the near pairs' ballots too
+AdjDev adj_arrays(const AdjInput &in, Carve &c, bool keep) {
   const size_t na = (size_t)in.n_frames * in.n_cv;
   AdjDev a{};
   a.nf = in.n_frames; a.n_cv = in.n_cv; a.min_sep = in.min_sep; a.n_tiles = in.n_tiles;
@@ -412,7 +413,7 @@ AdjDev adj_arrays(const AdjInput &in, Carve &c) {
   a.coef = c.take<double>(2 * (size_t)in.n_frames);
   a.phi = c.take<double>(1);
   const size_t tiles = (size_t)in.n_frames * in.n_tiles;
-  if (tiles <= KEEP_NEAR) {
+  if (keep && tiles <= KEEP_NEAR) {
     a.n_near = c.take<int>(tiles);
     a.near = c.take<unsigned>(tiles * CV_T);
   }
@@ -423,9 +424,29 @@ AdjDev adj_arrays(const AdjInput &in, Carve &c) {
 // block form pays longer than beside the pair kernel (see launch_cv).  5576
 // tiles: z and grad z 62 -> 50 us, H_z w 56 -> 37; 84 303 tiles: 277 -> 332 and
 // 230 -> 261.
-bool block_form(const AdjInput &in) {
-  const long long tiles = (long long)in.n_frames * in.n_tiles;
-  return tiles <= 128ll * in.n_sm && tiles <= (long long)KEEP_NEAR;
+bool block_form(const AdjInput &in, const AdjDev &a) {
+  return a.near && (long long)in.n_frames * in.n_tiles <= 128ll * in.n_sm;
+}
+
+// The arrays of a call and (extra[k] doubles each) others of its own out of the
+// workspace, without the ballots when there is no memory for them (the near
+// pairs are then listed again).  False: no memory.
+template <int N>
+bool adj_reserve(const AdjInput &in, AdjWorkspace &ws, AdjDev &a, const size_t (&extra)[N], double *(&out)[N]) {
+  for (int keep = 1; keep >= 0; --keep) {
+    Carve size{nullptr};
+    adj_arrays(in, size, keep);
+    for (size_t n : extra) size.take<double>(n);
+    Carve c{(char *)ws.reserve(size.off)};
+    if (!c.base) {
+      cudaGetLastError();
+      continue;
+    }
+    a = adj_arrays(in, c, keep);
+    for (int k = 0; k < N; ++k) out[k] = c.take<double>(extra[k]);
+    return true;
+  }
+  return false;
 }
 
 // The kernels of a call are dependent launches (each starts with PDL_WAIT): a
@@ -436,7 +457,7 @@ void launch_adj_cv(const AdjInput &in, const AdjDev &a, cudaStream_t st) {
   const long long tiles = (long long)a.nf * a.n_tiles;
   const unsigned grid = (unsigned)((tiles + ADJ_WARPS - 1) / ADJ_WARPS);
   if (tiles > 0) {
-    if (block_form(in)) launch_pdl(k_adj_cv<CV_BLOCK_WARPS, true>, dim3((unsigned)tiles), dim3(32 * CV_BLOCK_WARPS), st, a, in.k);
+    if (block_form(in, a)) launch_pdl(k_adj_cv<CV_BLOCK_WARPS, true>, dim3((unsigned)tiles), dim3(32 * CV_BLOCK_WARPS), st, a, in.k);
     else launch_pdl(a.near ? k_adj_cv<1, true> : k_adj_cv<1, false>, dim3(grid), dim3(32 * ADJ_WARPS), st, a, in.k);
   }
   launch_pdl(k_adj_fin, dim3(a.nf), dim3(FIN_THREADS), st, a);
@@ -449,7 +470,7 @@ void launch_adj_grad(const AdjInput &in, const AdjDev &a, double *grad, cudaStre
   cudaMemsetAsync(a.hx, 0, sizeof(long long) * 3 * na, st);
   const unsigned grid = (unsigned)((tiles + ADJ_WARPS - 1) / ADJ_WARPS);
   if (tiles > 0) {
-    if (block_form(in)) launch_pdl(k_adj_hw<CV_BLOCK_WARPS, true>, dim3((unsigned)tiles), dim3(32 * CV_BLOCK_WARPS), st, a, in.k);
+    if (block_form(in, a)) launch_pdl(k_adj_hw<CV_BLOCK_WARPS, true>, dim3((unsigned)tiles), dim3(32 * CV_BLOCK_WARPS), st, a, in.k);
     else launch_pdl(a.near ? k_adj_hw<1, true> : k_adj_hw<1, false>, dim3(grid), dim3(32 * ADJ_WARPS), st, a, in.k);
   }
   launch_pdl(k_adj_out, dim3((unsigned)((na + 255) / 256)), dim3(256), st, a, grad);
@@ -460,14 +481,10 @@ void launch_adj_grad(const AdjInput &in, const AdjDev &a, double *grad, cudaStre
 int adjoint_frames(const AdjInput &in, AdjWorkspace &ws, cudaStream_t st, std::string &err) {
   const int nf = in.n_frames;
   const size_t nx = 3 * (size_t)nf * in.n_cv;
-  Carve size{nullptr};
-  adj_arrays(in, size);
-  size.take<double>(nx);
-  size.take<double>(nx);
-  Carve c{(char *)ws.reserve(size.off)};
-  if (!c.base) { err = "cudaMalloc failed"; return SIM_ECUDA; }
-  const AdjDev a = adj_arrays(in, c);
-  double *dx = c.take<double>(nx), *dgrad = c.take<double>(nx);
+  AdjDev a;
+  double *own[1];
+  if (!adj_reserve(in, ws, a, {nx}, own)) { err = "cudaMalloc failed"; return SIM_ECUDA; }
+  double *dx = own[0], *dgrad = dx;  // the frames are read once, at the start
   cudaError_t e = cudaMemcpyAsync(dx, in.frames, sizeof(double) * nx, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess && in.coef)
     e = cudaMemcpyAsync(a.coef, in.coef, sizeof(double) * 2 * nf, cudaMemcpyHostToDevice, st);
@@ -505,14 +522,10 @@ int refine_frames(const AdjInput &in, double *frames, int n_iter, double step, d
   const int nf = in.n_frames, ncv = in.n_cv;
   const size_t nx = 3 * (size_t)nf * ncv;
   constexpr int SQ_BLOCKS = 64;
-  Carve size{nullptr};
-  adj_arrays(in, size);
-  for (int k = 0; k < 3; ++k) size.take<double>(nx);
-  size.take<double>(SQ_BLOCKS);
-  Carve c{(char *)ws.reserve(size.off)};
-  if (!c.base) { err = "cudaMalloc failed"; return SIM_ECUDA; }
-  const AdjDev a = adj_arrays(in, c);
-  double *X = c.take<double>(nx), *Y = c.take<double>(nx), *G = c.take<double>(nx), *part = c.take<double>(SQ_BLOCKS);
+  AdjDev a;
+  double *own[4];
+  if (!adj_reserve(in, ws, a, {nx, nx, nx, (size_t)SQ_BLOCKS}, own)) { err = "cudaMalloc failed"; return SIM_ECUDA; }
+  double *X = own[0], *Y = own[1], *G = own[2], *part = own[3];
   const unsigned gx_blocks = (unsigned)((nx + 255) / 256);
   // Phi at the frames now in a.frames (their z and grad z stay for grad())
   auto eval = [&](double &phi) -> cudaError_t {

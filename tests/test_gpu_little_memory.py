@@ -53,7 +53,7 @@ print("same")
 """
 
 
-@pytest.mark.parametrize("call", range(2), ids=["toy2d_run", "path_similarity"])
+@pytest.mark.parametrize("call", range(4), ids=["toy2d_run", "path_similarity", "phi_frames_adjoint", "phi_frames_refine"])
 def test_results_with_little_memory_left(call):
     from paper_1405_6104_gb300 import build
     build.build()
