@@ -238,9 +238,9 @@ __device__ __forceinline__ void adj_hw_pairs(AdjHwShared &sh, const CvTile &t, c
   const float2 g[3] = {__ffma2_rn(q, f2_nma(ux, uv, vx), __fmul2_rn(__fmul2_rn(f2, ux), uv)),
                        __ffma2_rn(q, f2_nma(uy, uv, vy), __fmul2_rn(__fmul2_rn(f2, uy), uv)),
                        __ffma2_rn(q, f2_nma(uz, uv, vz), __fmul2_rn(__fmul2_rn(f2, uz), uv))};
-  // r is not a number where r^2 is below the normal range: atoms that coincide
-  // (K = 0, as C' and C'' vanish with r)
-  cv_accumulate(sh, t, g, il0, jc0, il1, jc1, cp.r.x == cp.r.x, v1 && cp.r.y == cp.r.y);
+  // r, and with it every component, is not a number where r^2 is below the normal
+  // range: atoms that coincide (K = 0, as C' and C'' vanish with r)
+  cv_accumulate<true>(sh, t, g, il0, jc0, il1, jc1, true, v1);
 }
 
 // H_z w per frame with a bias, a warp (NW = 1) or a block of NW warps per (frame, tile)

@@ -32,13 +32,20 @@ __device__ __forceinline__ void cv_add_large(const CvTile &t, float fx, float fy
 // large for the split; pair 1 only when v1.  |f| < 512: f 2^(32 - CV_SPLIT) +
 // 1.5 2^23 is rounded to the high part, what is left of f 2^32 is exact and
 // rounds to the low one -- no 64-bit conversion, which the FP64 pipe does.
-template <class SH>
+// SKIP_NAN: a pair whose three components are not numbers adds nothing.
+template <bool SKIP_NAN = false, class SH>
 __device__ __forceinline__ void cv_accumulate(SH &sh, const CvTile &t, const float2 (&f)[3], int il0, int jc0, int il1,
                                               int jc1, bool v0, bool v1) {
   const float big0 = fmaxf(fmaxf(fabsf(f[0].x), fabsf(f[1].x)), fabsf(f[2].x));
   const float big1 = fmaxf(fmaxf(fabsf(f[0].y), fabsf(f[1].y)), fabsf(f[2].y));
-  if (v0 && !(big0 < 512.0f)) { cv_add_large(t, f[0].x, f[1].x, f[2].x, il0, jc0); v0 = false; }
-  if (v1 && !(big1 < 512.0f)) { cv_add_large(t, f[0].y, f[1].y, f[2].y, il1, jc1); v1 = false; }
+  if (v0 && !(big0 < 512.0f)) {
+    if (!SKIP_NAN || big0 == big0) cv_add_large(t, f[0].x, f[1].x, f[2].x, il0, jc0);
+    v0 = false;
+  }
+  if (v1 && !(big1 < 512.0f)) {
+    if (!SKIP_NAN || big1 == big1) cv_add_large(t, f[0].y, f[1].y, f[2].y, il1, jc1);
+    v1 = false;
+  }
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
     const float2 m = f2_all(12582912.0f);
