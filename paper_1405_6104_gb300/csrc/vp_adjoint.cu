@@ -48,7 +48,7 @@ struct AdjFramePos {
 __device__ __forceinline__ CvTile adj_tile(const AdjDev &a, const CvConst &k, int f, int t) {
   const int2 bij = a.tiles[t];
   const size_t base = (size_t)f * a.n_cv;
-  return CvTile{a.n_cv, bij.x, bij.y, a.min_sep, a.L, a.iL, k.rc2_far, a.cnat + (size_t)t * CV_T * CV_T,
+  return CvTile{a.n_cv, bij.x, bij.y, a.min_sep, a.L, a.iL, k.rc2_far, 0.f, a.cnat + (size_t)t * CV_T * CV_T,
                 a.gx + base, a.gy + base, a.gz + base, a.zpart + (size_t)f * a.n_tiles + t};
 }
 

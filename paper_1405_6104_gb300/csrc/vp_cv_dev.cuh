@@ -11,6 +11,7 @@ namespace vp {
 struct CvTile {
   int n_cv, bi, bj, min_sep;
   float L, iL, rc2_far;
+  float near2;              // set by cv_tile_far
   const float2 *cn;         // the tile's C~_nat
   long long *gx, *gy, *gz;  // the configuration's gradient sums (atom 0)
   double *z_part;           // the tile's partial sum of z
@@ -93,7 +94,7 @@ __device__ __forceinline__ ff2 cv_near_pairs(SH &sh, const CvConst &k, const CvT
 
 // whether the pairs of atom xi with xj0 and with xj1 are closer than the contact
 // cut-off (FP32; a position that is not a number is near nothing)
-__device__ __forceinline__ void cv_are_near(float4 xi, float4 xj0, float4 xj1, float L, float iL, float rc2_far, bool &n0,
+__device__ __forceinline__ void cv_are_near(float4 xi, float4 xj0, float4 xj1, float L, float iL, float near2, bool &n0,
                                             bool &n1) {
   const float2 m = f2_all(12582912.0f), il = f2_all(iL), l = f2_all(-L);  // see cv_delta2
   float2 dx = __fadd2_rn(make_float2(xj0.x, xj1.x), f2_all(-xi.x)), dy = __fadd2_rn(make_float2(xj0.y, xj1.y), f2_all(-xi.y)),
@@ -102,8 +103,8 @@ __device__ __forceinline__ void cv_are_near(float4 xi, float4 xj0, float4 xj1, f
   dy = __ffma2_rn(l, f2_sub(__fadd2_rn(__fmul2_rn(dy, il), m), m), dy);
   dz = __ffma2_rn(l, f2_sub(__fadd2_rn(__fmul2_rn(dz, il), m), m), dz);
   const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dx, dx, __fmul2_rn(dy, dy)));
-  n0 = r2.x < rc2_far;
-  n1 = r2.y < rc2_far;
+  n0 = r2.x < near2;
+  n1 = r2.y < near2;
 }
 
 // the accumulated gradient of atom a (0..63) of the tile, into the sums at gx, gy, gz
@@ -120,9 +121,12 @@ __device__ __forceinline__ void cv_flush_atom(SH &sh, int a, long long *gx, long
 
 // Whether no pair of the tile can be closer than the contact cut-off: the
 // periodic gap of the two 32-atom blocks' bounding boxes (lane l holds atom l
-// of either block).  Some 50 instructions that spare a far tile the 800 of its
-// distance tests.
-__device__ __forceinline__ bool cv_tile_far(const CvTile &t, bool iv, bool jv, float3 xi, float3 xj) {
+// of either block).  Some 60 instructions that spare a far tile the 800 of its
+// distance tests.  Otherwise t.near2 is what those take as near.
+__device__ __forceinline__ bool cv_tile_far(CvTile &t, bool iv, bool jv, float3 xi, float3 xj) {
+  const float3 ai = iv ? xi : make_float3(0.f, 0.f, 0.f), aj = jv ? xj : make_float3(0.f, 0.f, 0.f);
+  const float m = warp_max(fmaxf(fmaxf(fmaxf(fabsf(ai.x), fabsf(ai.y)), fabsf(ai.z)),
+                                 fmaxf(fmaxf(fabsf(aj.x), fabsf(aj.y)), fabsf(aj.z))));
   float g2 = 0.f;
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
@@ -131,10 +135,11 @@ __device__ __forceinline__ bool cv_tile_far(const CvTile &t, bool iv, bool jv, f
     const float bl = warp_min(jv ? b : 3e38f), bh = warp_max(jv ? b : -3e38f);
     float dc = 0.5f * (bl + bh) - 0.5f * (al + ah);
     dc = fabsf(dc - t.L * rintf(dc * t.iL)) - 0.5f * ((ah - al) + (bh - bl));
-    dc = fmaxf(dc, 0.f);
+    dc = fmaxf(dc - 1e-6f * m, 0.f);  // every rounding above
     g2 += dc * dc;
   }
-  return g2 > 1.001f * t.rc2_far;  // the margin covers every rounding
+  t.near2 = cv_near2(t.rc2_far, 4.0f * m * m);
+  return g2 > 1.001f * t.rc2_far;
 }
 
 // The near pairs of the tile by one warp, in rotation-major order, into
@@ -150,7 +155,7 @@ __device__ __forceinline__ int cv_near_list(const CvTile &t, unsigned short *s_n
   for (int k = 0; k < CV_T; k += 2) {
     const int j0 = (lane + k) & (CV_T - 1), j1 = (lane + k + 1) & (CV_T - 1);
     bool n0, n1;
-    cv_are_near(xi, s_x[CV_T + j0], s_x[CV_T + j1], t.L, t.iL, t.rc2_far, n0, n1);
+    cv_are_near(xi, s_x[CV_T + j0], s_x[CV_T + j1], t.L, t.iL, t.near2, n0, n1);
     n0 = n0 && j0 > sep;
     n1 = n1 && j1 > sep;
     const unsigned b0 = __ballot_sync(0xffffffffu, n0), b1 = __ballot_sync(0xffffffffu, n1);
@@ -191,7 +196,7 @@ __device__ __forceinline__ void cv_ballots_block(const CvTile &t, unsigned *s_ba
   for (int q = 0; q < KW; q += 2) {
     const int k = warp * KW + q, j0 = (lane + k) & (CV_T - 1), j1 = (lane + k + 1) & (CV_T - 1);
     bool n0, n1;
-    cv_are_near(xi, s_x[CV_T + j0], s_x[CV_T + j1], t.L, t.iL, t.rc2_far, n0, n1);
+    cv_are_near(xi, s_x[CV_T + j0], s_x[CV_T + j1], t.L, t.iL, t.near2, n0, n1);
     const unsigned b0 = __ballot_sync(0xffffffffu, n0 && j0 > sep), b1 = __ballot_sync(0xffffffffu, n1 && j1 > sep);
     if (lane == 0) {
       s_bal[k] = b0;
@@ -232,7 +237,7 @@ __device__ __forceinline__ float4 cv_atom(bool valid, float3 x) {
 // KEEP: the number of near pairs and the ballots that list them are left at
 // n_kept and kept, for a later pass over the same pairs.
 template <bool KEEP = false, class POS>
-__device__ __forceinline__ void cv_tile(const CvTile &t, const CvConst &k, CvWarpShared &sh, POS pos,
+__device__ __forceinline__ void cv_tile(CvTile t, const CvConst &k, CvWarpShared &sh, POS pos,
                                         int *n_kept = nullptr, unsigned *kept = nullptr) {
   const int lane = threadIdx.x & 31;
   const int i = t.bi * CV_T + lane, j = t.bj * CV_T + lane;
@@ -292,7 +297,7 @@ struct CvBlockShared {
 // positions of the tile's 64 atoms into s_x, its gradient sums cleared;
 // returns (in every thread) whether the tile is far
 template <int NW, class SH, class POS>
-__device__ __forceinline__ bool cv_block_begin(const CvTile &t, SH &sh, POS pos) {
+__device__ __forceinline__ bool cv_block_begin(CvTile &t, SH &sh, POS pos) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (threadIdx.x < 2 * CV_T) {
     const int a = (warp == 0 ? t.bi : t.bj) * CV_T + lane;
@@ -311,7 +316,7 @@ __device__ __forceinline__ bool cv_block_begin(const CvTile &t, SH &sh, POS pos)
 }
 
 template <int NW, bool KEEP = false, class POS>
-__device__ __forceinline__ void cv_tile_block(const CvTile &t, const CvConst &k, CvBlockShared &sh, POS pos,
+__device__ __forceinline__ void cv_tile_block(CvTile t, const CvConst &k, CvBlockShared &sh, POS pos,
                                               int *n_kept = nullptr, unsigned *kept = nullptr) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (cv_block_begin<NW>(t, sh, pos)) {
@@ -350,7 +355,7 @@ __device__ __forceinline__ void cv_tile_block(const CvTile &t, const CvConst &k,
 
 // the tile of work item W (the partial sum of z goes to the item's slot)
 __device__ __forceinline__ CvTile cv_item_tile(const Dev &d, const SimConst &c, const CvItem &W) {
-  return CvTile{W.n_cv, W.bi, W.bj, c.cv_min_sep, W.box, W.inv_box, c.cv_rc2_far,
+  return CvTile{W.n_cv, W.bi, W.bj, c.cv_min_sep, W.box, W.inv_box, c.cv_rc2_far, 0.f,
                 d.cnat_ff + (size_t)W.tile * CV_T * CV_T, d.gx + W.cv0, d.gy + W.cv0, d.gz + W.cv0, d.z_part + W.w};
 }
 

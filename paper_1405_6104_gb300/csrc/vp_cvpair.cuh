@@ -197,6 +197,14 @@ __device__ __forceinline__ CvPair2 cv_contact2(ff2 r2, const CvConst &k) {
   return o;
 }
 
+// The squared distance below which the FP32 tests take a pair as near: they round
+// a coordinate difference d by 2^-24 d before its images are taken off, so with
+// atoms hundreds of boxes apart the margin in rc2_far (1e-4) does not do, and the
+// limit grows with the largest d^2.  (Pairs beyond the cut-off add zeros.)
+__device__ __forceinline__ float cv_near2(float rc2_far, float d2) {
+  return fmaxf(rc2_far, fminf(1.1e-10f * d2 + rc2_far, 1e6f));
+}
+
 // exact minimum-image differences x_j - x_i as float-float
 __device__ __forceinline__ void cv_delta2(float4 xi0, float4 xi1, float4 xj0, float4 xj1, float L, float iL, ff2 &dx,
                                           ff2 &dy, ff2 &dz) {

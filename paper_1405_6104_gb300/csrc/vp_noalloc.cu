@@ -24,6 +24,7 @@
 #include <string>
 
 #include "../../include/vpath.h"
+#include "vp_cvpair.cuh"
 #include "vp_internal.cuh"
 
 #define VP_API extern "C" __attribute__((visibility("default")))
@@ -169,10 +170,11 @@ __global__ void __launch_bounds__(NW * 32) k_eval(const float *__restrict__ pos,
       if (i < k.n_cv && j < k.n_cv && j - i > k.min_sep) {
         const float *a = sh.s_x[lane], *b = sh.s_x[CV_T + jc];
         float dx = b[0] - a[0], dy = b[1] - a[1], dz = b[2] - a[2];
+        const float near2 = cv_near2(k.rc2_far, fmaxf(fmaxf(dx * dx, dy * dy), dz * dz));
         dx -= k.L * rintf(dx * k.iL);
         dy -= k.L * rintf(dy * k.iL);
         dz -= k.L * rintf(dz * k.iL);
-        if (dx * dx + dy * dy + dz * dz < k.rc2_far) flags[u] |= POS_NEAR;
+        if (dx * dx + dy * dy + dz * dz < near2) flags[u] |= POS_NEAR;
         a = sh.s_nf[lane];
         b = sh.s_nf[CV_T + jc];
         dx = b[0] - a[0]; dy = b[1] - a[1]; dz = b[2] - a[2];
