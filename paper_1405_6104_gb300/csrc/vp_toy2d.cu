@@ -626,8 +626,10 @@ extern "C" __attribute__((visibility("default"))) int toy2d_run(const toy2d_para
     }
     // one warp per block: the trials spread evenly over the SMs.  Two lanes per
     // trial up to about five warps per SM (8000 trials on 152 SMs: 3.3): beyond,
-    // the SM's FP64 unit is full and fewer instructions in all win.
-    const bool pair = (long long)active <= 76ll * n_sm;
+    // the SM's FP64 unit is full and fewer instructions in all win.  Parameters out
+    // of the quotients' range take one lane, whose step goes to the operators at
+    // once (8000 trials of 2000 steps with a friction of 1e-85: 15.6 ms in pairs).
+    const bool pair = c.plain && (long long)active <= 76ll * n_sm;
     const unsigned blocks = (unsigned)((active + (pair ? 15 : 31)) / (pair ? 16 : 32));
     if (pair) {
       if (tables) k_toy2d_pair<true><<<blocks, 32, 0, st>>>(c, l, ts);
