@@ -499,10 +499,15 @@ extern "C" __attribute__((visibility("default"))) int path_similarity(const int6
   // all ordered pairs need 32-bit ranks; those of paths of more distinct times
   // than the device ranks come from up to 16 host threads (their number is not
   // needed: only that it exceeds DISTINCT_CAP)
-  int *d_r32 = nullptr;
+  // They take the place of the times, which are ranked, where they fit (up to 512
+  // paths; an allocation and its free take some 100 us).
+  int *d_r32 = nt * 4 <= (size_t)group * (size_t)n_c * 8 ? (int *)d_times : nullptr, *r32_own = nullptr;
   std::vector<int> rk;
   if (ok && na > 0) {
-    ok = ck(cudaMalloc(&d_r32, nt * 4), "cudaMalloc");
+    if (!d_r32) {
+      ok = ck(cudaMalloc(&r32_own, nt * 4), "cudaMalloc");
+      d_r32 = r32_own;
+    }
     for (int32_t p0 = 0; ok && p0 < n_paths; p0 += 65535) {
       const int32_t m = std::min(n_paths - p0, 65535);
       k_widen<<<dim3((unsigned)((n_c + 255) / 256), (unsigned)m), 256, 0, st>>>(
@@ -552,7 +557,7 @@ extern "C" __attribute__((visibility("default"))) int path_similarity(const int6
     for (int32_t q = 0; q < n_pairs; ++q) s[q] = (double)hc[(size_t)q] / denom;
   }
   cudaFree(buf);
-  cudaFree(d_r32);
+  cudaFree(r32_own);
   if (!err.empty()) return put_err(errbuf, errlen, SIM_ECUDA, "path_similarity: " + err);
   return SIM_OK;
 }
