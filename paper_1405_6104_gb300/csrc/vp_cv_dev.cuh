@@ -135,11 +135,14 @@ __device__ __forceinline__ bool cv_tile_far(CvTile &t, bool iv, bool jv, float3 
     const float bl = warp_min(jv ? b : 3e38f), bh = warp_max(jv ? b : -3e38f);
     float dc = 0.5f * (bl + bh) - 0.5f * (al + ah);
     dc = fabsf(dc - t.L * rintf(dc * t.iL)) - 0.5f * ((ah - al) + (bh - bl));
-    dc = fmaxf(dc - 1e-6f * m, 0.f);  // every rounding above
+    dc = fmaxf(dc, 0.f);
     g2 += dc * dc;
   }
-  t.near2 = cv_near2(t.rc2_far, 4.0f * m * m);
-  return g2 > 1.001f * t.rc2_far;
+  const float m2 = m * m;
+  t.near2 = cv_near2(t.rc2_far, 4.0f * m2);
+  // a gap is off by 1e-6 m at most: with e = sqrt(3) 1e-6 m, (r + e)^2 is below
+  // 1.0005 r^2 + 2001 e^2
+  return g2 > fmaf(6e-9f, m2, 1.001f * t.rc2_far);
 }
 
 // The near pairs of the tile by one warp, in rotation-major order, into

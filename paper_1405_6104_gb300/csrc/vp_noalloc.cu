@@ -99,6 +99,17 @@ __device__ __forceinline__ double native_contact(double d2, const Consts &k) {
   return C * (1.0 - x * x * x * (10.0 - 15.0 * x + 6.0 * x * x));
 }
 
+// a contribution too large for the tile's halves (out of line: the kernel is
+// short enough for its code to be fetched cold)
+static __device__ __noinline__ void add_large(Scratch sc, int i, int j, float gx, float gy, float gz) {
+  const long long v[3] = {fx_from(gx), fx_from(gy), fx_from(gz)};
+  long long *const sum[3] = {sc.gx, sc.gy, sc.gz};
+  for (int c = 0; c < 3; ++c) {
+    red_add(sum[c] + i, (long long)(0ull - (unsigned long long)v[c]));
+    red_add(sum[c] + j, v[c]);
+  }
+}
+
 // One kernel: a block of NW warps per 32 x 32 tile of the contact-pair
 // triangle lists the pairs that are near in the configuration or in the native
 // structure (FP32 distances, a rotation of the tile per warp and step) and
@@ -250,17 +261,13 @@ __global__ void __launch_bounds__(NW * 32) k_eval(const float *__restrict__ pos,
       // 32 contributions below 2^16 stay within the 32-bit halves; a larger one
       // goes straight to the sums (contacts of a radius or switching range below
       // some 1e-5 nm).  Coincident atoms (wgt not a number) pull nowhere.
-      const bool large = !(fmaxf(fmaxf(fabsf(g[0]), fabsf(g[1])), fabsf(g[2])) < 65536.0f);
-      if (wgt != wgt) continue;
+      if (!(fmaxf(fmaxf(fabsf(g[0]), fabsf(g[1])), fabsf(g[2])) < 65536.0f)) {
+        if (wgt == wgt) add_large(sc, bi * CV_T + il, bj * CV_T + jc, g[0], g[1], g[2]);
+        continue;
+      }
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         const long long v = fx_from(g[c]);
-        if (large) {
-          long long *sum = c == 0 ? sc.gx : c == 1 ? sc.gy : sc.gz;
-          red_add(sum + bi * CV_T + il, (long long)(0ull - (unsigned long long)v));
-          red_add(sum + bj * CV_T + jc, v);
-          continue;
-        }
         atomicAdd(&sh.s_ghi[il][c], (int)((-v) >> 24));
         atomicAdd(&sh.s_glo[il][c], (unsigned)((-v) & 0xffffff));
         atomicAdd(&sh.s_ghi[CV_T + jc][c], (int)(v >> 24));
